@@ -117,99 +117,277 @@ __global__ void k_transpose_flip(const __nv_bfloat16* __restrict__ w, __nv_bfloa
   wT[i] = w[((size_t)co * Ci + ci) * taps + (taps - 1 - t)];
 }
 
-// Weight gradient, deterministic: block (g, ci * co-tile) sums, in a fixed order, the
-// (batch, tile) units g, g + G, g + 2G, ... into one partial per (output channel, tap), written
-// to part[g][co][ci][t]; k_wgrad_reduce then adds the G partials of every weight in order g = 0..G-1.
-// No floating-point atomics, so the result is the same on every run.
-__global__ void __launch_bounds__(512) k_conv_wgrad(const float* __restrict__ x,
-                                                    const float* __restrict__ dy,
-                                                    float* __restrict__ part, int B, int Ci, int Co,
-                                                    int n, int ks, int G) {
-  __shared__ float xs[HV];
-  __shared__ float dys[CT][NTV];
-  const int tid = threadIdx.x;
-  const int ntx = (n + BX - 1) / BX, nty = (n + BY - 1) / BY, ntz = (n + BZ - 1) / BZ;
-  const int tiles = ntx * nty * ntz;
-  const int g = blockIdx.x;
-  const int ci = blockIdx.y % Ci, cot = blockIdx.y / Ci;
-  const int co0 = cot * CT;
+// Weight gradient, deterministic.  dw[co][ci][t] is a product of Co x B n^3 by B n^3 x 27 Ci in
+// FP32 (274 GFLOP in a training step at 64^3, batch 8), so the FP32 pipes bound it and everything
+// else has to stay off their issue slots.  A block owns 16 output channels x CIT input channels
+// and the voxel tiles (units) g, g + G, ...; it stages a unit's x (with halo, [voxel][ci], rows
+// of CIT + 1 words: conflict free both ways) and dy ([voxel][16 co], 16-byte quads swizzled by
+// voxel) in shared memory by 4-byte asynchronous copies into two buffers, the next unit's under
+// the products of this one.  A thread owns one input channel, one dz, 8 output channels and one
+// of the KS slices of the tile's rows: it walks its rows in x with a 3 x 3 window of x in
+// registers, so a voxel costs 3 + 2 shared loads for 72 FMAs.  One block of 12 warps per SM: the
+// 72 sums want 167 registers.  The step's 15 weight gradients take 7.6 ms (36 TFLOP/s); one
+// (co, tap) per thread with two shared loads per FMA took 57.3 ms, this kernel with three blocks
+// of 6 warps at 96 registers (spilled sums) 14.3 ms, with two and loads through registers
+// 10.3 ms.  Packed fma.rn.f32x2 gains nothing (7.7 ms).
+// Partial sums part[g][co][ci][t] (and partb[g][co], from the blocks of the first input
+// channels) are added over g in a fixed order by k_wgrad_reduce: no floating-point atomics, the
+// same bits on every run.
+constexpr int WG_NT = 384, WG_TV = 256;
+
+struct WgTile {
+  int tx, ty, tz;      // voxels of a unit (tx * ty * tz <= WG_TV)
+  int ntx, nty, ntz;   // units of a sample along each axis
+};
+
+// 4 bytes to shared memory, asynchronously; zeros when !in (the address is then not read)
+__device__ __forceinline__ void cp4(float* dst, const float* src, bool in) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "r"(in ? 4 : 0)
+               : "memory");
+}
+
+template <int CIT>
+__global__ void __launch_bounds__(WG_NT, 1) k_wgrad3(const float* __restrict__ x,
+                                                     const float* __restrict__ dy,
+                                                     float* __restrict__ part,
+                                                     float* __restrict__ partb, int B, int Ci,
+                                                     int Co, int n, WgTile tl, int G) {
+  constexpr int KS = WG_NT / (6 * CIT), XS = CIT + 1, NW = WG_NT / 32;
+  extern __shared__ __align__(16) float wg_smem[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ci = tid % CIT, cog = (tid / CIT) & 1, dz = (tid / (2 * CIT)) % 3, ks = tid / (6 * CIT);
+  const int nci = (Ci + CIT - 1) / CIT;
+  const int ci0 = (blockIdx.y % nci) * CIT, co0 = (blockIdx.y / nci) * 16;
+  const int HX = tl.tx + 2, HY = tl.ty + 2, HZ = tl.tz + 2, HXY = HX * HY;
+  const int rows = tl.ty * tl.tz, TV = rows * tl.tx;
+  const int tiles = tl.ntx * tl.nty * tl.ntz;
   const size_t nv = (size_t)n * n * n;
-  const int taps = ks * ks * ks;
-  const int c = tid / taps, t = tid % taps;
-  int ox = 0, oy = 0, oz = 0;
-  if (ks == 3) { ox = t % 3 - 1; oy = (t / 3) % 3 - 1; oz = t / 9 - 1; }
-  float s = 0.f;
-  for (int u = g; u < tiles * B; u += G) {
-    const int b = u / tiles, tile = u % tiles;
-    const int tx0 = (tile % ntx) * BX, ty0 = ((tile / ntx) % nty) * BY, tz0 = (tile / (ntx * nty)) * BZ;
-    for (int i = tid; i < HV; i += blockDim.x) {
-      const int hx = i % HXn, hy = (i / HXn) % HYn, hz = i / (HXn * HYn);
-      xs[i] = xval(x + ((size_t)b * Ci + ci) * nv, n, tx0 + hx - 1, ty0 + hy - 1, tz0 + hz - 1);
-    }
-    for (int i = tid; i < CT * NTV; i += blockDim.x) {
-      const int cc = i / NTV, vv = i % NTV;
-      const int lx = vv % BX, ly = (vv / BX) % BY, lz = vv / (BX * BY);
-      const int gx = tx0 + lx, gy = ty0 + ly, gz = tz0 + lz;
-      const int co = co0 + cc;
-      dys[cc][vv] = (co < Co && gx < n && gy < n && gz < n)
-                        ? dy[((size_t)b * Co + co) * nv + ((size_t)gz * n + gy) * n + gx]
-                        : 0.f;
-    }
-    __syncthreads();
-    if (tid < CT * taps) {
-      for (int vv = 0; vv < NTV; ++vv) {
-        const int lx = vv % BX, ly = (vv / BX) % BY, lz = vv / (BX * BY);
-        s = fmaf(dys[c][vv], xs[((lz + 1 + oz) * HYn + (ly + 1 + oy)) * HXn + (lx + 1 + ox)], s);
+  // two buffers of dy [WG_TV][16] (quads swizzled) and x [(tz+2)(ty+2)(tx+2)][XS]
+  const int bufw = (WG_TV * 16 + HXY * HZ * XS + 3) & ~3;
+  const bool bias = partb && ci0 == 0;
+  float bsum = 0.f;                           // channel tid % 16, voxels tid / 16, + NT / 16, ...
+  float s[8][9];
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+#pragma unroll
+    for (int t = 0; t < 9; ++t) s[c][t] = 0.f;
+  auto stage = [&](int u, float* dys) {
+    float* xs = dys + WG_TV * 16;
+    const int b = u / tiles, tile = u - b * tiles;
+    const int tx0 = (tile % tl.ntx) * tl.tx, ty0 = ((tile / tl.ntx) % tl.nty) * tl.ty,
+              tz0 = (tile / (tl.ntx * tl.nty)) * tl.tz;
+    // Warp w of the 12 takes the channels w % CG, + CG, ... and the positions of its third (or
+    // sixth) of the tile; a lane's position is decoded once for all channels and planes.  The
+    // addresses are clamped into the tensor, what lies outside the grid arrives as zero.
+    constexpr int CG = CIT < 4 ? CIT : 4, PG = NW / CG;
+    const float* xb = x + ((size_t)b * Ci + ci0) * nv;
+    const int cw = warp % CG, pw = (warp / CG) * 32 + lane;
+    const int cmax = Ci - 1 - ci0;
+    for (int e = pw; e < HXY; e += PG * 32) {
+      const int hy = e / HX, hx = e - hy * HX;
+      const int gx = tx0 + hx - 1, gy = ty0 + hy - 1;
+      const bool inxy = gx >= 0 && gx < n && gy >= 0 && gy < n;
+      const int oxy = inxy ? gy * n + gx : 0;
+      float* d = xs + e * XS + cw;
+      for (int hz = 0; hz < HZ; ++hz, d += HXY * XS) {
+        const int gz = tz0 + hz - 1;
+        const bool in = inxy && gz >= 0 && gz < n;
+        const float* p = xb + (size_t)(in ? gz : 0) * n * n + oxy;
+#pragma unroll
+        for (int k = 0; k < CIT / CG; ++k) {
+          const int c = cw + k * CG;
+          cp4(d + k * CG, p + (size_t)min(c, cmax) * nv, in && c <= cmax);
+        }
       }
     }
+    const float* dyb = dy + ((size_t)b * Co + co0) * nv;
+    const int gw = warp & 3, omax = Co - 1 - co0;
+    for (int v = (warp >> 2) * 32 + lane; v < TV; v += NW / 4 * 32) {
+      const int lx = v % tl.tx, r = v / tl.tx, ly = r % tl.ty, lz = r / tl.ty;
+      const int gx = tx0 + lx, gy = ty0 + ly, gz = tz0 + lz;
+      const bool in = gx < n && gy < n && gz < n;
+      const float* p = dyb + (in ? ((size_t)gz * n + gy) * n + gx : 0);
+      float* d = dys + v * 16 + gw;
+      const int sw = (v >> 1) & 3;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int c = gw + 4 * k;
+        cp4(d + ((k ^ sw) << 2), p + (size_t)min(c, omax) * nv, in && c <= omax);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int units = tiles * B;
+  int buf = 0;
+  if ((int)blockIdx.x < units) stage(blockIdx.x, wg_smem);
+  for (int u = blockIdx.x; u < units; u += G, buf ^= 1) {
+    const float* dys = wg_smem + buf * bufw;
+    const float* xs = dys + WG_TV * 16;
+    if (u + G < units) {
+      stage(u + G, wg_smem + (buf ^ 1) * bufw);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncthreads();
+    for (int r = ks; r < rows; r += KS) {
+      const int ly = r % tl.ty, lz = r / tl.ty;
+      const float* xr = xs + (((lz + dz) * HY + ly) * HX) * XS + ci;
+      float w[3][3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) w[d][e] = xr[(d * HX + e) * XS];
+      int v = r * tl.tx;
+#pragma unroll 3
+      for (int lx = 0; lx < tl.tx; ++lx, ++v) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) w[d][2] = xr[(d * HX + lx + 2) * XS];
+        const int sw = (v >> 1) & 3;
+        const float4 p0 = reinterpret_cast<const float4*>(dys)[v * 4 + ((2 * cog) ^ sw)];
+        const float4 p1 = reinterpret_cast<const float4*>(dys)[v * 4 + ((2 * cog + 1) ^ sw)];
+        const float g8[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+#pragma unroll
+          for (int d = 0; d < 3; ++d)
+#pragma unroll
+            for (int e = 0; e < 3; ++e) s[c][d * 3 + e] = fmaf(g8[c], w[d][e], s[c][d * 3 + e]);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          w[d][0] = w[d][1];
+          w[d][1] = w[d][2];
+        }
+      }
+    }
+    if (bias) {
+      const int c = tid & 15, q = c >> 2;
+      for (int v = tid >> 4; v < TV; v += WG_NT / 16)
+        bsum += dys[(v * 4 + (q ^ ((v >> 1) & 3))) * 4 + (c & 3)];
+    }
     __syncthreads();
   }
-  if (tid < CT * taps && co0 + c < Co)
-    part[(size_t)g * Co * Ci * taps + ((size_t)(co0 + c) * Ci + ci) * taps + t] = s;
-}
-
-// dw[i] += sum_{g = 0..G-1} part[g][i], in that order.
-__global__ void k_wgrad_reduce(const float* __restrict__ part, float* __restrict__ dw, int64_t count,
-                               int G) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t st = (int64_t)gridDim.x * blockDim.x;
-  for (; i < count; i += st) {
-    float s = 0.f;
-    for (int g = 0; g < G; ++g) s += part[(size_t)g * count + i];
-    dw[i] += s;
+  // the KS row slices are added in order, through shared memory
+  const int slot = tid % (6 * CIT);
+  for (int k = 1; k < KS; ++k) {
+    if (ks == k)
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+#pragma unroll
+        for (int t = 0; t < 9; ++t) wg_smem[(c * 9 + t) * (6 * CIT) + slot] = s[c][t];
+    __syncthreads();
+    if (ks == 0)
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+#pragma unroll
+        for (int t = 0; t < 9; ++t) s[c][t] += wg_smem[(c * 9 + t) * (6 * CIT) + slot];
+    __syncthreads();
+  }
+  if (ks == 0 && ci0 + ci < Ci) {
+    float* po = part + (size_t)blockIdx.x * Co * Ci * 27;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int co = co0 + cog * 8 + c;
+      if (co < Co)
+#pragma unroll
+        for (int t = 0; t < 9; ++t) po[((size_t)co * Ci + ci0 + ci) * 27 + dz * 9 + t] = s[c][t];
+    }
+  }
+  if (bias) {
+    wg_smem[tid] = bsum;
+    __syncthreads();
+    if (tid < 16 && co0 + tid < Co) {
+      float t = 0.f;
+      for (int k = 0; k < WG_NT / 16; ++k) t += wg_smem[k * 16 + tid];
+      partb[(size_t)blockIdx.x * Co + co0 + tid] = t;
+    }
   }
 }
 
-// Bias gradient, deterministic: block (co, g) sums the fixed chunk g of the B * n^3 values of
-// channel co (tree reduction of fixed shape) into partb[co][g]; k_bias_reduce adds them in order.
-__global__ void k_bias_partial(const float* __restrict__ dy, float* __restrict__ partb, int B, int Co,
-                               int n, int GB) {
-  const int co = blockIdx.x, g = blockIdx.y;
-  const size_t nv = (size_t)n * n * n;
-  const size_t total = (size_t)B * nv, chunk = (total + GB - 1) / GB;
-  const size_t lo = (size_t)g * chunk, hi = lo + chunk < total ? lo + chunk : total;
-  float s = 0.f;
-  for (size_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-    const size_t b = i / nv, v = i % nv;
-    s += dy[(b * Co + co) * nv + v];
+// Weight gradient of a 1^3 convolution (the head): a thread walks voxels with 4 x 16 sums in
+// registers (4 output, 16 input channels per block), one coalesced load per channel; bound by
+// reading x and dy once.  The sums meet by a fixed shuffle tree, then over the warps in order.
+__global__ void __launch_bounds__(256) k_wgrad1(const float* __restrict__ x,
+                                                const float* __restrict__ dy,
+                                                float* __restrict__ part, float* __restrict__ partb,
+                                                int B, int Ci, int Co, int n, int G) {
+  __shared__ float red[8][68];
+  const int nci = (Ci + 15) / 16;
+  const int ci0 = (blockIdx.y % nci) * 16, co0 = (blockIdx.y / nci) * 4;
+  const int64_t nv = (int64_t)n * n * n;
+  const int64_t per = (nv * B + G - 1) / G;
+  const int64_t lo = blockIdx.x * per, hi = min(lo + per, nv * B);
+  float s[4][16], sb[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    sb[c] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) s[c][k] = 0.f;
   }
-  __shared__ float red[32];
-  s = warp_sum_f(s);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  for (int64_t i = lo + threadIdx.x; i < hi; i += 256) {
+    const int64_t b = i / nv, v = i - b * nv;
+    float g[4], xv[16];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) g[c] = co0 + c < Co ? __ldg(dy + (b * Co + co0 + c) * nv + v) : 0.f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) xv[k] = ci0 + k < Ci ? __ldg(x + (b * Ci + ci0 + k) * nv + v) : 0.f;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      sb[c] += g[c];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) s[c][k] = fmaf(g[c], xv[k], s[c][k]);
+    }
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const float t = warp_sum_f(s[c][k]);
+      if (lane == 0) red[warp][c * 16 + k] = t;
+    }
+    const float t = warp_sum_f(sb[c]);
+    if (lane == 0) red[warp][64 + c] = t;
+  }
   __syncthreads();
-  if (threadIdx.x < 32) {
-    float t = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
-    t = warp_sum_f(t);
-    if (threadIdx.x == 0) partb[(size_t)co * GB + g] = t;
+  if (threadIdx.x < 68) {
+    float t = 0.f;
+    for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+    if (threadIdx.x < 64) {
+      const int co = co0 + threadIdx.x / 16, ci = ci0 + threadIdx.x % 16;
+      if (co < Co && ci < Ci) part[((size_t)blockIdx.x * Co + co) * Ci + ci] = t;
+    } else if (partb && ci0 == 0 && co0 + (int)threadIdx.x - 64 < Co) {
+      partb[(size_t)blockIdx.x * Co + co0 + threadIdx.x - 64] = t;
+    }
   }
 }
 
-__global__ void k_bias_reduce(const float* __restrict__ partb, float* __restrict__ db, int Co, int GB) {
-  const int co = blockIdx.x * blockDim.x + threadIdx.x;
-  if (co >= Co) return;
+// dw[i] += sum_g part[g][i] (and db from partb): a block adds 32 values, its 8 warps the groups
+// g = w, w + 8, ..., then the warps' sums in order.
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ part,
+                                                      float* __restrict__ dw, int64_t count,
+                                                      const float* __restrict__ partb,
+                                                      float* __restrict__ db, int Co, int G) {
+  __shared__ float red[8][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t nb = (count + 31) / 32;
+  const bool isb = blockIdx.x >= nb;
+  const int64_t i = (isb ? blockIdx.x - nb : blockIdx.x) * 32 + lane, m = isb ? Co : count;
+  const float* p = isb ? partb : part;
   float s = 0.f;
-  for (int g = 0; g < GB; ++g) s += partb[(size_t)co * GB + g];
-  db[co] += s;
+  if (i < m) {
+#pragma unroll 4
+    for (int g = warp; g < G; g += 8) s += __ldg(p + (size_t)g * m + i);
+  }
+  red[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && i < m) {
+    float t = 0.f;
+    for (int w = 0; w < 8; ++w) t += red[w][lane];
+    (isb ? db : dw)[i] += t;
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -375,37 +553,91 @@ cudaError_t net_conv_dgrad(const float* dy, const void* w, void* wT_scratch, flo
   return net_conv_fwd(dy, wT_scratch, nullptr, dx, B, Co, Ci, n, ks, 0, 0, s);
 }
 
-// Partition of the weight-gradient sums: G voxel groups (about 2048 blocks in all, at most one
-// group per (batch, tile) unit), GB chunks per bias channel.
-static void wgrad_groups(int B, int Ci, int Co, int n, int* G, int* GB) {
-  const int units = tiles_of(n) * B;
-  const int cb = Ci * ((Co + CT - 1) / CT);
-  int g = (2048 + cb - 1) / cb;
-  *G = g < 1 ? 1 : (g > units ? units : g);
-  const int64_t total = (int64_t)B * n * n * n;
-  int64_t gb = (total + 8191) / 8192;
-  *GB = (int)(gb < 1 ? 1 : (gb > 64 ? 64 : gb));
+// Partition of the weight gradient: input channels per block (16, or the next power of two of
+// fewer), the voxel tile of a unit (rows of up to 32 voxels, split evenly so that 40 or 56 leave
+// no ragged end; ty grows while the tile has room, so that short rows keep a small halo), and the
+// number of groups G: one block per SM on 152 SMs (three for the 1^3 kernel, which waits on
+// memory), evened out over the units.
+struct WgPlan {
+  int cit, G;
+  WgTile tl;
+};
+static WgPlan wgrad_plan(int B, int Ci, int Co, int n, int ks) {
+  WgPlan p{};
+  const int64_t slots = 152 * (ks == 1 ? 3 : 1);
+  if (ks == 1) {
+    const int64_t nblk = (int64_t)((Ci + 15) / 16) * ((Co + 3) / 4);
+    const int64_t units = ((int64_t)B * n * n * n + 2047) / 2048;
+    const int64_t g = slots / nblk;
+    p.G = (int)(g < 1 ? 1 : (g > units ? units : g));
+    return p;
+  }
+  p.cit = Ci > 8 ? 16 : Ci > 4 ? 8 : Ci > 2 ? 4 : 2;
+  const auto even = [](int len, int most) {
+    const int k = (len + most - 1) / most;
+    return (len + k - 1) / k;
+  };
+  WgTile& t = p.tl;
+  t.tx = even(n, 32);
+  t.ty = even(n, t.tx > 16 ? 4 : t.tx > 8 ? 4 : 8);
+  const int room = WG_TV / (t.tx * t.ty);
+  t.tz = even(n, room < 1 ? 1 : (room > 4 ? 4 : room));
+  t.ntx = (n + t.tx - 1) / t.tx;
+  t.nty = (n + t.ty - 1) / t.ty;
+  t.ntz = (n + t.tz - 1) / t.tz;
+  const int64_t nblk = (int64_t)((Ci + p.cit - 1) / p.cit) * ((Co + 15) / 16);
+  const int64_t units = (int64_t)t.ntx * t.nty * t.ntz * B;
+  int64_t g = slots / nblk;
+  g = g < 1 ? 1 : (g > units ? units : g);
+  const int64_t rounds = (units + g - 1) / g;
+  p.G = (int)((units + rounds - 1) / rounds);
+  return p;
 }
 
 int64_t net_conv_wgrad_scratch(int B, int Ci, int Co, int n, int ks) {
-  int G, GB;
-  wgrad_groups(B, Ci, Co, n, &G, &GB);
-  return (int64_t)G * Co * Ci * ks * ks * ks + (int64_t)Co * GB;
+  const WgPlan p = wgrad_plan(B, Ci, Co, n, ks);
+  return (int64_t)p.G * Co * Ci * ks * ks * ks + (int64_t)p.G * Co;
+}
+
+template <int CIT>
+static cudaError_t launch_wgrad3(const float* x, const float* dy, float* part, float* partb, int B,
+                                 int Ci, int Co, int n, const WgPlan& p, cudaStream_t s) {
+  // two staging buffers, or the row slices' sums at the end
+  const auto words = [](int halo) { return 2 * ((WG_TV * 16 + halo * (CIT + 1) + 3) & ~3); };
+  const int fl = words((p.tl.tx + 2) * (p.tl.ty + 2) * (p.tl.tz + 2)), fe = 72 * 6 * CIT;
+  const int smem = 4 * (fl > fe ? fl : fe);
+  const int kMost = 4 * words(34 * 6 * 4);   // the largest tile's
+  static const cudaError_t set = cudaFuncSetAttribute(
+      k_wgrad3<CIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+  if (set != cudaSuccess) return set;
+  if (smem > kMost) return cudaErrorInvalidValue;
+  const dim3 grid(p.G, ((Ci + CIT - 1) / CIT) * ((Co + 15) / 16));
+  k_wgrad3<CIT><<<grid, WG_NT, smem, s>>>(x, dy, part, partb, B, Ci, Co, n, p.tl, p.G);
+  return cudaGetLastError();
 }
 
 cudaError_t net_conv_wgrad(const float* x, const float* dy, float* dw, float* db, float* scratch,
                            int B, int Ci, int Co, int n, int ks, cudaStream_t s) {
-  int G, GB;
-  wgrad_groups(B, Ci, Co, n, &G, &GB);
+  const WgPlan p = wgrad_plan(B, Ci, Co, n, ks);
   const int64_t count = (int64_t)Co * Ci * ks * ks * ks;
-  dim3 grid(G, Ci * ((Co + CT - 1) / CT));
-  k_conv_wgrad<<<grid, 512, 0, s>>>(x, dy, scratch, B, Ci, Co, n, ks, G);
-  k_wgrad_reduce<<<gs(count), 256, 0, s>>>(scratch, dw, count, G);
-  if (db) {
-    float* partb = scratch + (size_t)G * count;
-    k_bias_partial<<<dim3(Co, GB), 256, 0, s>>>(dy, partb, B, Co, n, GB);
-    k_bias_reduce<<<(Co + 127) / 128, 128, 0, s>>>(partb, db, Co, GB);
+  float* partb = db ? scratch + (size_t)p.G * count : nullptr;
+  cudaError_t e;
+  if (ks == 1) {
+    const dim3 grid(p.G, ((Ci + 15) / 16) * ((Co + 3) / 4));
+    k_wgrad1<<<grid, 256, 0, s>>>(x, dy, scratch, partb, B, Ci, Co, n, p.G);
+    e = cudaGetLastError();
+  } else if (p.cit == 16) {
+    e = launch_wgrad3<16>(x, dy, scratch, partb, B, Ci, Co, n, p, s);
+  } else if (p.cit == 8) {
+    e = launch_wgrad3<8>(x, dy, scratch, partb, B, Ci, Co, n, p, s);
+  } else if (p.cit == 4) {
+    e = launch_wgrad3<4>(x, dy, scratch, partb, B, Ci, Co, n, p, s);
+  } else {
+    e = launch_wgrad3<2>(x, dy, scratch, partb, B, Ci, Co, n, p, s);
   }
+  if (e != cudaSuccess) return e;
+  const unsigned nb = (unsigned)((count + 31) / 32 + (db ? (Co + 31) / 32 : 0));
+  k_wgrad_reduce<<<nb, 256, 0, s>>>(scratch, dw, count, partb, db, Co, p.G);
   return cudaGetLastError();
 }
 
