@@ -178,8 +178,7 @@ int lddmm_dice(lddmm_ctx* ctx, const uint16_t* A, const uint16_t* B, int64_t n, 
  * out[0] = d_H = max of both directed maxima; out[1] = d_M = median of the union of the directed
  * distances of S_A to S_B and of S_B to S_A (mean of the two middle values for an even count);
  * out[2], out[3] = the number of surface voxels of A and of B.  Host memory.
- * Allocates scratch for the surface lists and distances for the duration of the call and waits
- * for the result (bounded).  LDDMM_ERR_INVALID_ARG when a mask has no surface voxel. */
+ * Uses the context's work buffers (no allocation) and waits for the result (bounded).  LDDMM_ERR_INVALID_ARG when a mask has no surface voxel. */
 int lddmm_surface_distance(lddmm_ctx* ctx, const uint8_t* A, const uint8_t* B, double out[4]);
 
 /* Landmark errors e_k = |phi(x_k) - y_k| (§2.7) for the current v: phi(x) = x + u01(x) carries

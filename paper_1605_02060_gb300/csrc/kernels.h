@@ -92,20 +92,25 @@ void launch_from_storage(const void* src, float* dst, int64_t n, cudaStream_t s,
 // *flag |= bit when a[0..n) holds a NaN or an infinity.
 void launch_check_finite(const float* a, int64_t n, int* flag, cudaStream_t s, int bit = 1);
 void launch_fill(float* a, int64_t n, float value, cudaStream_t s);
-void launch_dice_hist(const uint16_t* A, const uint16_t* B, int64_t n,
-                      unsigned long long* hist /* 3 x 65536 */, cudaStream_t s);
+// hist (3 x 65536, zeroed): voxels per label of A, of B and of both at once; out = mean Dice over
+// the labels > 0 present in either (1 when there are none).
+void launch_dice(const uint16_t* A, const uint16_t* B, int64_t n,
+                 unsigned long long* hist /* 3 x 65536 */, double* out, cudaStream_t s);
 
 // ---- registration-quality measures of §2.7 (kernels_metrics.cu) ----
-// Surface voxels of mask m appended to list as (x, y, z, 0); *count receives their number
-// (entries past cap are counted but not written, so cap = 0 only counts).
-cudaError_t surface_list(const Grid& g, const uint8_t* m, int4* list, unsigned* count,
-                         unsigned cap, cudaStream_t s);
-// d[i] = distance (physical units) from src[i] to the nearest point of dst.
-cudaError_t nearest_distances(const int4* src, unsigned ns, const int4* dst, unsigned nd,
-                              float hx, float hy, float hz, double* d, cudaStream_t s);
-// out[0] = max of d[0..n), out[1] = k1-th, out[2] = k2-th smallest (0-based); one block.
-cudaError_t order_stats(const double* d, unsigned n, unsigned k1, unsigned k2, double* out,
-                        cudaStream_t s);
+// 8x8x8-voxel cells of a grid.
+int64_t surface_cells(const Grid& g);
+int64_t surface_select_bytes();
+// start[0..cells) and start[cells + 1 ..]: where each cell's surface voxels of mask A, of mask B
+// begin; start[cells], start[2 cells + 1]: their numbers.
+cudaError_t surface_count(const Grid& g, const uint8_t* A, const uint8_t* B, unsigned* start,
+                          cudaStream_t s);
+// After surface_count: list (na + nb entries), the directed distances dA (na) and dB (nb), sel
+// (surface_select_bytes() of scratch) and out[0] = their maximum, out[1], out[2] = the two middle values (equal for an odd number).
+cudaError_t surface_distances(const Grid& g, const uint8_t* A, const uint8_t* B, unsigned* start,
+                              uint16_t* list, unsigned na, unsigned nb, float hx, float hy,
+                              float hz, double* dA, double* dB, void* sel, double* out,
+                              cudaStream_t s);
 // e[k] = |(x_k + u01(x_k) - y_k) h| for n points (float [n][3], voxel coordinates).
 cudaError_t landmark_errors(const Grid& g, const float* u01, const float* xk, const float* yk,
                             int n, float hx, float hy, float hz, double* e, cudaStream_t s);

@@ -965,22 +965,102 @@ void launch_fill(float* a, int64_t n, float value, cudaStream_t s) {
   k_fill<<<152 * 8, 256, 0, s>>>(a, n, value);
 }
 
-__global__ void k_dice_hist(const uint16_t* __restrict__ A, const uint16_t* __restrict__ B,
-                            int64_t n, unsigned long long* hist) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (; i < n; i += stride) {
-    const unsigned a = A[i], b = B[i];
-    if (a) atomicAdd(&hist[a], 1ull);
-    if (b) atomicAdd(&hist[65536 + b], 1ull);
-    if (a && a == b) atomicAdd(&hist[2 * 65536 + a], 1ull);
+// Label counts for Dice.  Neighbouring voxels mostly carry one label: a lane reads 8 voxels
+// (16 bytes of each map where the maps are aligned), a warp adds each distinct label of its
+// lanes' uniform groups once, and labels below kDiceSm are counted in shared memory first.  (A
+// global 64-bit atomic per voxel and map took 631 us at 264x160x228; this takes 17 us.)
+constexpr int kDiceSm = 2048;
+
+__global__ void __launch_bounds__(512) k_dice_hist(const uint16_t* __restrict__ A,
+                                                   const uint16_t* __restrict__ B, int64_t n,
+                                                   int vec, unsigned long long* hist) {
+  __shared__ unsigned sh[3 * kDiceSm];
+  for (int i = threadIdx.x; i < 3 * kDiceSm; i += blockDim.x) sh[i] = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  auto add = [&](int which, unsigned label, unsigned c) {
+    if (label < kDiceSm) atomicAdd(&sh[which * kDiceSm + label], c);
+    else atomicAdd(&hist[(size_t)which * 65536 + label], (unsigned long long)c);
+  };
+  const int64_t groups = (n + 7) / 8;
+  for (int64_t g0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll; g0 < groups;
+       g0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t g = g0 + lane, i0 = g * 8;
+    __align__(16) uint16_t a[8], b[8];
+    if (vec && i0 + 8 <= n) {
+      *reinterpret_cast<uint4*>(a) = __ldg(reinterpret_cast<const uint4*>(A + i0));
+      *reinterpret_cast<uint4*>(b) = __ldg(reinterpret_cast<const uint4*>(B + i0));
+    } else {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        a[k] = i0 + k < n ? A[i0 + k] : 0;
+        b[k] = i0 + k < n ? B[i0 + k] : 0;
+      }
+    }
+    bool ua = true, ub = true;
+#pragma unroll
+    for (int k = 1; k < 8; ++k) {
+      ua = ua && a[k] == a[0];
+      ub = ub && b[k] == b[0];
+    }
+    // lanes whose 8 voxels carry one label: the lanes of equal labels count together
+    const unsigned ka = ua ? a[0] : 0u, kb = ub ? b[0] : 0u, kc = ua && ub && a[0] == b[0] ? a[0] : 0u;
+    const unsigned key[3] = {ka, kb, kc};
+#pragma unroll
+    for (int w = 0; w < 3; ++w) {
+      if (!__any_sync(0xffffffffu, key[w])) continue;
+      const unsigned peers = __match_any_sync(0xffffffffu, key[w]);
+      if (key[w] && lane == __ffs(peers) - 1) add(w, key[w], 8u * __popc(peers));
+    }
+    if (!ua || !ub) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        if (!ua && a[k]) add(0, a[k], 1u);
+        if (!ub && b[k]) add(1, b[k], 1u);
+        if (a[k] && a[k] == b[k]) add(2, a[k], 1u);
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 3 * kDiceSm; i += blockDim.x)
+    if (sh[i]) atomicAdd(&hist[(size_t)(i / kDiceSm) * 65536 + i % kDiceSm], (unsigned long long)sh[i]);
+}
+
+// Mean over the labels 1..65535 present in either map of 2 |both| / (|A| + |B|), summed in FP64 in
+// a fixed order; one block.
+__global__ void __launch_bounds__(1024) k_dice_mean(const unsigned long long* __restrict__ hist,
+                                                    double* out) {
+  __shared__ double rs[32], rc[32];
+  double s = 0.0, c = 0.0;
+#pragma unroll 4
+  for (int l = threadIdx.x; l < 65536; l += 1024) {
+    const unsigned long long na = hist[l], nb = hist[65536 + l];
+    if (l == 0 || na + nb == 0) continue;
+    s += 2.0 * (double)hist[2 * 65536 + l] / (double)(na + nb);
+    c += 1.0;
+  }
+  s = warp_sum(s);
+  c = warp_sum(c);
+  if ((threadIdx.x & 31) == 0) {
+    rs[threadIdx.x >> 5] = s;
+    rc[threadIdx.x >> 5] = c;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    s = warp_sum(rs[threadIdx.x]);
+    c = warp_sum(rc[threadIdx.x]);
+    if (threadIdx.x == 0) *out = c > 0.0 ? s / c : 1.0;
   }
 }
 
-void launch_dice_hist(const uint16_t* A, const uint16_t* B, int64_t n, unsigned long long* hist,
-                      cudaStream_t s) {
-  if (n <= 0) return;
-  k_dice_hist<<<152 * 8, 256, 0, s>>>(A, B, n, hist);
+void launch_dice(const uint16_t* A, const uint16_t* B, int64_t n, unsigned long long* hist,
+                 double* out, cudaStream_t s) {
+  if (n > 0) {
+    const int64_t nb = (n + 8 * 512 - 1) / (8 * 512);
+    const int vec = (((uintptr_t)A | (uintptr_t)B) & 15) == 0;
+    k_dice_hist<<<(int)(nb < 152 * 4 ? nb : 152 * 4), 512, 0, s>>>(A, B, n, vec, hist);
+  }
+  k_dice_mean<<<1, 1024, 0, s>>>(hist, out);
 }
 
 }  // namespace lddmm

@@ -57,7 +57,7 @@ struct lddmm_ctx {
   Acc* acc_init = nullptr;  // the accumulators' start value (device copy, written at creation)
   Acc* acc_host = nullptr;  // pinned
   int* flag = nullptr;      // device int
-  unsigned long long* hist = nullptr;  // 3 x 65536
+  unsigned long long* hist = nullptr;  // 3 x 65536, and the mean Dice
   // map state
   const float* u10 = nullptr;
   const float* u01 = nullptr;
@@ -675,9 +675,9 @@ int lddmm_create(const lddmm_params* p, const float* I0, const float* I1, const 
        A(dalloc(&ctx->uB[0], 4 * N)) && A(dalloc(&ctx->uB[1], 4 * N)) &&
        A(dalloc(&ctx->uF[0], 4 * N)) && A(dalloc(&ctx->uF[1], 4 * N)) &&
        A(dalloc(&ctx->J1, T * N)) && A(dalloc(&ctx->W, T * N)) && A(dalloc(&ctx->b, ctx->kcap)) &&
-       A(dalloc(&ctx->work, ctx->kcap)) && A(dalloc(&ctx->J0T, N)) && A(dalloc(&ctx->stage, 3 * N)) &&
+       A(dalloc(&ctx->work, ctx->kcap)) && A(dalloc(&ctx->J0T, N)) && A(dalloc(&ctx->stage, 3 * N + 64 + surface_select_bytes() / 4)) &&
        A(dalloc(&ctx->acc, 1)) && A(dalloc(&ctx->acc_init, 1)) && A(dalloc(&ctx->flag, 1)) &&
-       A(dalloc(&ctx->hist, 3 * 65536)) &&
+       A(dalloc(&ctx->hist, 3 * 65536 + 1)) &&
        A(cudaMallocHost((void**)&ctx->acc_host, sizeof(Acc)));
   if (ok && (p->flags & 1)) ok = A(dalloc(&ctx->v_prev, ve));
   g_fail_alloc_countdown = 0;
@@ -876,22 +876,15 @@ int lddmm_dice(lddmm_ctx* ctx, const uint16_t* A, const uint16_t* B, int64_t n, 
     if (!db) { CK(cudaMemcpyAsync(tmp + n, B, n * 2, cudaMemcpyDefault, ctx->stream)); b = tmp + n; }
   }
   CK(cudaMemsetAsync(ctx->hist, 0, 3 * 65536 * sizeof(unsigned long long), ctx->stream));
-  launch_dice_hist(a, b, n, ctx->hist, ctx->stream);
+  // the mean goes through the pinned accumulator block (free outside an energy read)
+  double* mean = reinterpret_cast<double*>(ctx->hist + 3 * 65536);
+  launch_dice(a, b, n, ctx->hist, mean, ctx->stream);
   CK(cudaGetLastError());
-  std::vector<unsigned long long> h(3 * 65536);
-  CK(cudaMemcpyAsync(h.data(), ctx->hist, h.size() * 8, cudaMemcpyDeviceToHost, ctx->stream));
+  CK(cudaMemcpyAsync(ctx->acc_host, mean, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
   int rc = wait_stream(ctx);
   if (tmp) cudaFree(tmp);
   if (rc) return rc;
-  double s = 0.0;
-  int cnt = 0;
-  for (int l = 1; l < 65536; ++l) {
-    const unsigned long long na = h[l], nb = h[65536 + l], ni = h[2 * 65536 + l];
-    if (na + nb == 0) continue;
-    s += 2.0 * (double)ni / (double)(na + nb);
-    ++cnt;
-  }
-  *out = cnt ? s / cnt : 1.0;
+  std::memcpy(out, ctx->acc_host, sizeof(double));
   return LDDMM_OK;
 }
 
@@ -900,61 +893,51 @@ int lddmm_surface_distance(lddmm_ctx* ctx, const uint8_t* A, const uint8_t* B, d
   const Level& L = ctx->levels[ctx->cur];
   const Grid& g = L.g;
   cudaStream_t s = ctx->stream;
-  // scratch: host masks, the two counters, then the lists and distances once sized
-  uint8_t* mk = nullptr;
-  unsigned* cnt = nullptr;
-  int4* list = nullptr;
-  double* d = nullptr;
-  double* st = nullptr;
-  auto done = [&](int rc) {
-    cudaStreamSynchronize(s);
-    cudaFree(mk); cudaFree(cnt); cudaFree(list); cudaFree(d); cudaFree(st);
-    cudaGetLastError();
-    return rc;
+  // Scratch in the context's own buffers (all free between calls): stage holds the cells' starts
+  // (8 bytes per 8x8x8 cell and 8 more), the order statistics, host masks (2 N bytes) and the
+  // voxel lists (at most 4 N bytes); b and work hold the distances (at most 8 N bytes each).
+  const int64_t ncell = surface_cells(g);
+  char* p = reinterpret_cast<char*>(ctx->stage);
+  auto take = [&](int64_t bytes) {
+    char* q = p;
+    p += (bytes + 15) / 16 * 16;
+    return q;
   };
+  double* st = reinterpret_cast<double*>(take(3 * sizeof(double)));
+  unsigned* start = reinterpret_cast<unsigned*>(take(2 * (ncell + 1) * sizeof(unsigned)));
+  uint8_t* mk = reinterpret_cast<uint8_t*>(take(2 * (int64_t)g.N));
+  uint16_t* list = reinterpret_cast<uint16_t*>(take(4 * (int64_t)g.N));
+  void* sel = take(surface_select_bytes());
+  double* dA = reinterpret_cast<double*>(ctx->b);
+  double* dB = reinterpret_cast<double*>(ctx->work);
   const uint8_t* ma = A;
   const uint8_t* mb = B;
-  const bool da = is_device_ptr(A), db = is_device_ptr(B);
-  if (cudaMalloc((void**)&cnt, 2 * sizeof(unsigned)) != cudaSuccess ||
-      cudaMalloc((void**)&st, 3 * sizeof(double)) != cudaSuccess)
-    return done(fail(ctx, LDDMM_ERR_OOM, "device allocation failed"));
-  if (!da || !db) {
-    if (cudaMalloc((void**)&mk, 2 * (size_t)g.N) != cudaSuccess)
-      return done(fail(ctx, LDDMM_ERR_OOM, "device allocation failed"));
-    if (!da) { cudaMemcpyAsync(mk, A, g.N, cudaMemcpyDefault, s); ma = mk; }
-    if (!db) { cudaMemcpyAsync(mk + g.N, B, g.N, cudaMemcpyDefault, s); mb = mk + g.N; }
+  if (!is_device_ptr(A)) {
+    CK(cudaMemcpyAsync(mk, A, g.N, cudaMemcpyDefault, s));
+    ma = mk;
   }
-  // count the surface voxels, then list them
-  unsigned h[2] = {0, 0};
-  cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned), s);
-  surface_list(g, ma, nullptr, cnt, 0u, s);
-  surface_list(g, mb, nullptr, cnt + 1, 0u, s);
-  cudaMemcpyAsync(h, cnt, sizeof(h), cudaMemcpyDeviceToHost, s);
+  if (!is_device_ptr(B)) {
+    CK(cudaMemcpyAsync(mk + g.N, B, g.N, cudaMemcpyDefault, s));
+    mb = mk + g.N;
+  }
+  // the results go through the pinned accumulator block (free outside an energy read)
+  CK(surface_count(g, ma, mb, start, s));
+  unsigned* h = reinterpret_cast<unsigned*>(ctx->acc_host);
+  CK(cudaMemcpyAsync(h, start + ncell, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+  CK(cudaMemcpyAsync(h + 1, start + 2 * ncell + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, s));
   int rc = wait_stream(ctx);
-  if (rc) return done(rc);
-  if (cudaGetLastError() != cudaSuccess) return done(fail(ctx, LDDMM_ERR_CUDA, "surface count failed"));
-  if (h[0] == 0 || h[1] == 0) return done(fail(ctx, LDDMM_ERR_INVALID_ARG, "a mask has no surface voxel"));
+  if (rc) return rc;
   const unsigned na = h[0], nb = h[1];
-  if (cudaMalloc((void**)&list, (size_t)(na + nb) * sizeof(int4)) != cudaSuccess ||
-      cudaMalloc((void**)&d, (size_t)(na + nb) * sizeof(double)) != cudaSuccess)
-    return done(fail(ctx, LDDMM_ERR_OOM, "device allocation failed"));
-  cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned), s);
-  surface_list(g, ma, list, cnt, na, s);
-  surface_list(g, mb, list + na, cnt + 1, nb, s);
-  nearest_distances(list, na, list + na, nb, L.hx, L.hy, L.hz, d, s);
-  nearest_distances(list + na, nb, list, na, L.hx, L.hy, L.hz, d + na, s);
-  const unsigned n = na + nb;
-  order_stats(d, n, (n - 1) / 2, n / 2, st, s);
-  double r[3];
-  cudaMemcpyAsync(r, st, sizeof(r), cudaMemcpyDeviceToHost, s);
-  if (cudaGetLastError() != cudaSuccess) return done(fail(ctx, LDDMM_ERR_CUDA, "surface distance launch failed"));
-  rc = wait_stream(ctx);
-  if (rc) return done(rc);
+  if (na == 0 || nb == 0) return fail(ctx, LDDMM_ERR_INVALID_ARG, "a mask has no surface voxel");
+  CK(surface_distances(g, ma, mb, start, list, na, nb, L.hx, L.hy, L.hz, dA, dB, sel, st, s));
+  double* r = reinterpret_cast<double*>(ctx->acc_host);
+  CK(cudaMemcpyAsync(r, st, 3 * sizeof(double), cudaMemcpyDeviceToHost, s));
+  if ((rc = wait_stream(ctx))) return rc;
   out[0] = r[0];
   out[1] = 0.5 * (r[1] + r[2]);
   out[2] = (double)na;
   out[3] = (double)nb;
-  return done(LDDMM_OK);
+  return LDDMM_OK;
 }
 
 int lddmm_shoot(lddmm_ctx* ctx, const float* v0) {
