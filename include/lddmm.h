@@ -214,8 +214,8 @@ int lddmm_histogram_match(const float* I0, const float* M0, const float* I1, con
  * (erosion, then dilation), then closed with the ball of radius r_close (dilation, then
  * erosion); ball = offsets with dx^2 + dy^2 + dz^2 <= r^2; voxels beyond the grid count as
  * background (the paper: 50 um and 125 um radii).  I: float [nz][ny][nx], out: uint8, device
- * memory.  r_open, r_close in [0, 16] (0 skips that step).  Allocates one scratch volume for
- * the duration of the call and waits for it (bounded).  No context. */
+ * memory.  r_open, r_close in [0, 16] (0 skips that step).  Allocates scratch (two bits per
+ * voxel) for the duration of the call and waits for it (bounded).  No context. */
 int lddmm_mask_morphology(const float* I, int nx, int ny, int nz, float threshold, int r_open,
                           int r_close, uint8_t* out, void* stream);
 

@@ -1032,32 +1032,17 @@ int lddmm_histogram_match(const float* I0, const float* M0, const float* I1, con
   for (const void* p : ps)
     if (!is_device_ptr(p)) return fail(nullptr, LDDMM_ERR_INVALID_ARG, "device memory expected");
   cudaStream_t s = (cudaStream_t)stream;
-  // scratch: two range records (3 ints each, 16-byte slots), two histograms, the nodes
-  char* scr = nullptr;
-  const size_t hb = (size_t)bins * sizeof(unsigned long long);
-  if (cudaMalloc((void**)&scr, 32 + 2 * hb + 2 * 66 * sizeof(double)) != cudaSuccess) {
+  void* scr = nullptr;
+  if (cudaMalloc(&scr, match_scratch_bytes(bins)) != cudaSuccess) {
     cudaGetLastError();
     return fail(nullptr, LDDMM_ERR_OOM, "device allocation failed");
   }
-  int* st0 = reinterpret_cast<int*>(scr);
-  int* st1 = st0 + 4;
-  unsigned long long* c0 = reinterpret_cast<unsigned long long*>(scr + 32);
-  unsigned long long* c1 = c0 + bins;
-  double* nodes = reinterpret_cast<double*>(scr + 32 + 2 * hb);
   int cnt[8] = {0};
-  cudaError_t e = masked_range(I0, M0, n, st0, s);
-  if (e == cudaSuccess) e = masked_range(I1, M1, n, st1, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(cnt, scr, 32, cudaMemcpyDeviceToHost, s);
+  cudaError_t e = histogram_match(I0, M0, I1, M1, n, bins, points, scr, out, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(cnt, scr, sizeof(cnt), cudaMemcpyDeviceToHost, s);
   int rc = e == cudaSuccess ? wait_plain(s) : fail(nullptr, LDDMM_ERR_CUDA, cudaGetErrorString(e));
   if (rc == LDDMM_OK && (cnt[2] == 0 || cnt[6] == 0))
     rc = fail(nullptr, LDDMM_ERR_INVALID_ARG, "a mask is empty");
-  if (rc == LDDMM_OK) {
-    e = masked_hist(I0, M0, n, st0, bins, c0, s);
-    if (e == cudaSuccess) e = masked_hist(I1, M1, n, st1, bins, c1, s);
-    if (e == cudaSuccess) e = match_nodes(st0, c0, st1, c1, bins, points, nodes, s);
-    if (e == cudaSuccess) e = apply_match(I0, M0, n, nodes, points, out, s);
-    rc = e == cudaSuccess ? wait_plain(s) : fail(nullptr, LDDMM_ERR_CUDA, cudaGetErrorString(e));
-  }
   cudaFree(scr);
   return rc;
 }
@@ -1069,25 +1054,27 @@ int lddmm_mask_morphology(const float* I, int nx, int ny, int nz, float threshol
     return fail(nullptr, LDDMM_ERR_INVALID_ARG, "bad argument");
   if (!is_device_ptr(I) || !is_device_ptr(out))
     return fail(nullptr, LDDMM_ERR_INVALID_ARG, "device memory expected");
-  const Grid g{nx, ny, nz, (int64_t)nx * ny * nz};
   cudaStream_t s = (cudaStream_t)stream;
-  uint8_t* tmp = nullptr;
-  if (cudaMalloc((void**)&tmp, (size_t)g.N) != cudaSuccess) {
+  const int64_t words = mask_bits_words(nx, ny, nz);
+  uint32_t* bits = nullptr;
+  if (cudaMalloc((void**)&bits, (size_t)(2 * words) * sizeof(uint32_t)) != cudaSuccess) {
     cudaGetLastError();
     return fail(nullptr, LDDMM_ERR_OOM, "device allocation failed");
   }
-  // out -> tmp -> out per pair of operations
-  cudaError_t e = threshold_mask(I, g.N, threshold, out, s);
-  if (e == cudaSuccess && r_open > 0) {
-    e = ball_op(g, out, r_open, true, tmp, s);
-    if (e == cudaSuccess) e = ball_op(g, tmp, r_open, false, out, s);
+  uint32_t* m = bits;
+  uint32_t* tmp = bits + words;
+  cudaError_t e = threshold_bits(I, nx, ny, nz, threshold, m, s);
+  if (r_open > 0) {
+    if (e == cudaSuccess) e = ball_bits(nx, ny, nz, m, r_open, true, tmp, s);
+    if (e == cudaSuccess) e = ball_bits(nx, ny, nz, tmp, r_open, false, m, s);
   }
-  if (e == cudaSuccess && r_close > 0) {
-    e = ball_op(g, out, r_close, false, tmp, s);
-    if (e == cudaSuccess) e = ball_op(g, tmp, r_close, true, out, s);
+  if (r_close > 0) {
+    if (e == cudaSuccess) e = ball_bits(nx, ny, nz, m, r_close, false, tmp, s);
+    if (e == cudaSuccess) e = ball_bits(nx, ny, nz, tmp, r_close, true, m, s);
   }
+  if (e == cudaSuccess) e = unpack_bits(nx, ny, nz, m, out, s);
   const int rc = e == cudaSuccess ? wait_plain(s) : fail(nullptr, LDDMM_ERR_CUDA, cudaGetErrorString(e));
-  cudaFree(tmp);
+  cudaFree(bits);
   return rc;
 }
 
