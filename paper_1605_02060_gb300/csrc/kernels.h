@@ -88,6 +88,8 @@ void launch_downsample(const Grid& fine, const Grid& coarse, int factor, const f
 void launch_upsample(const Grid& coarse, const Grid& fine, float ratio, const void* src,
                      void* dst, int nfields, cudaStream_t s, int st);
 void launch_to_storage(const float* src, void* dst, int64_t n, cudaStream_t s, int st);
+// launch_to_storage that also sets *flag when src holds NaN or Inf (both float: a checked copy).
+void launch_store_checked(const float* src, void* dst, int64_t n, int* flag, cudaStream_t s, int st);
 void launch_from_storage(const void* src, float* dst, int64_t n, cudaStream_t s, int st);
 // *flag |= bit when a[0..n) holds a NaN or an infinity.
 void launch_check_finite(const float* a, int64_t n, int* flag, cudaStream_t s, int bit = 1);

@@ -917,26 +917,79 @@ void launch_upsample(const Grid& coarse, const Grid& fine, float ratio, const vo
 
 // --------------------------------------------------------------------------------------------
 // Storage conversion (fp32 <-> bf16, round to nearest) for the precision form.
-__global__ void k_to_bf16(const float* __restrict__ a, __nv_bfloat16* __restrict__ b, int64_t n) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (; i < n; i += stride) b[i] = __float2bfloat16_rn(a[i]);
+// A block takes 4096 elements, a thread 4 consecutive ones four times over with all its loads
+// requested first, where both arrays allow 16-byte (float) and 8-byte (bf16) accesses; else (and
+// in the last block) one element at a time.
+template <typename T> struct Quad;
+template <> struct Quad<float> {
+  typedef float4 V;
+  static __device__ __forceinline__ float4 get(V v) { return v; }
+  static __device__ __forceinline__ V put(float4 f) { return f; }
+};
+template <> struct Quad<__nv_bfloat16> {
+  typedef uint2 V;
+  static __device__ __forceinline__ float4 get(V v) {
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
+                       __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+  }
+  static __device__ __forceinline__ V put(float4 f) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(f.x, f.y), b = __floats2bfloat162_rn(f.z, f.w);
+    return make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+  }
+};
+
+// dst = src in the destination's type; CHECK: *flag |= bit when src holds NaN or Inf.  One pass over
+// memory for a field that is stored and checked (a copy and a scan took 525 us for the 1.16 GB
+// velocity of 264x160x228, T = 10; this takes 321 us, 7.2 TB/s).
+template <typename S, typename D, bool CHECK>
+__global__ void __launch_bounds__(256) k_convert(const S* __restrict__ src, D* __restrict__ dst,
+                                                 int64_t n, int vec, int* flag, int bit) {
+  // block b: elements 4096 b .. 4096 b + 4095, 4 x 1024 of them contiguous
+  const int64_t b0 = (int64_t)blockIdx.x * 4096;
+  int bad = 0;
+  if (vec && b0 + 4096 <= n) {
+    const typename Quad<S>::V* s4 = reinterpret_cast<const typename Quad<S>::V*>(src + b0) + threadIdx.x;
+    typename Quad<D>::V* d4 = reinterpret_cast<typename Quad<D>::V*>(dst + b0) + threadIdx.x;
+    float4 f[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) f[k] = Quad<S>::get(__ldg(s4 + k * 256));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (CHECK)
+        bad |= !isfinite(f[k].x) | !isfinite(f[k].y) | !isfinite(f[k].z) | !isfinite(f[k].w);
+      d4[k * 256] = Quad<D>::put(f[k]);
+    }
+  } else {
+    for (int64_t i = b0 + threadIdx.x; i < min(b0 + 4096, n); i += 256) {
+      const float f = ldf(src + i);
+      if (CHECK) bad |= !isfinite(f);
+      stf(dst + i, f);
+    }
+  }
+  if (CHECK && bad) atomicOr(flag, bit);
 }
-__global__ void k_to_f32(const __nv_bfloat16* __restrict__ a, float* __restrict__ b, int64_t n) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (; i < n; i += stride) b[i] = __bfloat162float(a[i]);
+
+template <typename S, typename D, bool CHECK>
+static void convert(const S* src, D* dst, int64_t n, int* flag, int bit, cudaStream_t s) {
+  const int vec = (uintptr_t)src % (4 * sizeof(S)) == 0 && (uintptr_t)dst % (4 * sizeof(D)) == 0;
+  k_convert<S, D, CHECK><<<(unsigned)((n + 4095) / 4096), 256, 0, s>>>(src, dst, n, vec, flag, bit);
 }
 
 void launch_to_storage(const float* src, void* dst, int64_t n, cudaStream_t s, int st) {
   if (n <= 0) return;
-  if (st) k_to_bf16<<<152 * 8, 256, 0, s>>>(src, (__nv_bfloat16*)dst, n);
+  if (st) convert<float, __nv_bfloat16, false>(src, (__nv_bfloat16*)dst, n, nullptr, 0, s);
   else cudaMemcpyAsync(dst, src, n * sizeof(float), cudaMemcpyDeviceToDevice, s);
+}
+
+void launch_store_checked(const float* src, void* dst, int64_t n, int* flag, cudaStream_t s, int st) {
+  if (n <= 0) return;
+  if (st) convert<float, __nv_bfloat16, true>(src, (__nv_bfloat16*)dst, n, flag, 1, s);
+  else convert<float, float, true>(src, (float*)dst, n, flag, 1, s);
 }
 
 void launch_from_storage(const void* src, float* dst, int64_t n, cudaStream_t s, int st) {
   if (n <= 0) return;
-  if (st) k_to_f32<<<152 * 8, 256, 0, s>>>((const __nv_bfloat16*)src, dst, n);
+  if (st) convert<__nv_bfloat16, float, false>((const __nv_bfloat16*)src, dst, n, nullptr, 0, s);
   else cudaMemcpyAsync(dst, src, n * sizeof(float), cudaMemcpyDeviceToDevice, s);
 }
 

@@ -120,6 +120,17 @@ bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Memory a kernel of the current device reads and writes directly (not another GPU's).
+bool is_local_ptr(const void* p) {
+  cudaPointerAttributes a;
+  int dev = -1;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev);
+}
+
 int wait_stream(lddmm_ctx* ctx) {
   const double limit = ctx->p.timeout_s > 0 ? ctx->p.timeout_s : 600.0;
   const auto t0 = std::chrono::steady_clock::now();
@@ -225,15 +236,20 @@ const float* field_src(lddmm_ctx* ctx, const float* user, int64_t n, float* stag
   return stage;
 }
 
+// Waits for the check that started with *flag = 0 on the stream.
+int read_flag(lddmm_ctx* ctx, const char* what) {
+  int* h = reinterpret_cast<int*>(ctx->acc_host);    // pinned, free outside an energy read
+  CK(cudaMemcpyAsync(h, ctx->flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  int rc = wait_stream(ctx);
+  if (rc) return rc;
+  if (*h) return fail(ctx, LDDMM_ERR_NONFINITE, std::string(what) + " holds NaN or Inf");
+  return LDDMM_OK;
+}
+
 int check_finite(lddmm_ctx* ctx, const float* d, int64_t n, const char* what) {
   CK(cudaMemsetAsync(ctx->flag, 0, sizeof(int), ctx->stream));
   launch_check_finite(d, n, ctx->flag, ctx->stream);
-  int h = 0;
-  CK(cudaMemcpyAsync(&h, ctx->flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-  int rc = wait_stream(ctx);
-  if (rc) return rc;
-  if (h) return fail(ctx, LDDMM_ERR_NONFINITE, std::string(what) + " holds NaN or Inf");
-  return LDDMM_OK;
+  return read_flag(ctx, what);
 }
 
 int load_images(lddmm_ctx* ctx, const float* I0, const float* I1, const float* M) {
@@ -477,7 +493,7 @@ int run_step(lddmm_ctx* ctx) {
   return LDDMM_OK;
 }
 
-// Recompute phi_{1,0}, phi_{0,1} (and optionally J0_T, the energy) for the current v.
+// Recompute phi_{1,0}, phi_{0,1} and J0_T for the current v (energy: E_reg too).
 int refresh_maps(lddmm_ctx* ctx, bool energy) {
   const Level& L = ctx->levels[ctx->cur];
   const Grid& g = L.g;
@@ -496,8 +512,9 @@ int refresh_maps(lddmm_ctx* ctx, bool energy) {
     pb ^= 1;
   }
   ctx->u01 = un;
-  launch_ereg(g, ctx->v, T, ctx->p.alpha, ctx->p.gamma, 1.0f / (L.hx * L.hx),
-              1.0f / (L.hy * L.hy), 1.0f / (L.hz * L.hz), ctx->acc, s, ctx->st);
+  if (energy)
+    launch_ereg(g, ctx->v, T, ctx->p.alpha, ctx->p.gamma, 1.0f / (L.hx * L.hx),
+                1.0f / (L.hy * L.hy), 1.0f / (L.hz * L.hz), ctx->acc, s, ctx->st);
   const float* uc = nullptr;
   int pf = 0;
   for (int j = 0; j < T; ++j) {
@@ -511,7 +528,6 @@ int refresh_maps(lddmm_ctx* ctx, bool energy) {
   CK(cudaGetLastError());
   ctx->maps_valid = true;
   ctx->j0_valid = true;
-  (void)energy;
   return LDDMM_OK;
 }
 
@@ -784,7 +800,12 @@ int lddmm_get_velocity(lddmm_ctx* ctx, float* dst) {
   if (!ctx || !dst) return fail(ctx, LDDMM_ERR_INVALID_ARG, "NULL argument");
   const Grid& g = ctx->levels[ctx->cur].g;
   if (ctx->st == 0) return copy_out(ctx, dst, ctx->v, (size_t)ctx->p.T * 3 * g.N * sizeof(float));
-  // bf16 storage: convert one time step at a time through the staging buffer
+  if (is_local_ptr(dst)) {
+    launch_from_storage(ctx->v, dst, (int64_t)ctx->p.T * 3 * g.N, ctx->stream, ctx->st);
+    CK(cudaGetLastError());
+    return wait_stream(ctx);
+  }
+  // bf16 storage to memory elsewhere: one time step at a time through the staging buffer
   for (int j = 0; j < ctx->p.T; ++j) {
     launch_from_storage(vptr(ctx, j, g.N), ctx->stage, 3 * (int64_t)g.N, ctx->stream, ctx->st);
     int rc = copy_out(ctx, dst + (size_t)j * 3 * g.N, ctx->stage, (size_t)3 * g.N * sizeof(float));
@@ -798,7 +819,13 @@ int lddmm_set_velocity(lddmm_ctx* ctx, const float* src) {
   const Grid& g = ctx->levels[ctx->cur].g;
   const int64_t n = (int64_t)ctx->p.T * 3 * g.N;
   int rc;
-  if (ctx->st == 0) {
+  if (is_local_ptr(src)) {
+    // stored and checked in one pass
+    CK(cudaMemsetAsync(ctx->flag, 0, sizeof(int), ctx->stream));
+    launch_store_checked(src, ctx->v, n, ctx->flag, ctx->stream, ctx->st);
+    CK(cudaGetLastError());
+    if ((rc = read_flag(ctx, "velocity"))) return rc;
+  } else if (ctx->st == 0) {
     CK(cudaMemcpyAsync(ctx->v, src, n * sizeof(float), cudaMemcpyDefault, ctx->stream));
     if ((rc = check_finite(ctx, ctx->v, n, "velocity"))) return rc;
   } else {
