@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <thread>
@@ -131,19 +132,26 @@ bool is_local_ptr(const void* p) {
   return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev);
 }
 
-int wait_stream(lddmm_ctx* ctx) {
-  const double limit = ctx->p.timeout_s > 0 ? ctx->p.timeout_s : 600.0;
+// Bounded host wait.  The first two milliseconds poll without sleeping (a sleep of 5 us takes the
+// kernel's timer slack, some 55 us, on top: as long as a small call's work).
+template <typename Fail>
+int wait_on(cudaStream_t s, double limit, Fail failed) {
   const auto t0 = std::chrono::steady_clock::now();
   for (;;) {
-    cudaError_t e = cudaStreamQuery(ctx->stream);
+    cudaError_t e = cudaStreamQuery(s);
     if (e == cudaSuccess) return LDDMM_OK;
     if (e != cudaErrorNotReady)
-      return fail(ctx, LDDMM_ERR_CUDA, std::string("stream: ") + cudaGetErrorString(e));
+      return failed(LDDMM_ERR_CUDA, std::string("stream: ") + cudaGetErrorString(e));
     const double el =
         std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-    if (el > limit) return fail(ctx, LDDMM_ERR_TIMEOUT, "timed out waiting for the GPU stream");
-    std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 5 : 200));
+    if (el > limit) return failed(LDDMM_ERR_TIMEOUT, "timed out waiting for the GPU stream");
+    if (el > 2e-3) std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 5 : 200));
   }
+}
+
+int wait_stream(lddmm_ctx* ctx) {
+  return wait_on(ctx->stream, ctx->p.timeout_s > 0 ? ctx->p.timeout_s : 600.0,
+                 [&](int code, const std::string& msg) { return fail(ctx, code, msg); });
 }
 
 void prof_mark(void* user, int kid, int phase) {
@@ -1036,17 +1044,46 @@ int lddmm_landmark_error(lddmm_ctx* ctx, const float* xk, const float* yk, int n
 
 namespace {
 // Bounded wait for calls without a context.
-int wait_plain(cudaStream_t s, double limit = 600.0) {
-  const auto t0 = std::chrono::steady_clock::now();
-  for (;;) {
-    cudaError_t e = cudaStreamQuery(s);
-    if (e == cudaSuccess) return LDDMM_OK;
-    if (e != cudaErrorNotReady)
-      return fail(nullptr, LDDMM_ERR_CUDA, std::string("stream: ") + cudaGetErrorString(e));
-    const double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-    if (el > limit) return fail(nullptr, LDDMM_ERR_TIMEOUT, "timed out waiting for the GPU stream");
-    std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 5 : 200));
+int wait_plain(cudaStream_t s) {
+  return wait_on(s, 600.0, [](int code, const std::string& msg) { return fail(nullptr, code, msg); });
+}
+
+// Scratch of the calls without a context: stream-ordered, from a pool of the library's own (one per
+// device; safe with any number of threads and streams).  The pool keeps at most 32 MB when idle,
+// and gives that back when a context is destroyed.  (cudaMalloc and cudaFree, which waits for the
+// whole device, took 150 us a call.)
+constexpr int kPools = 64;
+std::mutex g_pool_lock;
+cudaMemPool_t g_pools[kPools] = {};
+
+cudaMemPool_t scratch_pool() {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kPools) return nullptr;
+  std::lock_guard<std::mutex> hold(g_pool_lock);
+  if (!g_pools[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) return nullptr;
+    cuuint64_t keep = 32ull << 20;
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    g_pools[dev] = pool;
   }
+  return g_pools[dev];
+}
+
+void trim_scratch_pools() {
+  std::lock_guard<std::mutex> hold(g_pool_lock);
+  for (cudaMemPool_t p : g_pools)
+    if (p) cudaMemPoolTrimTo(p, 0);
+}
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s) {
+  cudaMemPool_t pool = scratch_pool();
+  if (!pool) return cudaErrorMemoryAllocation;
+  return cudaMallocFromPoolAsync(p, bytes, pool, s);
 }
 }  // namespace
 
@@ -1060,7 +1097,7 @@ int lddmm_histogram_match(const float* I0, const float* M0, const float* I1, con
     if (!is_device_ptr(p)) return fail(nullptr, LDDMM_ERR_INVALID_ARG, "device memory expected");
   cudaStream_t s = (cudaStream_t)stream;
   void* scr = nullptr;
-  if (cudaMalloc(&scr, match_scratch_bytes(bins)) != cudaSuccess) {
+  if (scratch_alloc(&scr, match_scratch_bytes(bins), s) != cudaSuccess) {
     cudaGetLastError();
     return fail(nullptr, LDDMM_ERR_OOM, "device allocation failed");
   }
@@ -1070,7 +1107,7 @@ int lddmm_histogram_match(const float* I0, const float* M0, const float* I1, con
   int rc = e == cudaSuccess ? wait_plain(s) : fail(nullptr, LDDMM_ERR_CUDA, cudaGetErrorString(e));
   if (rc == LDDMM_OK && (cnt[2] == 0 || cnt[6] == 0))
     rc = fail(nullptr, LDDMM_ERR_INVALID_ARG, "a mask is empty");
-  cudaFree(scr);
+  cudaFreeAsync(scr, s);
   return rc;
 }
 
@@ -1084,7 +1121,7 @@ int lddmm_mask_morphology(const float* I, int nx, int ny, int nz, float threshol
   cudaStream_t s = (cudaStream_t)stream;
   const int64_t words = mask_bits_words(nx, ny, nz);
   uint32_t* bits = nullptr;
-  if (cudaMalloc((void**)&bits, (size_t)(2 * words) * sizeof(uint32_t)) != cudaSuccess) {
+  if (scratch_alloc((void**)&bits, (size_t)(2 * words) * sizeof(uint32_t), s) != cudaSuccess) {
     cudaGetLastError();
     return fail(nullptr, LDDMM_ERR_OOM, "device allocation failed");
   }
@@ -1101,7 +1138,7 @@ int lddmm_mask_morphology(const float* I, int nx, int ny, int nz, float threshol
   }
   if (e == cudaSuccess) e = unpack_bits(nx, ny, nz, m, out, s);
   const int rc = e == cudaSuccess ? wait_plain(s) : fail(nullptr, LDDMM_ERR_CUDA, cudaGetErrorString(e));
-  cudaFree(bits);
+  cudaFreeAsync(bits, s);
   return rc;
 }
 
@@ -1268,6 +1305,7 @@ void lddmm_destroy(lddmm_ctx* ctx) {
   for (cudaEvent_t e : ctx->prof_ev) cudaEventDestroy(e);
   release(ctx);
   delete ctx;
+  trim_scratch_pools();
 }
 
 }  // extern "C"
