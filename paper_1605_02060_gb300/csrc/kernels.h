@@ -60,7 +60,7 @@ void launch_fwd_flow(const Grid& g, const void* vj, const float* u_cur, float* u
 void launch_fwd_fused(const Grid& g, const void* vj, const float* u_cur, float* u_next,
                       float dtx, float dty, float dtz, const void* I0, const float* J1j,
                       const float* Wj, float* b, float c, float ihx, float ihy, float ihz,
-                      int bsplit, int px, cudaStream_t s, int st, int rk = 0);
+                      int bsplit, int px, int py, cudaStream_t s, int st, int rk = 0);
 // J0_T = I0 o (id + u) and E_data = sum M (J0_T - I1)^2 into acc, from the planar map u = u_T.
 void launch_j0_edata(const Grid& g, const float* u, const void* I0, const void* I1,
                      const void* M, float* J0T, Acc* acc, cudaStream_t s, int st);
@@ -184,12 +184,10 @@ cudaError_t apply_K(const KPlan& kp, int mode, const float* in, float* out, floa
 // Output addressing of a pre-split pass: line l = (a D + b) E + e is written at column n to
 // element (a F + b) P + e + n G, as bf16 hi/lo planes `plane` elements apart (KS_OUT_SPLIT), as
 // fp32 (KS_OUT_F32), or as the update out <- out - eps (2 out - C) of fp32 rows (KS_OUT_UPD) or
-// of bf16 rows (KS_OUT_UPD_BF16, arithmetic in FP32, one rounding);
-// sym: scale by the K symbol of the z-forward product.
+// of bf16 rows (KS_OUT_UPD_BF16, arithmetic in FP32, one rounding).
 enum { KS_OUT_SPLIT = 0, KS_OUT_F32 = 1, KS_OUT_UPD = 2, KS_OUT_UPD_BF16 = 3 };
 struct KsOut {
   int kind;
-  int sym;
   void* out;
   long long plane;
   long long D, E, F, P, G;
@@ -197,15 +195,16 @@ struct KsOut {
 // cuTensorMapEncodeTiled from the driver, as void* (nullptr when unavailable).
 void* tma_encode_fn();
 // The pre-split path (all six products on k_dft_ks).  Row pitch of a split line (elements),
-// support test, and the floats a buffer needs for any intermediate field of ncomp components.
+// the sizes it takes, whether it applies, and the floats a buffer needs for any intermediate field of ncomp components.
 int ks_pitch(int L);
+bool ks_shape(int nx, int ny, int nz);
 bool ks_supported(const KPlan& kp);
 long long ks_field_floats(int nx, int ny, int nz, int ncomp);
 cudaError_t ks_axis_pass(const KPlan& kp, int axis, bool inverse, int split, const void* in,
                          long long nlines, const KsOut& o, float eps, cudaStream_t s,
                          bool zz = false);
 // True when apply_K(kp, mode, ..., ncomp, cap) takes the pre-split path; its input may then be
-// given already split (in_split): bf16 hi/lo planes [ncomp][nz][ny][ks_pitch(nx)].
+// given already split (in_split): bf16 hi/lo planes [ncomp][nz][ks_pitch(ny)][ks_pitch(nx)].
 bool ks_path(const KPlan& kp, int mode, int ncomp, long long cap);
 // The pre-split K of `in` (3 components, on the pre-split path only) with the update fused into
 // its last product for a velocity stored in bf16: v <- bf16(v - eps (2 v - K in)), the

@@ -295,66 +295,59 @@ static cudaError_t apply_K_fp32(const KPlan& kp, const float* in, float* out, fl
 }
 
 // Tensor-core K over pre-split intermediate fields.  Every pass reads its input with the
-// transformed axis contiguous and writes its output in the next pass's line order:
-//   x fwd:  [c][z][y][x]  (split, x rows, pitch Px)  -> [c][x'][Pz][y] (split, y rows, pitch Py)
-//   y fwd:                                            -> [c][x'][y'][z] (split, z rows, pitch Pz)
-//   z fwd + symbol:                                   -> [c][x'][y'][z'] (split, same order)
-//   z inv:                                            -> [c][z][x'][y'] (split, y rows, pitch Py)
-//   y inv:                                            -> [c][z][y][x']  (split, x rows, pitch Px)
-//   x inv:                                            -> fp32 [c][z][y][x], or the update of v
+// transformed axis contiguous and writes its output in the next pass's line order (Xp, Yp, Zp: the
+// sizes rounded up to 8, the pitches of x, y and z rows):
+//   x fwd:  [c][z][Yp][x] (split, x rows)  -> [c][x'][Zp][y]   (split, y rows)
+//   y fwd:                                  -> [c][x'][Yp][z]   (split, z rows)
+//   z fwd + symbol + z inv (one pass):      -> [c][z][Xp][y']   (split, y rows)
+//   y inv:                                  -> [c][z][y][x']    (split, x rows)
+//   x inv:                                  -> fp32 [c][z][y][x], or the update of v
 // The buffers alternate between work and out (in may alias out).  A plain fp32 input is first
 // split into work; without the update the result then lands in work and is copied to out.
-// The x forward output holds Pz (z rounded up to 8) planes per x' so that the y forward pass
-// runs over Pz lines per output row: its 8-line output pieces then start 16-byte aligned (the
-// staged epilogue).  Lines z >= nz are never written by the x pass and read whatever the buffer
-// holds; the y pass stores their results into the pitch padding of the z rows, which no later
-// pass reads (rows of a product are independent).
+// Each pass runs over whole groups of 8 lines in its output rows (Yp, Zp, Yp and Xp lines a row), so
+// that its 8-line output pieces start 16-byte aligned and stay within a row at any grid size.  The
+// lines past an axis's end are written by no pass and read whatever the buffer holds; the rows of
+// a product are independent, and their results land in the pitch padding of the next field, which
+// its pass does not read (the TMA maps end at the line length).
 static cudaError_t apply_K_ks(const KPlan& kp, int split, const float* in, float* out,
                               float* work, int ncomp, cudaStream_t s, const Hook& hook,
                               void* v_upd, float eps, bool in_split, int upd_kind = KS_OUT_UPD) {
   const long long X = kp.nx, Y = kp.ny, Z = kp.nz, C = ncomp;
-  const long long Px = ks_pitch(kp.nx), Py = ks_pitch(kp.ny), Pz = ks_pitch(kp.nz);
+  const long long Xp = ks_pitch(kp.nx), Yp = ks_pitch(kp.ny), Zp = ks_pitch(kp.nz);
   cudaError_t e;
   float* bA = work;   // receives the x forward product
   float* bB = out;
   const void* src = in;
   if (!in_split) {
-    const KsOut o0{KS_OUT_SPLIT, 0, work, C * Z * Y * Px, 1, 1, 1, Px, 1};
+    const KsOut o0{KS_OUT_SPLIT, work, C * Z * Yp * Xp, Y, 1, Yp, Xp, 1};
     if ((e = ks_split_rows(in, C * Z * Y, kp.nx, split, o0, s)) != cudaSuccess) return e;
     src = work;
     bA = out;
     bB = work;
   }
-  // z forward, symbol and z inverse run as one fused pass when the z inverse output rows (y
-  // lines) hold a multiple of 8 lines; its output then lands where the z inverse pass puts it
-  const bool zz = Y % 8 == 0;
   struct Pass2 {
     int kid, axis;
     bool inv, zz;
     long long nlines;
     KsOut o;
   };
-  const Pass2 ps[5] = {
-      {KID_KX_FWD, 0, false, false, C * Z * Y, {KS_OUT_SPLIT, 0, bA, C * X * Pz * Py, Z, Y, X * Pz, Py, Pz * Py}},
-      {KID_KY_FWD, 1, false, false, C * X * Pz, {KS_OUT_SPLIT, 0, bB, C * X * Y * Pz, 1, Pz, Y, Pz, Pz}},
-      {KID_KZ_SYM, 2, false, false, C * X * Y, {KS_OUT_SPLIT, 1, bA, C * X * Y * Pz, 1, 1, 1, Pz, 1}},
-      {zz ? KID_KZ_FUSED : KID_KZ_INV, 2, true, zz, C * X * Y,
-       {KS_OUT_SPLIT, 0, zz ? bA : bB, C * Z * X * Py, X, Y, Z * X, Py, X * Py}},
-      {KID_KY_INV, 1, true, false, C * Z * X, {KS_OUT_SPLIT, 0, zz ? bB : bA, C * Z * Y * Px, 1, X, Y, Px, Px}}};
-  for (int p = 0; p < 5; ++p) {
-    if (zz && p == 2) continue;
-    hook(ps[p].kid, 0);
-    e = ks_axis_pass(kp, ps[p].axis, ps[p].inv, split, src, ps[p].nlines, ps[p].o, 0.f, s,
-                     ps[p].zz);
-    hook(ps[p].kid, 1);
+  const Pass2 ps[4] = {
+      {KID_KX_FWD, 0, false, false, C * Z * Yp, {KS_OUT_SPLIT, bA, C * X * Zp * Yp, Z, Yp, X * Zp, Yp, Zp * Yp}},
+      {KID_KY_FWD, 1, false, false, C * X * Zp, {KS_OUT_SPLIT, bB, C * X * Yp * Zp, 1, Zp, Yp, Zp, Zp}},
+      {KID_KZ_FUSED, 2, true, true, C * X * Yp, {KS_OUT_SPLIT, bA, C * Z * Xp * Yp, X, Yp, Z * Xp, Yp, Xp * Yp}},
+      {KID_KY_INV, 1, true, false, C * Z * Xp, {KS_OUT_SPLIT, bB, C * Z * Y * Xp, 1, Xp, Y, Xp, Xp}}};
+  for (const Pass2& p : ps) {
+    hook(p.kid, 0);
+    e = ks_axis_pass(kp, p.axis, p.inv, split, src, p.nlines, p.o, 0.f, s, p.zz);
+    hook(p.kid, 1);
     if (e != cudaSuccess) return e;
-    src = ps[p].o.out;
+    src = p.o.out;
   }
   // x inverse: from the last output into v_upd (update) or fp32 rows in the other buffer
-  void* dst = v_upd ? v_upd : (void*)(src == bA ? bB : bA);
-  const KsOut o6{v_upd ? upd_kind : KS_OUT_F32, 0, dst, 0, 1, 1, 1, X, 1};
+  void* dst = v_upd ? v_upd : (void*)bA;
+  const KsOut o5{v_upd ? upd_kind : KS_OUT_F32, dst, 0, 1, 1, 1, X, 1};
   hook(KID_KX_INV, 0);
-  e = ks_axis_pass(kp, 0, true, split, src, C * Z * Y, o6, eps, s);
+  e = ks_axis_pass(kp, 0, true, split, src, C * Z * Y, o5, eps, s);
   hook(KID_KX_INV, 1);
   if (e != cudaSuccess) return e;
   if (!v_upd && dst != out)

@@ -353,14 +353,15 @@ __device__ __forceinline__ float J0_at(const Grid& g, const float* __restrict__ 
 
 // b_j at voxel (x, y, z) = idx, as fp32 components (bsplit == 0), or split into bf16 hi/lo
 // planes for the pre-split K (bsplit 1: hi plane only, 2: hi and lo): element
-// ((comp Z + z) Y + y) px + x of each plane, planes 3 Z Y px elements apart.
+// ((comp Z + z) py + y) px + x of each plane, planes 3 Z py px elements apart (px, py: X, Y rounded
+// up as K's first pass wants them).
 template <bool Q, typename ST>
 __device__ __forceinline__ void fwd_terms_at(const Grid& g, const float* __restrict__ uc,
                                              const ST* __restrict__ I0,
                                              const float* __restrict__ J1j,
                                              const float* __restrict__ Wj, float* __restrict__ b,
                                              float c, float ihx, float ihy, float ihz, int bsplit,
-                                             int px, int x, int y, int z, int idx) {
+                                             int px, int py, int x, int y, int z, int idx) {
   const float w = Wj[idx];
   float bx = 0.f, by = 0.f, bz = 0.f;
   if (w != 0.0f) {
@@ -399,8 +400,8 @@ __device__ __forceinline__ void fwd_terms_at(const Grid& g, const float* __restr
   }
   if (bsplit) {
     __nv_bfloat16* h = reinterpret_cast<__nv_bfloat16*>(b);
-    const int64_t cs = (int64_t)g.nz * g.ny * px;
-    const int64_t o = ((int64_t)z * g.ny + y) * px + x;
+    const int64_t cs = (int64_t)g.nz * py * px;
+    const int64_t o = ((int64_t)z * py + y) * px + x;
     const float bc[3] = {bx, by, bz};
 #pragma unroll
     for (int e = 0; e < 3; ++e) {
@@ -426,7 +427,7 @@ __global__ void __launch_bounds__(256) k_fwd_fused_march(
     Grid g, const ST* __restrict__ vj, const float* __restrict__ uc, float* __restrict__ un,
     float dtx, float dty, float dtz, const ST* __restrict__ I0, const float* __restrict__ J1j,
     const float* __restrict__ Wj, float* __restrict__ b, float c, float ihx, float ihy, float ihz,
-    int bsplit, int px) {
+    int bsplit, int px, int py) {
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
   if (x < g.nx && y < g.ny) {
     const int z0 = blockIdx.z * ZC, z1 = min(z0 + ZC, g.nz);
@@ -456,7 +457,7 @@ __global__ void __launch_bounds__(256) k_fwd_fused_march(
         oy += r.y;
         oz += r.z;
       }
-      fwd_terms_at<Q>(g, uc, I0, J1j, Wj, b, c, ihx, ihy, ihz, bsplit, px, x, y, z, idx);
+      fwd_terms_at<Q>(g, uc, I0, J1j, Wj, b, c, ihx, ihy, ihz, bsplit, px, py, x, y, z, idx);
       MapL<Q>::put(un, g.N, idx, ox, oy, oz);
       a0 = n0;
       a1 = n1;
@@ -553,12 +554,12 @@ __global__ void __launch_bounds__(256) k_fwd_last_march(Grid g, const ST* __rest
 void launch_fwd_fused(const Grid& g, const void* vj, const float* u_cur, float* u_next,
                       float dtx, float dty, float dtz, const void* I0, const float* J1j,
                       const float* Wj, float* b, float c, float ihx, float ihy, float ihz,
-                      int bsplit, int px, cudaStream_t s, int st, int rk) {
+                      int bsplit, int px, int py, cudaStream_t s, int st, int rk) {
   const dim3 grid((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + kFlowZ - 1) / kFlowZ);
 #define FWD_FUSED(ST_, RK_)                                                                    \
   k_fwd_fused_march<ST_, kFlowZ, RK_, false><<<grid, kBlock3d, 0, s>>>(                       \
       g, (const ST_*)vj, u_cur, u_next, dtx, dty, dtz, (const ST_*)I0, J1j, Wj, b, c, ihx, ihy, \
-      ihz, bsplit, px)
+      ihz, bsplit, px, py)
   if (st) {
     if (rk) FWD_FUSED(__nv_bfloat16, true); else FWD_FUSED(__nv_bfloat16, false);
   } else {

@@ -18,13 +18,9 @@
 //   warps 2-9   epilogue: tcgen05.ld of 16/32 columns (warp w reads TMEM lanes 32(w%4)..+31, the
 //               two warps of a lane quadrant split the columns), optional K symbol or the
 //               gradient-descent update, stores;
-//   warps 10-13 x axis longer than 256: the output columns 256.. in FP32 on the CUDA cores,
-//               one line per thread, read from the same A stages (hi + lo) as the MMA; an A
-//               stage is free once the MMA has committed and these 128 threads have arrived.
-//               Passes without such columns whose outputs are staged give these warps to
-//               the epilogue (three warps per TMEM lane quadrant instead of two): the epilogue's
-//               element-wise conversions and stores, not the tensor cores, set those passes'
-//               pace, and more warps hide more of their latency.
+//   warps 10-13 where shared memory allows, a third column range of the epilogue: its
+//               element-wise conversions and stores, not the tensor cores, set the pace of those
+//               passes, and more warps hide more of their latency.
 // Every wait is bounded and observes a CTA-wide abort flag; on abort the kernel drains its
 // copies and MMAs, frees TMEM and reports through *err.
 #include <cuda.h>
@@ -64,11 +60,11 @@ struct KsArgs {
   int nparts;          // epilogue column ranges (four warps each, one per TMEM lane quadrant)
   KsOut o;             // output addressing
   float eps;           // KS_OUT_UPD: step size
-  const float* lx;     // symbol (o.sym): lambda per x, y, z frequency
+  const float* lx;     // symbol (zz): lambda per x, y, z frequency
   const float* ly;
   const float* lz;
   float alpha, gamma;
-  int X, Y;            // symbol: line l = (c X + x) Y + y
+  int X, Y;            // zz: line l = (c X + x) Y + y, Y rounded up to 8
   int* err;
   uint32_t poll;       // probes per pipeline wait before the CTA aborts
   int zz;              // the fused z pass: forward product, symbol, inverse product
@@ -81,16 +77,11 @@ __host__ __device__ inline int ks_bbytes(int split, int Nc) { return (split ? 2 
 constexpr int KS_SROW = 17;
 // transposed split outputs: per column range (2 or 3 of them), a tile of 16 columns x 128 lines
 // of bf16 hi and lo, through which the four lane-quadrant warps of the range store runs of 128
-// consecutive lines
+// consecutive lines (their rows hold a multiple of 8 lines, so 8-line pieces are aligned)
 constexpr int KS_CTILE = 2 * 16 * 128 * 2;
-// (only when the output rows hold a multiple of 8 lines, so that the 8-line pieces are aligned:
-// with other row lengths the per-lane stores measured faster)
-__host__ __device__ inline bool ks_staged(const KsArgs& a) {
-  return a.o.G != 1 && a.o.kind == KS_OUT_SPLIT && a.o.E % 8 == 0;
-}
 __host__ __device__ inline int ks_sbytes(const KsArgs& a) {
   if (a.o.G == 1) return 4 * a.nparts * 32 * KS_SROW * 4;   // row outputs: a tile per warp
-  return ks_staged(a) ? a.nparts * KS_CTILE : 0;
+  return a.nparts * KS_CTILE;
 }
 __host__ __device__ inline int ks_smem(const KsArgs& a) {
   return 1024 + a.AS * ks_abytes(a.split) + (a.bres ? a.nkb : a.BS) * ks_bbytes(a.split, a.Nc) +
@@ -123,16 +114,6 @@ __device__ __forceinline__ void split1(float x, uint16_t& h, uint16_t& l) {
   l = bf16_bits(__float2bfloat16_rn(x - __bfloat162float(hb)));
 }
 
-// 8 bf16 (one 16-byte word, element 0 in the low half of the first word) added to x[0..7]
-__device__ __forceinline__ void add_bf8(uint4 w, float* x) {
-  const uint32_t u[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    x[2 * j] += __uint_as_float(u[j] << 16);
-    x[2 * j + 1] += __uint_as_float(u[j] & 0xffff0000u);
-  }
-}
-
 // Bulk prefetch of [p, p + bytes) into L2 (16-byte aligned, bytes a multiple of 16).
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
@@ -148,33 +129,6 @@ __device__ __forceinline__ void prefetch_l2_inner(const void* p, uint32_t bytes)
 __device__ __forceinline__ long long out_base(const KsOut& o, long long l) {
   const long long e = l % o.E, t = l / o.E;
   return (t / o.D * o.F + t % o.D) * o.P + e;
-}
-
-// Store cnt (<= NMAX) consecutive output columns n0.. of one line, one element at a time
-// (transposed outputs whose runs are not vector aligned, and the FP32 tail columns), split into
-// bf16 hi/lo or plain fp32 (the update's tail columns are stored by the tail threads).  The loops
-// are unrolled over NMAX so that vc stays in registers.
-template <int NMAX>
-__device__ __forceinline__ void store_scalar(const KsOut& o, int split, long long base, int n0,
-                                             const float* vc, int cnt) {
-  if (o.kind == KS_OUT_SPLIT) {
-    uint16_t* oh = reinterpret_cast<uint16_t*>(o.out);
-#pragma unroll
-    for (int j = 0; j < NMAX; ++j) {
-      if (j < cnt) {
-        uint16_t h, lo;
-        split1(vc[j], h, lo);
-        const long long off = base + (long long)(n0 + j) * o.G;
-        oh[off] = h;
-        if (split) oh[o.plane + off] = lo;
-      }
-    }
-  } else {
-    float* of = reinterpret_cast<float*>(o.out);
-#pragma unroll
-    for (int j = 0; j < NMAX; ++j)
-      if (j < cnt) of[base + (long long)(n0 + j) * o.G] = vc[j];
-  }
 }
 
 __host__ __device__ inline bool is_upd_host(int kind) {
@@ -197,58 +151,55 @@ __device__ __forceinline__ uint32_t pack_bf16x2(uint16_t a, uint16_t b) {
 }
 
 // Row-wise outputs (o.G == 1, line l at l * o.P): the 16 columns n0.. of the warp's 32 lines
-// line0.. (lane = line on entry) leave through the warp's shared-memory tile, so that a lane
-// writes 8 consecutive bf16 columns (split, 16-byte stores) or 4 consecutive fp32 columns
-// (plain or the update, 16-byte loads and stores) of one line, and a store instruction covers
-// 16 or 8 lines.  (Transposed outputs, consecutive lines = consecutive positions, are already
-// coalesced across the lanes and are stored element by element from registers.)
+// line0.. (lane = line on entry) leave through the warp's shared-memory tile.  VEC (rows start on a
+// 4-element boundary: X a multiple of 4): a lane reads and writes 4 consecutive columns of one
+// line, 8 lines per instruction.  Else one column, 2 lines (two runs of 64 bytes) per instruction.
 // The old v that the update combines with the 16 columns n0.. of the warp's 32 lines, in the
-// lane order store_rows uses (4 consecutive fp32 columns of one line per 16-byte load).
+// lane order store_rows uses: old[4 it + k] (VEC) or old[it].
+template <bool VEC>
 __device__ __forceinline__ void load_old_rows(const KsOut& o, int lane, long long line0,
-                                              long long nlines, int n0, int ncols, float4* old) {
+                                              long long nlines, int n0, int ncols, float* old) {
   const float* of = reinterpret_cast<const float*>(o.out);
   const uint16_t* ob = reinterpret_cast<const uint16_t*>(o.out);
+  if constexpr (VEC) {
 #pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    const int idx = it * 32 + lane, r = idx >> 2, c4 = (idx & 3) * 4;
-    const long long l = line0 + r;
-    if (l < nlines && n0 + c4 + 4 <= ncols) {
-      if (o.kind == KS_OUT_UPD_BF16)
-        old[it] = bf4_to_f4(*reinterpret_cast<const uint2*>(ob + l * o.P + n0 + c4));
-      else
-        old[it] = *reinterpret_cast<const float4*>(of + l * o.P + n0 + c4);
+    for (int it = 0; it < 4; ++it) {
+      const int idx = it * 32 + lane, r = idx >> 2, c4 = (idx & 3) * 4;
+      const long long l = line0 + r;
+      if (l < nlines && n0 + c4 + 4 <= ncols) {
+        float4 q;
+        if (o.kind == KS_OUT_UPD_BF16)
+          q = bf4_to_f4(*reinterpret_cast<const uint2*>(ob + l * o.P + n0 + c4));
+        else
+          q = *reinterpret_cast<const float4*>(of + l * o.P + n0 + c4);
+        old[4 * it] = q.x;
+        old[4 * it + 1] = q.y;
+        old[4 * it + 2] = q.z;
+        old[4 * it + 3] = q.w;
+      }
+    }
+  } else {
+    const int c = lane & 15;
+#pragma unroll
+    for (int it = 0; it < 16; ++it) {
+      const long long l = line0 + 2 * it + (lane >> 4);
+      if (l < nlines && n0 + c < ncols)
+        old[it] = o.kind == KS_OUT_UPD_BF16 ? __uint_as_float((uint32_t)ob[l * o.P + n0 + c] << 16)
+                                            : of[l * o.P + n0 + c];
     }
   }
 }
 
-__device__ __forceinline__ void store_rows(const KsOut& o, int split, float eps, float* sg,
-                                           int lane, long long line0, long long nlines, int n0,
-                                           int ncols, const float* vc, const float4* old) {
+template <bool VEC>
+__device__ __forceinline__ void store_rows(const KsOut& o, float eps, float* sg, int lane,
+                                           long long line0, long long nlines, int n0, int ncols,
+                                           const float* vc, const float* old) {
 #pragma unroll
   for (int j = 0; j < 16; ++j) sg[lane * KS_SROW + j] = vc[j];
   __syncwarp();
-  if (o.kind == KS_OUT_SPLIT) {
-    uint16_t* oh = reinterpret_cast<uint16_t*>(o.out);
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-      const int idx = it * 32 + lane, r = idx >> 1, c8 = (idx & 1) * 8;
-      const long long l = line0 + r;
-      if (l < nlines && n0 + c8 + 8 <= ncols) {
-        uint16_t h[8], lo[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) split1(sg[r * KS_SROW + c8 + k], h[k], lo[k]);
-        const long long off = l * o.P + n0 + c8;
-        *reinterpret_cast<uint4*>(oh + off) =
-            make_uint4(pack_bf16x2(h[0], h[1]), pack_bf16x2(h[2], h[3]), pack_bf16x2(h[4], h[5]),
-                       pack_bf16x2(h[6], h[7]));
-        if (split)
-          *reinterpret_cast<uint4*>(oh + o.plane + off) =
-              make_uint4(pack_bf16x2(lo[0], lo[1]), pack_bf16x2(lo[2], lo[3]),
-                         pack_bf16x2(lo[4], lo[5]), pack_bf16x2(lo[6], lo[7]));
-      }
-    }
-  } else {
-    float* of = reinterpret_cast<float*>(o.out);
+  float* of = reinterpret_cast<float*>(o.out);
+  uint16_t* ob = reinterpret_cast<uint16_t*>(o.out);
+  if constexpr (VEC) {
 #pragma unroll
     for (int it = 0; it < 4; ++it) {
       const int idx = it * 32 + lane, r = idx >> 2, c4 = (idx & 3) * 4;
@@ -257,15 +208,27 @@ __device__ __forceinline__ void store_rows(const KsOut& o, int split, float eps,
         const float* q = sg + r * KS_SROW + c4;
         float4 w = make_float4(q[0], q[1], q[2], q[3]);
         if (is_upd(o.kind)) {
-          const float4 p = old[it];
-          w = make_float4(p.x - eps * (2.f * p.x - w.x), p.y - eps * (2.f * p.y - w.y),
-                          p.z - eps * (2.f * p.z - w.z), p.w - eps * (2.f * p.w - w.w));
+          const float* p = old + 4 * it;
+          w = make_float4(p[0] - eps * (2.f * p[0] - w.x), p[1] - eps * (2.f * p[1] - w.y),
+                          p[2] - eps * (2.f * p[2] - w.z), p[3] - eps * (2.f * p[3] - w.w));
         }
         if (o.kind == KS_OUT_UPD_BF16)
-          *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(o.out) + l * o.P + n0 + c4) =
-              f4_to_bf4(w);
+          *reinterpret_cast<uint2*>(ob + l * o.P + n0 + c4) = f4_to_bf4(w);
         else
           *reinterpret_cast<float4*>(of + l * o.P + n0 + c4) = w;
+      }
+    }
+  } else {
+    const int c = lane & 15;
+#pragma unroll
+    for (int it = 0; it < 16; ++it) {
+      const int r = 2 * it + (lane >> 4);
+      const long long l = line0 + r;
+      if (l < nlines && n0 + c < ncols) {
+        float w = sg[r * KS_SROW + c];
+        if (is_upd(o.kind)) w = old[it] - eps * (2.f * old[it] - w);
+        if (o.kind == KS_OUT_UPD_BF16) ob[l * o.P + n0 + c] = bf16_bits(__float2bfloat16_rn(w));
+        else of[l * o.P + n0 + c] = w;
       }
     }
   }
@@ -275,13 +238,18 @@ __device__ __forceinline__ void store_rows(const KsOut& o, int split, float eps,
 // Epilogue kinds: each pass is compiled with only its own output path, so that the registers of
 // the other paths do not count against it (the kernel runs at the 128-register limit of 448
 // threads).
-enum { EPI_T_STAGED = 0, EPI_T = 1, EPI_ROWS = 2, EPI_UPD = 3, EPI_ZZ = 4 };
+// threads).  EPI_T transposed split outputs, EPI_ZZ the fused z pass's, EPI_ROWS and EPI_UPD rows
+// that start on a 4-element boundary, EPI_ROWS_1 and EPI_UPD_1 other rows.  EPI_ZZ_RN forms and
+// divides by the symbol with the roundings of k_dft_tc, for the grids (X no multiple of 4) that
+// come from it: with plain bf16 products one FP32 rounding decides bf16 digits, which a
+// registration's iterations carry on.
+enum { EPI_T = 0, EPI_ROWS, EPI_ROWS_1, EPI_UPD, EPI_UPD_1, EPI_ZZ, EPI_ZZ_RN, EPI_COUNT };
 
 __host__ __device__ inline int ks_epi(const KsArgs& a) {
-  if (a.zz) return EPI_ZZ;
-  if (is_upd_host(a.o.kind)) return EPI_UPD;
-  if (a.o.G == 1) return EPI_ROWS;
-  return ks_staged(a) ? EPI_T_STAGED : EPI_T;
+  if (a.zz) return a.X % 4 == 0 ? EPI_ZZ : EPI_ZZ_RN;
+  if (is_upd_host(a.o.kind)) return a.o.P % 4 == 0 ? EPI_UPD : EPI_UPD_1;
+  if (a.o.G == 1) return a.o.P % 4 == 0 ? EPI_ROWS : EPI_ROWS_1;
+  return EPI_T;
 }
 
 template <int EPI>
@@ -290,7 +258,8 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
                                                      const __grid_constant__ CUtensorMap tmB2,
                                                      const __grid_constant__ CUtensorMap tmO,
                                                      KsArgs a) {
-  constexpr bool ZZ = EPI == EPI_ZZ;
+  constexpr bool ZZ = EPI == EPI_ZZ || EPI == EPI_ZZ_RN, UPD = EPI == EPI_UPD || EPI == EPI_UPD_1;
+  constexpr bool VEC = EPI == EPI_UPD || EPI == EPI_ROWS;
   extern __shared__ __align__(1024) uint8_t smem_dyn[];
   __shared__ __align__(8) uint64_t b_afull[KS_MAXS], b_aempty[KS_MAXS], b_bfull[KS_MAXS],
       b_bempty[KS_MAXS];
@@ -562,8 +531,6 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
     auto chunk_at = [&](int k) { return k < ntl ? tb + k : cbeg + (k - ntl); };
     const KsOut& o = a.o;
     const int Lc = min(a.L, a.Nc);                   // valid tensor-core output columns
-    // columns written per line (row-wise split outputs stop at the row pitch)
-    const int ncols = (o.G == 1 && o.kind == KS_OUT_SPLIT) ? min(a.Nc, (int)o.P) : Lc;
     float* sg = stg + (warp - 2) * (32 * KS_SROW);
     for (int i = 0; i < my_tiles; ++i) {
       // the fused z pass drains its one inverse accumulator (columns 256..) every tile
@@ -571,15 +538,11 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
       const uint32_t use = ZZ ? (uint32_t)i : (uint32_t)(i >> 1);
       const long long l = (long long)(blockIdx.x + i * gridDim.x) * 128 + q * 32 + lane;
       const bool valid = l < a.nlines;
-      // output address of (line l, column 0) and the symbol's (x, y) part
-      long long base = 0;
+      // the symbol's (x, y) part; lines run over Y rounded up to 8 (ly is padded that far)
       float sxy = 1.f;
-      if (valid) {
-        base = out_base(o, l);
-        if (o.sym || ZZ) {
-          const int ry = (int)(l % a.Y), rx = (int)((l / a.Y) % a.X);
-          sxy = a.gamma + a.alpha * (a.lx[rx] + a.ly[ry]);
-        }
+      if (ZZ && valid) {
+        const int ry = (int)(l % a.Y), rx = (int)((l / a.Y) % a.X);
+        sxy = EPI == EPI_ZZ_RN ? a.lx[rx] + a.ly[ry] : a.gamma + a.alpha * (a.lx[rx] + a.ly[ry]);
       }
       bool conv_ok = true;
       if constexpr (ZZ) {
@@ -610,10 +573,17 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
               for (int jj = 0; jj < 2; ++jj) {
                 const int j = 2 * j4 + jj;
                 uint16_t h0, l0, h1, l1;
-                const float d0 = fmaf(a.alpha, zl[2 * jj], sxy);
-                const float d1 = fmaf(a.alpha, zl[2 * jj + 1], sxy);
-                split1(__fdividef(vc[2 * j], d0 * d0), h0, l0);
-                split1(__fdividef(vc[2 * j + 1], d1 * d1), h1, l1);
+                if constexpr (EPI == EPI_ZZ_RN) {
+                  const float d0 = fmaf(a.alpha, sxy + zl[2 * jj], a.gamma);
+                  const float d1 = fmaf(a.alpha, sxy + zl[2 * jj + 1], a.gamma);
+                  split1(__fdiv_rn(vc[2 * j], d0 * d0), h0, l0);
+                  split1(__fdiv_rn(vc[2 * j + 1], d1 * d1), h1, l1);
+                } else {
+                  const float d0 = fmaf(a.alpha, zl[2 * jj], sxy);
+                  const float d1 = fmaf(a.alpha, zl[2 * jj + 1], sxy);
+                  split1(__fdividef(vc[2 * j], d0 * d0), h0, l0);
+                  split1(__fdividef(vc[2 * j + 1], d1 * d1), h1, l1);
+                }
                 hw[j] = pack_bf16x2(h0, h1);
                 lw[j] = pack_bf16x2(l0, l1);
               }
@@ -629,7 +599,7 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
       const long long line0 = l - lane;
       // the update reads the old v of this warp's columns: start bringing it into L2 while the
       // tensor cores are still on the tile
-      if (EPI == EPI_UPD && valid && cend * 16 > cbeg * 16) {
+      if (UPD && valid && cend * 16 > cbeg * 16) {
         const int c1 = min(cend * 16, Lc);
         const int es = o.kind == KS_OUT_UPD_BF16 ? 2 : 4;
         if (c1 > cbeg * 16)
@@ -639,12 +609,12 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
       // the update: the old v of the first pair of chunks is requested before the wait for the
       // accumulator, each later pair's just before its TMEM load (pairs never straddle the two
       // products: a part holds 0 or 2 chunks of the second)
-      float4 oldv[8];
-      if (EPI == EPI_UPD && cnt > 0) {
-        load_old_rows(o, lane, line0, a.nlines, chunk_at(0) * 16, ncols, oldv);
-        if (cnt > 1) load_old_rows(o, lane, line0, a.nlines, chunk_at(1) * 16, ncols, oldv + 4);
+      float oldv[32];
+      if (UPD && cnt > 0) {
+        load_old_rows<VEC>(o, lane, line0, a.nlines, chunk_at(0) * 16, Lc, oldv);
+        if (cnt > 1) load_old_rows<VEC>(o, lane, line0, a.nlines, chunk_at(1) * 16, Lc, oldv + 16);
       }
-      constexpr bool staged = EPI == EPI_T_STAGED || ZZ;
+      constexpr bool staged = EPI == EPI_T || ZZ;
       int got = (conv_ok && ptx::mbar_wait_or_abort(ptx::smem_u32(&b_tfull[ab]), use & 1, abort, a.poll)) ? 1 : 0;
       if constexpr (staged) {
         // the four warps of a column range meet at named barriers below: they give up together
@@ -709,13 +679,6 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
         const int tp = q * 32 + lane, grp = tp & 15;
         const long long lg0 = line0 - q * 32 + grp * 8;     // first line of this thread's group
         const long long gb = lg0 < a.nlines ? out_base(o, lg0) : 0;
-        // 8 lines in one run: one 16-byte store when 16-byte aligned, else two of 8 bytes.  A
-        // group that crosses the end of an output row (E lines) continues at the next row's
-        // base nb from its line k on.
-        const bool run = lg0 + 7 < a.nlines && out_base(o, lg0 + 7) == gb + 7;
-        const int vec = !run ? 0 : ((gb & 7) == 0 ? 2 : ((gb & 3) == 0 ? 1 : 0));
-        const int kcut = run ? 8 : (int)min((long long)8, o.E - lg0 % o.E);
-        const long long nb = (!run && lg0 + kcut < a.nlines) ? out_base(o, lg0 + kcut) : 0;
         const int np = a.split ? 2 : 1;
         for (int k = 0; k < cnt; ++k) {
           const int c = chunk_at(k);
@@ -739,24 +702,10 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
             if (pl < np && n < Lc) {
               uint16_t* oh = reinterpret_cast<uint16_t*>(o.out) + (pl ? o.plane : 0);
               const uint16_t* src = tile + (pl * 16 + j) * 128 + grp * 8;
-              if (vec == 2) {
+              // rows hold whole, aligned groups of 8 lines
+              if (lg0 < a.nlines)
                 *reinterpret_cast<uint4*>(oh + gb + (long long)n * o.G) =
                     *reinterpret_cast<const uint4*>(src);
-              } else if (vec == 1) {
-                const uint4 w = *reinterpret_cast<const uint4*>(src);
-                uint2* d = reinterpret_cast<uint2*>(oh + gb + (long long)n * o.G);
-                d[0] = make_uint2(w.x, w.y);
-                d[1] = make_uint2(w.z, w.w);
-              } else {
-                for (int e = 0; e < 8; ++e) {
-                  if (lg0 + e < a.nlines) {
-                    // rows shorter than 8 lines: a group can span several of them
-                    const long long off = o.E < 8 ? out_base(o, lg0 + e)
-                                                  : (e < kcut ? gb + e : nb + (e - kcut));
-                    oh[off + (long long)n * o.G] = src[e];
-                  }
-                }
-              }
             }
           }
           asm volatile("bar.sync %0, 128;" ::"r"(2 + part) : "memory");
@@ -765,9 +714,9 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
       for (int k = 0; k < cnt; k += 2) {
         const int cp = chunk_at(k);
         const int npair = (k + 1 < cnt && k + 1 != ntl) ? 2 : 1;
-        if (EPI == EPI_UPD && k > 0) {
-          load_old_rows(o, lane, line0, a.nlines, cp * 16, ncols, oldv);
-          if (npair == 2) load_old_rows(o, lane, line0, a.nlines, cp * 16 + 16, ncols, oldv + 4);
+        if (UPD && k > 0) {
+          load_old_rows<VEC>(o, lane, line0, a.nlines, cp * 16, Lc, oldv);
+          if (npair == 2) load_old_rows<VEC>(o, lane, line0, a.nlines, cp * 16 + 16, Lc, oldv + 16);
         }
         float v[32];
         if (npair == 2) ptx::tmem_ld32(tcol(cp), v);
@@ -781,17 +730,7 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
           if (u2 >= npair) break;
           const int n0 = (cp + u2) * 16;
           float* vc = v + 16 * u2;
-          if (o.sym && valid) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              const float den = fmaf(a.alpha, __ldg(a.lz + min(n0 + j, a.L - 1)), sxy);
-              vc[j] = __fdividef(vc[j], den * den);
-            }
-          }
-          if constexpr (EPI == EPI_ROWS || EPI == EPI_UPD)   // whole warp
-            store_rows(o, a.split, a.eps, sg, lane, line0, a.nlines, n0, ncols, vc, oldv + 4 * u2);
-          else if (valid)
-            store_scalar<16>(o, a.split, base, n0, vc, min(16, Lc - n0));
+          store_rows<VEC>(o, a.eps, sg, lane, line0, a.nlines, n0, Lc, vc, oldv + 16 * u2);
         }
       }
       }
@@ -855,19 +794,20 @@ void* tma_encode_fn() { return reinterpret_cast<void*>(encode_fn()); }
 
 int ks_pitch(int L) { return (L + 7) / 8 * 8; }
 
+// Any grid up to 264 x 256 x 256 (the widest tables that fit beside two A stages).  At 141x97x109
+// one K of three components takes 104 us here, 285 us on k_dft_tc, which splits fp32 lines by all
+// threads before each product.
+bool ks_shape(int nx, int ny, int nz) { return nx <= 264 && ny <= 256 && nz <= 256; }
+
 bool ks_supported(const KPlan& kp) {
   if (!tma_encode_fn() || !kp.ks[0][0] || !kp.ks[1][0] || !kp.ks[2][0]) return false;
-  return kp.nx % 4 == 0 && kp.nx <= 264 && kp.ny <= 256 && kp.nz <= 256;
+  return ks_shape(kp.nx, kp.ny, kp.nz);
 }
 
 long long ks_field_floats(int nx, int ny, int nz, int ncomp) {
-  const long long X = nx, Y = ny, Z = nz;
-  const long long px = ks_pitch(nx), py = ks_pitch(ny), pz = ks_pitch(nz);
-  long long m = X * Y * Z;                      // fp32 rows
-  if (Z * Y * px > m) m = Z * Y * px;           // split [c][z][y][x] (x rows)
-  if (X * pz * py > m) m = X * pz * py;         // [c][x'][Pz][y] and [c][z][x'][y']
-  if (X * Y * pz > m) m = X * Y * pz;           // [c][x'][y'][z]
-  return m * ncomp;                             // two bf16 planes = one float per value
+  const long long X = nx, Z = nz, xp = ks_pitch(nx), yp = ks_pitch(ny), zp = ks_pitch(nz);
+  const long long a = Z * yp * xp, b = X * zp * yp;   // x and y rows; y and z rows
+  return (a > b ? a : b) * ncomp;                     // two bf16 planes = one float per value
 }
 
 cudaError_t ks_split_rows(const float* in, long long nrows, int L, int split, const KsOut& o,
@@ -898,16 +838,20 @@ cudaError_t ks_axis_pass(const KPlan& kp, int axis, bool inverse, int split, con
   a.ntiles = (int)((nlines + 127) / 128);
   a.o = o;
   a.eps = eps;
-  // row-wise outputs: line l at l * P (P a multiple of 8 bf16 or 4 floats)
+  // row-wise outputs: line l at l * P
   if (o.G == 1 && (o.D != 1 || o.E != 1 || o.F != 1)) return cudaErrorInvalidValue;
   a.lx = kp.lx; a.ly = kp.ly; a.lz = kp.lz;
   a.alpha = kp.alpha; a.gamma = kp.gamma;
-  a.X = kp.nx; a.Y = kp.ny;
+  a.X = kp.nx; a.Y = ks_pitch(kp.ny);
   a.err = kp.err;
   a.poll = kp.poll_limit ? kp.poll_limit : (1u << 22);
   a.zz = zz ? 1 : 0;
-  // the fused pass drains through the staging tiles: its output rows hold a multiple of 8 lines
-  if (zz && (axis != 2 || o.sym || !ks_staged(a) || a.Nt)) return cudaErrorInvalidValue;
+  const bool rows = o.G == 1;
+  // transposed outputs leave in aligned pieces of 8 lines (their rows hold whole such pieces)
+  if (!rows && (o.kind != KS_OUT_SPLIT || o.E % 8 || o.P % 8 || o.G % 8 || nlines % 8))
+    return cudaErrorInvalidValue;
+  if (rows && o.kind == KS_OUT_SPLIT) return cudaErrorInvalidValue;
+  if (zz && (axis != 2 || rows || a.Nt)) return cudaErrorInvalidValue;
   const int P = ks_pitch(a.L);
   const int np = split ? 2 : 1;
   // A: [2 planes][nlines][P] bf16, box 64 k x 128 lines, 128-byte swizzle; k >= L and lines
@@ -943,12 +887,12 @@ cudaError_t ks_axis_pass(const KPlan& kp, int axis, bool inverse, int split, con
   // outputs (or addresses the map cannot describe) take the per-thread stores.
   CUtensorMap tmO = tmA;
   a.ostore = 0;
-  if (ks_staged(a) && o.E % 32 == 0 && nlines % (o.E * o.D) == 0 &&
+  if (!rows && o.E % 32 == 0 && nlines % (o.E * o.D) == 0 &&
       (reinterpret_cast<uintptr_t>(o.out) & 15) == 0 &&
-      o.P % 8 == 0 && o.G % 8 == 0 && (o.F * o.P) % 8 == 0 && (!split || o.plane % 8 == 0)) {
-    const long long rows = (nlines + o.E - 1) / o.E;
+      (!split || o.plane % 8 == 0)) {
+    const long long nrows = (nlines + o.E - 1) / o.E;
     cuuint64_t dims[5] = {(cuuint64_t)o.E, (cuuint64_t)o.D, (cuuint64_t)min(a.L, a.Nc),
-                          (cuuint64_t)((rows + o.D - 1) / o.D), (cuuint64_t)(split ? 2 : 1)};
+                          (cuuint64_t)((nrows + o.D - 1) / o.D), (cuuint64_t)(split ? 2 : 1)};
     cuuint64_t strides[4] = {(cuuint64_t)o.P * 2, (cuuint64_t)o.G * 2, (cuuint64_t)(o.F * o.P) * 2,
                              (cuuint64_t)(split ? o.plane : o.F * o.P) * 2};
     cuuint32_t box[5] = {32, 1, 16, 1, 1}, es[5] = {1, 1, 1, 1, 1};
@@ -959,11 +903,11 @@ cudaError_t ks_axis_pass(const KPlan& kp, int axis, bool inverse, int split, con
   }
   // Shared memory (<= 225 KB): B resident when all its k-blocks fit next to 2 A stages;
   // otherwise 3 A stages (2 when needed) and as many streamed B stages as fit (at least 2).
-  // Staged and row outputs take 12 epilogue warps (three column ranges) when that still
-  // leaves room for 2 A and 2 B stages, else 8.
+  // 12 epilogue warps (three column ranges) when that still leaves room for 2 A and 2 B stages,
+  // else 8.
   const int ab = ks_abytes(split), bb = ks_bbytes(split, a.Nc);
   bool fits = false;
-  for (int parts = (ks_staged(a) || o.G == 1) ? 3 : 2; parts >= 2 && !fits; --parts) {
+  for (int parts = 3; parts >= 2 && !fits; --parts) {
     a.nparts = parts;
     const int budget = KS_SMEM_CAP - 1024 - ks_sbytes(a);
     if (!zz && a.nkb * bb + 2 * ab <= budget) {
@@ -987,14 +931,16 @@ cudaError_t ks_axis_pass(const KPlan& kp, int axis, bool inverse, int split, con
   if (a.Nt && (a.nparts - 1) * (a.Nc / 16) / a.nparts > KS_NMAIN / 16) return cudaErrorNotSupported;
   const int smem = ks_smem(a);
   const int epi = ks_epi(a);
-  auto kern = epi == EPI_T_STAGED ? k_dft_ks<EPI_T_STAGED>
-            : epi == EPI_T        ? k_dft_ks<EPI_T>
+  auto kern = epi == EPI_T        ? k_dft_ks<EPI_T>
             : epi == EPI_ROWS     ? k_dft_ks<EPI_ROWS>
-            : epi == EPI_ZZ       ? k_dft_ks<EPI_ZZ>
-                                  : k_dft_ks<EPI_UPD>;
+            : epi == EPI_ROWS_1   ? k_dft_ks<EPI_ROWS_1>
+            : epi == EPI_UPD      ? k_dft_ks<EPI_UPD>
+            : epi == EPI_UPD_1    ? k_dft_ks<EPI_UPD_1>
+            : epi == EPI_ZZ_RN    ? k_dft_ks<EPI_ZZ_RN>
+                                  : k_dft_ks<EPI_ZZ>;
   // The limit is set once per kernel, to the cap every pass stays under: a per-pass value would
   // lower it below what an earlier launch of the same kernel (a recorded graph node) needs.
-  static bool limit_set[5] = {false, false, false, false, false};
+  static bool limit_set[EPI_COUNT] = {};
   if (smem > KS_SMEM_CAP) return cudaErrorNotSupported;
   if (!limit_set[epi]) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -416,8 +416,8 @@ int record_step(lddmm_ctx* ctx) {
     // the residual b_j and the map of step j + 1 in one pass over u_j
     hk(KID_FWD_FUSED, 0);
     launch_fwd_fused(g, vj, uc, unx, dtx, dty, dtz, L.I0, ctx->J1 + j * N, ctx->W + j * N,
-                     ctx->b, c, 1.0f / L.hx, 1.0f / L.hy, 1.0f / L.hz, bsplit, ks_pitch(g.nx), s,
-                     ctx->st, rk_of(ctx));
+                     ctx->b, c, 1.0f / L.hx, 1.0f / L.hy, 1.0f / L.hz, bsplit, ks_pitch(g.nx),
+                     ks_pitch(g.ny), s, ctx->st, rk_of(ctx));
     hk(KID_FWD_FUSED, 1);
     if (j == T - 1) {     // J0_T = I0 o phi_{1,0} and E_data
       hk(KID_J0_EDATA, 0);
@@ -675,7 +675,8 @@ int lddmm_create(const lddmm_params* p, const float* I0, const float* I1, const 
   ctx->kcap = 3 * N;
   for (int l = 0; l < nl; ++l) {
     const Grid& g = ctx->levels[l].g;
-    ctx->kcap = std::max<int64_t>(ctx->kcap, ks_field_floats(g.nx, g.ny, g.nz, 3));
+    if (p->k_mode != LDDMM_K_FP32 && ks_shape(g.nx, g.ny, g.nz))
+      ctx->kcap = std::max<int64_t>(ctx->kcap, ks_field_floats(g.nx, g.ny, g.nz, 3));
   }
   const int64_t T = p->T;
   auto A = [&](cudaError_t e) {
