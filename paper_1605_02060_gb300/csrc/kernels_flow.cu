@@ -152,20 +152,43 @@ __global__ void __launch_bounds__(256) k_disp_march(Grid g, const ST* __restrict
   }
 }
 
-// Four planes per thread: deep enough to overlap the two latencies, short enough that the grid
-// (ceil(nz/4) blocks along z) fills the GPU several times over.
+// Planes a thread marches.  Four overlap the latencies of consecutive planes and fill a large grid
+// several times over; a small grid has too few blocks for that, and its time is the length of the
+// march.  The lines are drawn by the number of four-plane blocks (the SMs hold 1216 of these
+// blocks at a time), where the two sides measured equal (us per launch, 1 / 2 / 4 / 8 planes):
+//                              33x20x29 (48)   64^3 (256)        132x80x114 (1450)    264x160x228 (10260)
+//   k_disp_march               1.9/2.8/4.0/5.9  3.7/3.6/4.6/7.3  12.3/11.5/11.9/10.9  103/75/70/71
+//   k_back_terms_march         2.2/2.8/3.9/6.6  4.4/4.2/4.6/6.7  14.7/14.1/12.8/12.6  103/94/84/80
+//   k_fwd_fused_march          5.1/8.3/14/25    7.8/10/16/27     24/26/35/43          150/132/130/140
+// (128^3, 2048 blocks: k_fwd_fused_march 36/37/42/51; 200x120x160, 4200: 65/59/65/76.)
 constexpr int kFlowZ = 4;
+
+static int flow_blocks(const Grid& g) {
+  return ((g.nx + 31) / 32) * ((g.ny + 7) / 8) * ((g.nz + 3) / 4);
+}
+static dim3 flow_grid(const Grid& g, int zc) {
+  return dim3((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + zc - 1) / zc);
+}
+
+template <typename ST, int SGN, bool Q, int ZC>
+static void launch_disp_march_z(const Grid& g, const void* vj, const float* uin, float* uout,
+                                float dtx, float dty, float dtz, cudaStream_t s, int rk) {
+  const dim3 grid = flow_grid(g, ZC);
+  if (rk)
+    k_disp_march<ST, SGN, ZC, true, Q><<<grid, kBlock3d, 0, s>>>(g, (const ST*)vj, uin, uout, dtx,
+                                                                 dty, dtz);
+  else
+    k_disp_march<ST, SGN, ZC, false, Q><<<grid, kBlock3d, 0, s>>>(g, (const ST*)vj, uin, uout, dtx,
+                                                                  dty, dtz);
+}
 
 template <typename ST, int SGN, bool Q>
 static void launch_disp_march(const Grid& g, const void* vj, const float* uin, float* uout,
                               float dtx, float dty, float dtz, cudaStream_t s, int rk) {
-  const dim3 grid((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + kFlowZ - 1) / kFlowZ);
-  if (rk)
-    k_disp_march<ST, SGN, kFlowZ, true, Q><<<grid, kBlock3d, 0, s>>>(g, (const ST*)vj, uin, uout,
-                                                                     dtx, dty, dtz);
+  if (flow_blocks(g) <= 256)
+    launch_disp_march_z<ST, SGN, Q, 1>(g, vj, uin, uout, dtx, dty, dtz, s, rk);
   else
-    k_disp_march<ST, SGN, kFlowZ, false, Q><<<grid, kBlock3d, 0, s>>>(g, (const ST*)vj, uin,
-                                                                      uout, dtx, dty, dtz);
+    launch_disp_march_z<ST, SGN, Q, kFlowZ>(g, vj, uin, uout, dtx, dty, dtz, s, rk);
 }
 
 template <bool Q>
@@ -317,6 +340,19 @@ void launch_interleave(const void* a, const void* b, void* out, int64_t n, cudaS
     k_interleave<<<nb, t, 0, s>>>((const float*)a, (const float*)b, (float2*)out, n);
 }
 
+template <typename ST>
+static void launch_back_terms(const Grid& g, const float* uc, const void* IM, float* J1j, float* Wj,
+                              Acc* acc, cudaStream_t s) {
+  const typename Pair<ST>::T* im = reinterpret_cast<const typename Pair<ST>::T*>(IM);
+  const int nb = flow_blocks(g);
+  if (nb <= 256)
+    k_back_terms_march<ST, 1, true><<<flow_grid(g, 1), kBlock3d, 0, s>>>(g, uc, im, J1j, Wj, acc);
+  else if (nb <= 8192)
+    k_back_terms_march<ST, 4, true><<<flow_grid(g, 4), kBlock3d, 0, s>>>(g, uc, im, J1j, Wj, acc);
+  else
+    k_back_terms_march<ST, 8, true><<<flow_grid(g, 8), kBlock3d, 0, s>>>(g, uc, im, J1j, Wj, acc);
+}
+
 void launch_flow_back(const Grid& g, const void* vj, const float* u_next, float* u_cur,
                       const void* IM, float* J1j, float* Wj, float dtx, float dty, float dtz,
                       Acc* acc, cudaStream_t s, const Hook& hook, int st, int rk) {
@@ -324,13 +360,8 @@ void launch_flow_back(const Grid& g, const void* vj, const float* u_next, float*
   disp_step(+1, g, vj, u_next, u_cur, dtx, dty, dtz, s, st, rk, 1);
   hook(KID_BACK_DISP, 1);
   hook(KID_BACK_TERMS, 0);
-  const dim3 grid((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + kFlowZ - 1) / kFlowZ);
-  if (st)
-    k_back_terms_march<__nv_bfloat16, kFlowZ, true><<<grid, kBlock3d, 0, s>>>(
-        g, u_cur, (const __nv_bfloat162*)IM, J1j, Wj, acc);
-  else
-    k_back_terms_march<float, kFlowZ, true><<<grid, kBlock3d, 0, s>>>(g, u_cur, (const float2*)IM,
-                                                                      J1j, Wj, acc);
+  if (st) launch_back_terms<__nv_bfloat16>(g, u_cur, IM, J1j, Wj, acc, s);
+  else launch_back_terms<float>(g, u_cur, IM, J1j, Wj, acc, s);
   hook(KID_BACK_TERMS, 1);
 }
 
@@ -555,16 +586,23 @@ void launch_fwd_fused(const Grid& g, const void* vj, const float* u_cur, float* 
                       float dtx, float dty, float dtz, const void* I0, const float* J1j,
                       const float* Wj, float* b, float c, float ihx, float ihy, float ihz,
                       int bsplit, int px, int py, cudaStream_t s, int st, int rk) {
-  const dim3 grid((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + kFlowZ - 1) / kFlowZ);
-#define FWD_FUSED(ST_, RK_)                                                                    \
-  k_fwd_fused_march<ST_, kFlowZ, RK_, false><<<grid, kBlock3d, 0, s>>>(                       \
+  const int nb = flow_blocks(g);
+#define FWD_FUSED_Z(ST_, RK_, ZC_)                                                             \
+  k_fwd_fused_march<ST_, ZC_, RK_, false><<<flow_grid(g, ZC_), kBlock3d, 0, s>>>(             \
       g, (const ST_*)vj, u_cur, u_next, dtx, dty, dtz, (const ST_*)I0, J1j, Wj, b, c, ihx, ihy, \
       ihz, bsplit, px, py)
+#define FWD_FUSED(ST_, RK_)                                                                    \
+  do {                                                                                         \
+    if (nb <= 2048) FWD_FUSED_Z(ST_, RK_, 1);                                                  \
+    else if (nb <= 8192) FWD_FUSED_Z(ST_, RK_, 2);                                             \
+    else FWD_FUSED_Z(ST_, RK_, 4);                                                             \
+  } while (0)
   if (st) {
     if (rk) FWD_FUSED(__nv_bfloat16, true); else FWD_FUSED(__nv_bfloat16, false);
   } else {
     if (rk) FWD_FUSED(float, true); else FWD_FUSED(float, false);
   }
+#undef FWD_FUSED_Z
 #undef FWD_FUSED
 }
 
