@@ -114,6 +114,21 @@ __device__ __forceinline__ void split1(float x, uint16_t& h, uint16_t& l) {
   l = bf16_bits(__float2bfloat16_rn(x - __bfloat162float(hb)));
 }
 
+// The same of two values at once, packed: h = hi parts, l = lo parts, x0 in the low halves.
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t& h, uint32_t& l) {
+  const __nv_bfloat162 hb = __floats2bfloat162_rn(x0, x1);
+  h = *reinterpret_cast<const uint32_t*>(&hb);
+  const __nv_bfloat162 lb = __floats2bfloat162_rn(x0 - __uint_as_float(h << 16),
+                                                  x1 - __uint_as_float(h & 0xffff0000u));
+  l = *reinterpret_cast<const uint32_t*>(&lb);
+}
+// x / y through the hardware reciprocal (y a normal number: the symbol's square)
+__device__ __forceinline__ float div_fast(float x, float y) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(y));
+  return x * r;
+}
+
 // Bulk prefetch of [p, p + bytes) into L2 (16-byte aligned, bytes a multiple of 16).
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
@@ -144,10 +159,6 @@ __device__ __forceinline__ float4 bf4_to_f4(uint2 u) {
 __device__ __forceinline__ uint2 f4_to_bf4(float4 w) {
   const __nv_bfloat162 a = __floats2bfloat162_rn(w.x, w.y), b = __floats2bfloat162_rn(w.z, w.w);
   return make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
-}
-
-__device__ __forceinline__ uint32_t pack_bf16x2(uint16_t a, uint16_t b) {
-  return (uint32_t)a | ((uint32_t)b << 16);
 }
 
 // Row-wise outputs (o.G == 1, line l at l * o.P): the 16 columns n0.. of the warp's 32 lines
@@ -253,6 +264,18 @@ __host__ __device__ inline int ks_epi(const KsArgs& a) {
   return EPI_T;
 }
 
+// What bounds the passes at 264x160x228 (us; in brackets the HBM time of their bytes), from clocks
+// read in each role.  The tensor cores do not: an M = 128, K = 16 product takes N / 2 cycles (40 at
+// least), 24 us of the x passes, 12 of the y and 36 of the z.
+//   x forward 63 (34)  shared-memory bandwidth: MMA operands, 340 KB of table a tile and the
+//                      staged stores use 13.5k of a tile's 19k cycles;
+//   y         47 (34)  HBM, 5.0 TB/s;
+//   z fused   91 (34)  the epilogue warps: converting 5.6k and draining 9.9k of a tile's 24k cycles,
+//                      the drain waiting on the stores of 64-byte rows (95 before the TMEM loads ran
+//                      one chunk ahead and the splits worked on pairs; with a fourth column range,
+//                      576 threads at 96 registers, 107);
+//   x inverse 88 (51)  the epilogue's reads and writes of v in 64-byte pieces, 2.0k cycles a chunk
+//                      (106 with the old v requested a pair of chunks earlier, at 168 registers).
 template <int EPI>
 __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUtensorMap tmA,
                                                      const __grid_constant__ CUtensorMap tmB,
@@ -558,12 +581,15 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
         conv_ok = ptx::mbar_wait_or_abort(ptx::smem_u32(&b_tfull[0]), (uint32_t)i & 1u, abort, a.poll);
         ptx::tc_fence_after();
         const uint32_t t1 = tmem + ((uint32_t)(q * 32) << 16);
+        // the first chunk's load, then always the next one's while this one is converted
+        uint32_t uc[16], un[16];
+        if (conv_ok && part < nch) ptx::tmem_issue16(t1 + (uint32_t)(part * 16), uc);
         for (int kb = 0; conv_ok && kb < nkb; ++kb) {
           const int c1 = min(4 * kb + 4, nch);
-          for (int c = 4 * kb; c < c1; ++c) {
-            if (c % nparts != part) continue;
-            float vc[16];
-            ptx::tmem_ld16(t1 + (uint32_t)(c * 16), vc);
+          // this part's chunks of the block: c = part (mod nparts)
+          for (int c = 4 * kb + (part + nparts * nkb * 4 - 4 * kb) % nparts; c < c1; c += nparts) {
+            ptx::tmem_wait16(uc);
+            if (c + nparts < nch) ptx::tmem_issue16(t1 + (uint32_t)((c + nparts) * 16), un);
             const float4* lz4 = reinterpret_cast<const float4*>(a.lz + c * 16);
             uint32_t hw[8], lw[8];
 #pragma unroll
@@ -573,24 +599,22 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
 #pragma unroll
               for (int jj = 0; jj < 2; ++jj) {
                 const int j = 2 * j4 + jj;
-                uint16_t h0, l0, h1, l1;
+                const float v0 = __uint_as_float(uc[2 * j]), v1 = __uint_as_float(uc[2 * j + 1]);
                 if constexpr (EPI == EPI_ZZ_RN) {
                   const float d0 = fmaf(a.alpha, sxy + zl[2 * jj], a.gamma);
                   const float d1 = fmaf(a.alpha, sxy + zl[2 * jj + 1], a.gamma);
-                  split1(__fdiv_rn(vc[2 * j], d0 * d0), h0, l0);
-                  split1(__fdiv_rn(vc[2 * j + 1], d1 * d1), h1, l1);
+                  split2(__fdiv_rn(v0, d0 * d0), __fdiv_rn(v1, d1 * d1), hw[j], lw[j]);
                 } else {
                   const float d0 = fmaf(a.alpha, zl[2 * jj], sxy);
                   const float d1 = fmaf(a.alpha, zl[2 * jj + 1], sxy);
-                  split1(__fdividef(vc[2 * j], d0 * d0), h0, l0);
-                  split1(__fdividef(vc[2 * j + 1], d1 * d1), h1, l1);
+                  split2(div_fast(v0, d0 * d0), div_fast(v1, d1 * d1), hw[j], lw[j]);
                 }
-                hw[j] = pack_bf16x2(h0, h1);
-                lw[j] = pack_bf16x2(l0, l1);
               }
             }
             ptx::tmem_st8(t1 + (uint32_t)(c * 16), hw);
             if (a.split) ptx::tmem_st8(t1 + (uint32_t)(c * 16 + 8), lw);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) uc[j] = un[j];
           }
           ptx::tmem_wait_st();
           ptx::tc_fence_before();
@@ -642,12 +666,14 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
         uint16_t* wt = reinterpret_cast<uint16_t*>(stg) + part * (KS_CTILE / 2) + q * (2 * 16 * 32);
         const uint32_t wts = ptx::smem_u32(wt);
         const bool gvalid = line0 < a.nlines;
-        const long long t = line0 / o.E;
-        const int e0 = (int)(line0 - t * o.E), r1 = (int)(t % o.D), r3 = (int)(t / o.D);
+        const int E = (int)o.E, D = (int)o.D;
+        const int t = (int)line0 / E, e0 = (int)line0 - t * E, r3 = t / D, r1 = t - r3 * D;
+        uint32_t uc[16], un[16];
+        if (cnt > 0) ptx::tmem_issue16(tcol(chunk_at(0)), uc);
         for (int k = 0; k < cnt; ++k) {
           const int c = chunk_at(k);
-          float vc[16];
-          ptx::tmem_ld16(tcol(c), vc);
+          ptx::tmem_wait16(uc);
+          if (k + 1 < cnt) ptx::tmem_issue16(tcol(chunk_at(k + 1)), un);
           if (k + 1 == ntl) {             // the second product's columns are read
             ptx::tc_fence_before();
             ptx::mbar_arrive(ptx::smem_u32(&b_ttail));
@@ -655,11 +681,13 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
           if (lane == 0) ptx::bulk_wait_read_all();   // the previous boxes have left the tile
           __syncwarp();
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            uint16_t h, lo;
-            split1(vc[j], h, lo);
-            wt[j * 32 + lane] = h;
-            wt[512 + j * 32 + lane] = lo;
+          for (int j = 0; j < 16; j += 2) {
+            uint32_t h, lo;
+            split2(__uint_as_float(uc[j]), __uint_as_float(uc[j + 1]), h, lo);
+            wt[j * 32 + lane] = (uint16_t)h;
+            wt[(j + 1) * 32 + lane] = (uint16_t)(h >> 16);
+            wt[512 + j * 32 + lane] = (uint16_t)lo;
+            wt[512 + (j + 1) * 32 + lane] = (uint16_t)(lo >> 16);
           }
           ptx::fence_proxy_async_smem();
           __syncwarp();
@@ -668,6 +696,8 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
             if (a.split) ptx::tma_store_5d(&tmO, wts + 1024u, e0, r1, c * 16, r3, 1);
             ptx::bulk_commit();
           }
+#pragma unroll
+          for (int j = 0; j < 16; ++j) uc[j] = un[j];
         }
       } else if constexpr (staged) {
         // Transposed split output.  Per 16-column chunk the four quadrant warps of this column
