@@ -117,28 +117,22 @@ __global__ void k_transpose_flip(const __nv_bfloat16* __restrict__ w, __nv_bfloa
   wT[i] = w[((size_t)co * Ci + ci) * taps + (taps - 1 - t)];
 }
 
-// Weight gradient, deterministic.  dw[co][ci][t] is a product of Co x B n^3 by B n^3 x 27 Ci in
-// FP32 (274 GFLOP in a training step at 64^3, batch 8), so the FP32 pipes bound it and everything
-// else has to stay off their issue slots.  A block owns 16 output channels x CIT input channels
-// and the voxel tiles (units) g, g + G, ...; it stages a unit's x (with halo, [voxel][ci], rows
-// of CIT + 1 words: conflict free both ways) and dy ([voxel][16 co], 16-byte quads swizzled by
-// voxel) in shared memory by 4-byte asynchronous copies into two buffers, the next unit's under
-// the products of this one.  A thread owns one input channel, one dz, 8 output channels and one
-// of the KS slices of the tile's rows: it walks its rows in x with a 3 x 3 window of x in
-// registers, so a voxel costs 3 + 2 shared loads for 72 FMAs.  One block of 12 warps per SM: the
-// 72 sums want 167 registers.  The step's 15 weight gradients take 7.6 ms (36 TFLOP/s); one
-// (co, tap) per thread with two shared loads per FMA took 57.3 ms, this kernel with three blocks
-// of 6 warps at 96 registers (spilled sums) 14.3 ms, with two and loads through registers
-// 10.3 ms.  Packed fma.rn.f32x2 gains nothing (7.7 ms).
-// Partial sums part[g][co][ci][t] (and partb[g][co], from the blocks of the first input
-// channels) are added over g in a fixed order by k_wgrad_reduce: no floating-point atomics, the
-// same bits on every run.
-constexpr int WG_NT = 384, WG_TV = 256;
-
-struct WgTile {
-  int tx, ty, tz;      // voxels of a unit (tx * ty * tz <= WG_TV)
-  int ntx, nty, ntz;   // units of a sample along each axis
-};
+// Weight gradient, deterministic: dw[co][ci][t] is summed voxel by voxel in a fixed order.  Units
+// (batch, 8x8x4 tile) g, g + G, .. make one chain of FMAs per group g (x fastest, then y, z inside a
+// tile); part[g][co][ci][t] holds its end, and k_wgrad_reduce adds the groups in order.  No
+// floating-point atomics, the same bits on every run and for every shape of the block.
+// It is a product of Co x B n^3 by B n^3 x 27 Ci in FP32 (274 GFLOP in a training step at 64^3,
+// batch 8), so the FP32 pipes bound it and everything else has to stay off their issue slots.  A
+// block owns 16 output channels x CIT input channels of one group; it stages a unit's x (with halo,
+// [voxel][ci], rows of CIT + 1 words: conflict free both ways) and dy ([voxel][16 co], 16-byte quads
+// swizzled by voxel) by 4-byte asynchronous copies into two buffers, the next unit's under the
+// products of this one.  A thread owns one input channel, one dz and 2 output channels: it walks
+// the tile's 32 rows with a 3 x 3 window of x in registers, so a voxel costs 3 + 1 shared loads at
+// constant offsets for 18 FMAs.  The step's 14 such gradients take 8.2 ms; with one (co, tap) per
+// thread and two shared loads per FMA they took 57.
+constexpr int WG_CPT = 2, WG_HX = BX + 2, WG_HXY = (BX + 2) * (BY + 2), WG_HV = WG_HXY * (BZ + 2);
+__host__ __device__ constexpr int wg_threads(int cit) { return (cit * 3 * (CT / WG_CPT) + 31) / 32 * 32; }
+__host__ __device__ constexpr int wg_words(int cit) { return NTV * CT + WG_HV * (cit + 1); }
 
 // 4 bytes to shared memory, asynchronously; zeros when !in (the address is then not read)
 __device__ __forceinline__ void cp4(float* dst, const float* src, bool in) {
@@ -149,72 +143,57 @@ __device__ __forceinline__ void cp4(float* dst, const float* src, bool in) {
 }
 
 template <int CIT>
-__global__ void __launch_bounds__(WG_NT, 1) k_wgrad3(const float* __restrict__ x,
-                                                     const float* __restrict__ dy,
-                                                     float* __restrict__ part,
-                                                     float* __restrict__ partb, int B, int Ci,
-                                                     int Co, int n, WgTile tl, int G) {
-  constexpr int KS = WG_NT / (6 * CIT), XS = CIT + 1, NW = WG_NT / 32;
+__global__ void __launch_bounds__(wg_threads(CIT), 1) k_wgrad3(const float* __restrict__ x,
+                                                               const float* __restrict__ dy,
+                                                               float* __restrict__ part, int B,
+                                                               int Ci, int Co, int n, int G) {
+  constexpr int NT = wg_threads(CIT), NW = NT / 32, XS = CIT + 1, COG = CT / WG_CPT;
   extern __shared__ __align__(16) float wg_smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ci = tid % CIT, cog = (tid / CIT) & 1, dz = (tid / (2 * CIT)) % 3, ks = tid / (6 * CIT);
+  const int ci = tid % CIT, cog = (tid / CIT) % COG, dz = tid / (CIT * COG);
   const int nci = (Ci + CIT - 1) / CIT;
-  const int ci0 = (blockIdx.y % nci) * CIT, co0 = (blockIdx.y / nci) * 16;
-  const int HX = tl.tx + 2, HY = tl.ty + 2, HZ = tl.tz + 2, HXY = HX * HY;
-  const int rows = tl.ty * tl.tz, TV = rows * tl.tx;
-  const int tiles = tl.ntx * tl.nty * tl.ntz;
+  const int ci0 = (blockIdx.y % nci) * CIT, co0 = (blockIdx.y / nci) * CT;
+  const int ntx = (n + BX - 1) / BX, nty = (n + BY - 1) / BY, ntz = (n + BZ - 1) / BZ;
+  const int tiles = ntx * nty * ntz;
   const size_t nv = (size_t)n * n * n;
-  // two buffers of dy [WG_TV][16] (quads swizzled) and x [(tz+2)(ty+2)(tx+2)][XS]
-  const int bufw = (WG_TV * 16 + HXY * HZ * XS + 3) & ~3;
-  const bool bias = partb && ci0 == 0;
-  float bsum = 0.f;                           // channel tid % 16, voxels tid / 16, + NT / 16, ...
-  float s[8][9];
+  float s[WG_CPT][9];
 #pragma unroll
-  for (int c = 0; c < 8; ++c)
+  for (int c = 0; c < WG_CPT; ++c)
 #pragma unroll
     for (int t = 0; t < 9; ++t) s[c][t] = 0.f;
   auto stage = [&](int u, float* dys) {
-    float* xs = dys + WG_TV * 16;
+    float* xs = dys + NTV * CT;
     const int b = u / tiles, tile = u - b * tiles;
-    const int tx0 = (tile % tl.ntx) * tl.tx, ty0 = ((tile / tl.ntx) % tl.nty) * tl.ty,
-              tz0 = (tile / (tl.ntx * tl.nty)) * tl.tz;
-    // Warp w of the 12 takes the channels w % CG, + CG, ... and the positions of its third (or
-    // sixth) of the tile; a lane's position is decoded once for all channels and planes.  The
-    // addresses are clamped into the tensor, what lies outside the grid arrives as zero.
-    constexpr int CG = CIT < 4 ? CIT : 4, PG = NW / CG;
+    const int tx0 = (tile % ntx) * BX, ty0 = ((tile / ntx) % nty) * BY, tz0 = (tile / (ntx * nty)) * BZ;
+    // A warp takes the channels w % CG, + CG, ..; a lane's position is decoded once for all of them.
+    // Addresses are clamped into the tensor, what lies outside the grid arrives as zero.
+    constexpr int CG = NW >= 4 && CIT >= 4 ? 4 : 1, PG = NW / CG;
     const float* xb = x + ((size_t)b * Ci + ci0) * nv;
-    const int cw = warp % CG, pw = (warp / CG) * 32 + lane;
-    const int cmax = Ci - 1 - ci0;
-    for (int e = pw; e < HXY; e += PG * 32) {
-      const int hy = e / HX, hx = e - hy * HX;
-      const int gx = tx0 + hx - 1, gy = ty0 + hy - 1;
-      const bool inxy = gx >= 0 && gx < n && gy >= 0 && gy < n;
-      const int oxy = inxy ? gy * n + gx : 0;
+    const int cw = warp % CG, cmax = Ci - 1 - ci0;
+    for (int e = (warp / CG) * 32 + lane; e < WG_HV; e += PG * 32) {
+      const int hz = e / WG_HXY, r = e - hz * WG_HXY, hy = r / WG_HX, hx = r - hy * WG_HX;
+      const int gx = tx0 + hx - 1, gy = ty0 + hy - 1, gz = tz0 + hz - 1;
+      const bool in = gx >= 0 && gx < n && gy >= 0 && gy < n && gz >= 0 && gz < n;
+      const float* p = xb + (in ? ((size_t)gz * n + gy) * n + gx : 0);
       float* d = xs + e * XS + cw;
-      for (int hz = 0; hz < HZ; ++hz, d += HXY * XS) {
-        const int gz = tz0 + hz - 1;
-        const bool in = inxy && gz >= 0 && gz < n;
-        const float* p = xb + (size_t)(in ? gz : 0) * n * n + oxy;
 #pragma unroll
-        for (int k = 0; k < CIT / CG; ++k) {
-          const int c = cw + k * CG;
-          cp4(d + k * CG, p + (size_t)min(c, cmax) * nv, in && c <= cmax);
-        }
+      for (int k = 0; k < CIT / CG; ++k) {
+        const int c = cw + k * CG;
+        cp4(d + k * CG, p + (size_t)min(c, cmax) * nv, in && c <= cmax);
       }
     }
+    constexpr int DG = NW >= 4 ? 4 : 1;
     const float* dyb = dy + ((size_t)b * Co + co0) * nv;
-    const int gw = warp & 3, omax = Co - 1 - co0;
-    for (int v = (warp >> 2) * 32 + lane; v < TV; v += NW / 4 * 32) {
-      const int lx = v % tl.tx, r = v / tl.tx, ly = r % tl.ty, lz = r / tl.ty;
-      const int gx = tx0 + lx, gy = ty0 + ly, gz = tz0 + lz;
+    const int gw = warp % DG, omax = Co - 1 - co0;
+    for (int v = (warp / DG) * 32 + lane; v < NTV; v += NW / DG * 32) {
+      const int gx = tx0 + v % BX, gy = ty0 + v / BX % BY, gz = tz0 + v / (BX * BY);
       const bool in = gx < n && gy < n && gz < n;
       const float* p = dyb + (in ? ((size_t)gz * n + gy) * n + gx : 0);
-      float* d = dys + v * 16 + gw;
       const int sw = (v >> 1) & 3;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int c = gw + 4 * k;
-        cp4(d + ((k ^ sw) << 2), p + (size_t)min(c, omax) * nv, in && c <= omax);
+      for (int k = 0; k < CT / DG; ++k) {
+        const int c = gw + DG * k;
+        cp4(dys + v * CT + (((c >> 2) ^ sw) << 2) + (c & 3), p + (size_t)min(c, omax) * nv, in && c <= omax);
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -223,171 +202,177 @@ __global__ void __launch_bounds__(WG_NT, 1) k_wgrad3(const float* __restrict__ x
   int buf = 0;
   if ((int)blockIdx.x < units) stage(blockIdx.x, wg_smem);
   for (int u = blockIdx.x; u < units; u += G, buf ^= 1) {
-    const float* dys = wg_smem + buf * bufw;
-    const float* xs = dys + WG_TV * 16;
+    const float* dys = wg_smem + buf * wg_words(CIT);
+    const float* xs = dys + NTV * CT;
     if (u + G < units) {
-      stage(u + G, wg_smem + (buf ^ 1) * bufw);
+      stage(u + G, wg_smem + (buf ^ 1) * wg_words(CIT));
       asm volatile("cp.async.wait_group 1;" ::: "memory");
     } else {
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncthreads();
-    for (int r = ks; r < rows; r += KS) {
-      const int ly = r % tl.ty, lz = r / tl.ty;
-      const float* xr = xs + (((lz + dz) * HY + ly) * HX) * XS + ci;
-      float w[3][3];
+    if (dz < 3) {
+      const int q = cog * WG_CPT >> 2, qo = cog * WG_CPT & 3;   // the thread's quad of dy, place in it
+      for (int r = 0; r < BY * BZ; ++r) {
+        const float* xr = xs + (((r / BY + dz) * (BY + 2) + r % BY) * WG_HX) * XS + ci;
+        const float* dr = dys + r * BX * CT + qo;
+        float w[3][3];
 #pragma unroll
-      for (int d = 0; d < 3; ++d)
+        for (int d = 0; d < 3; ++d)
 #pragma unroll
-        for (int e = 0; e < 2; ++e) w[d][e] = xr[(d * HX + e) * XS];
-      int v = r * tl.tx;
-#pragma unroll 3
-      for (int lx = 0; lx < tl.tx; ++lx, ++v) {
+          for (int e = 0; e < 2; ++e) w[d][e] = xr[(d * WG_HX + e) * XS];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) w[d][2] = xr[(d * HX + lx + 2) * XS];
-        const int sw = (v >> 1) & 3;
-        const float4 p0 = reinterpret_cast<const float4*>(dys)[v * 4 + ((2 * cog) ^ sw)];
-        const float4 p1 = reinterpret_cast<const float4*>(dys)[v * 4 + ((2 * cog + 1) ^ sw)];
-        const float g8[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+        for (int lx = 0; lx < BX; ++lx) {
 #pragma unroll
-        for (int c = 0; c < 8; ++c)
+          for (int d = 0; d < 3; ++d) w[d][2] = xr[(d * WG_HX + lx + 2) * XS];
+          const float2 g = *reinterpret_cast<const float2*>(dr + lx * CT + ((q ^ ((lx >> 1) & 3)) << 2));
 #pragma unroll
           for (int d = 0; d < 3; ++d)
 #pragma unroll
-            for (int e = 0; e < 3; ++e) s[c][d * 3 + e] = fmaf(g8[c], w[d][e], s[c][d * 3 + e]);
+            for (int e = 0; e < 3; ++e) {
+              s[0][d * 3 + e] = fmaf(g.x, w[d][e], s[0][d * 3 + e]);
+              s[1][d * 3 + e] = fmaf(g.y, w[d][e], s[1][d * 3 + e]);
+            }
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          w[d][0] = w[d][1];
-          w[d][1] = w[d][2];
+          for (int d = 0; d < 3; ++d) {
+            w[d][0] = w[d][1];
+            w[d][1] = w[d][2];
+          }
         }
       }
     }
-    if (bias) {
-      const int c = tid & 15, q = c >> 2;
-      for (int v = tid >> 4; v < TV; v += WG_NT / 16)
-        bsum += dys[(v * 4 + (q ^ ((v >> 1) & 3))) * 4 + (c & 3)];
-    }
     __syncthreads();
   }
-  // the KS row slices are added in order, through shared memory
-  const int slot = tid % (6 * CIT);
-  for (int k = 1; k < KS; ++k) {
-    if (ks == k)
-#pragma unroll
-      for (int c = 0; c < 8; ++c)
-#pragma unroll
-        for (int t = 0; t < 9; ++t) wg_smem[(c * 9 + t) * (6 * CIT) + slot] = s[c][t];
-    __syncthreads();
-    if (ks == 0)
-#pragma unroll
-      for (int c = 0; c < 8; ++c)
-#pragma unroll
-        for (int t = 0; t < 9; ++t) s[c][t] += wg_smem[(c * 9 + t) * (6 * CIT) + slot];
-    __syncthreads();
-  }
-  if (ks == 0 && ci0 + ci < Ci) {
+  if (dz < 3 && ci0 + ci < Ci) {
     float* po = part + (size_t)blockIdx.x * Co * Ci * 27;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const int co = co0 + cog * 8 + c;
+    for (int c = 0; c < WG_CPT; ++c) {
+      const int co = co0 + cog * WG_CPT + c;
       if (co < Co)
 #pragma unroll
         for (int t = 0; t < 9; ++t) po[((size_t)co * Ci + ci0 + ci) * 27 + dz * 9 + t] = s[c][t];
     }
   }
-  if (bias) {
-    wg_smem[tid] = bsum;
-    __syncthreads();
-    if (tid < 16 && co0 + tid < Co) {
-      float t = 0.f;
-      for (int k = 0; k < WG_NT / 16; ++k) t += wg_smem[k * 16 + tid];
-      partb[(size_t)blockIdx.x * Co + co0 + tid] = t;
-    }
-  }
 }
 
-// Weight gradient of a 1^3 convolution (the head): a thread walks voxels with 4 x 16 sums in
-// registers (4 output, 16 input channels per block), one coalesced load per channel; bound by
-// reading x and dy once.  The sums meet by a fixed shuffle tree, then over the warps in order.
-__global__ void __launch_bounds__(256) k_wgrad1(const float* __restrict__ x,
-                                                const float* __restrict__ dy,
-                                                float* __restrict__ part, float* __restrict__ partb,
-                                                int B, int Ci, int Co, int n, int G) {
-  __shared__ float red[8][68];
+// The same for a 1^3 convolution (the head): a block owns 16 x 16 channels of one group, a thread one
+// pair of them; x and dy of a unit lie in shared memory as [voxel][16 channels] (17 words), the next
+// unit's copies run under this one's chain.
+__global__ void __launch_bounds__(256, 1) k_wgrad1(const float* __restrict__ x,
+                                                   const float* __restrict__ dy,
+                                                   float* __restrict__ part, int B, int Ci, int Co,
+                                                   int n, int G) {
+  extern __shared__ __align__(16) float wg_smem[];
+  constexpr int S1 = CT + 1, HALF = NTV * S1, W1 = 2 * HALF;
+  const int tid = threadIdx.x;
   const int nci = (Ci + 15) / 16;
-  const int ci0 = (blockIdx.y % nci) * 16, co0 = (blockIdx.y / nci) * 4;
-  const int64_t nv = (int64_t)n * n * n;
-  const int64_t per = (nv * B + G - 1) / G;
-  const int64_t lo = blockIdx.x * per, hi = min(lo + per, nv * B);
-  float s[4][16], sb[4];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    sb[c] = 0.f;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) s[c][k] = 0.f;
-  }
-  for (int64_t i = lo + threadIdx.x; i < hi; i += 256) {
-    const int64_t b = i / nv, v = i - b * nv;
-    float g[4], xv[16];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) g[c] = co0 + c < Co ? __ldg(dy + (b * Co + co0 + c) * nv + v) : 0.f;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) xv[k] = ci0 + k < Ci ? __ldg(x + (b * Ci + ci0 + k) * nv + v) : 0.f;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      sb[c] += g[c];
-#pragma unroll
-      for (int k = 0; k < 16; ++k) s[c][k] = fmaf(g[c], xv[k], s[c][k]);
+  const int ci0 = (blockIdx.y % nci) * 16, co0 = (blockIdx.y / nci) * CT;
+  const int ntx = (n + BX - 1) / BX, nty = (n + BY - 1) / BY, ntz = (n + BZ - 1) / BZ;
+  const int tiles = ntx * nty * ntz, units = tiles * B;
+  const size_t nv = (size_t)n * n * n;
+  const int ni = min(16, Ci - ci0), no = min(CT, Co - co0);
+  auto stage = [&](int u, float* xs) {
+    const int b = u / tiles, tile = u - b * tiles;
+    const int gx = (tile % ntx) * BX + tid % BX, gy = ((tile / ntx) % nty) * BY + tid / BX % BY,
+              gz = (tile / (ntx * nty)) * BZ + tid / (BX * BY);
+    const bool in = gx < n && gy < n && gz < n;
+    const size_t o = in ? ((size_t)gz * n + gy) * n + gx : 0;
+    const float* xb = x + ((size_t)b * Ci + ci0) * nv + o;
+    const float* db = dy + ((size_t)b * Co + co0) * nv + o;
+    for (int c = 0; c < ni; ++c) cp4(xs + tid * S1 + c, xb + (size_t)c * nv, in);
+    for (int c = 0; c < no; ++c) cp4(xs + HALF + tid * S1 + c, db + (size_t)c * nv, in);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int ci = tid & 15, co = tid >> 4;
+  float s = 0.f;
+  int buf = 0;
+  if ((int)blockIdx.x < units) stage(blockIdx.x, wg_smem);
+  for (int u = blockIdx.x; u < units; u += G, buf ^= 1) {
+    if (u + G < units) {
+      stage(u + G, wg_smem + (buf ^ 1) * W1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const float t = warp_sum_f(s[c][k]);
-      if (lane == 0) red[warp][c * 16 + k] = t;
+    __syncthreads();
+    if (ci < ni && co < no) {
+      const float* xs = wg_smem + buf * W1 + ci;
+      const float* ds = wg_smem + buf * W1 + HALF + co;
+#pragma unroll 16
+      for (int v = 0; v < NTV; ++v) s = fmaf(ds[v * S1], xs[v * S1], s);
     }
-    const float t = warp_sum_f(sb[c]);
-    if (lane == 0) red[warp][64 + c] = t;
+    __syncthreads();
   }
+  if (ci < ni && co < no) part[((size_t)blockIdx.x * Co + co0 + co) * Ci + ci0 + ci] = s;
+}
+
+// dw[i] += sum_{g = 0..G-1} part[g][i], in that order; 16 loads in flight.
+__global__ void __launch_bounds__(64) k_wgrad_reduce(const float* __restrict__ part,
+                                                     float* __restrict__ dw, int64_t count, int G) {
+  const int64_t i = (int64_t)blockIdx.x * 64 + threadIdx.x;
+  if (i >= count) return;
+  const float* p = part + i;
+  float s = 0.f;
+  int g = 0;
+  for (; g + 16 <= G; g += 16) {
+    float v[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v[k] = __ldg(p + (size_t)(g + k) * count);
+#pragma unroll
+    for (int k = 0; k < 16; ++k) s += v[k];
+  }
+  for (; g < G; ++g) s += __ldg(p + (size_t)g * count);
+  dw[i] += s;
+}
+
+// Bias gradient, deterministic: block (co, g) sums the fixed chunk g of the B * n^3 values of
+// channel co (a thread every 256th value, eight loads in flight; then a tree of fixed shape) into
+// partb[co][g]; k_bias_reduce adds them in order.
+__global__ void __launch_bounds__(256) k_bias_partial(const float* __restrict__ dy,
+                                                      float* __restrict__ partb, int B, int Co,
+                                                      int n, int GB) {
+  const int co = blockIdx.x, g = blockIdx.y;
+  const size_t nv = (size_t)n * n * n;
+  const size_t total = (size_t)B * nv, chunk = (total + GB - 1) / GB;
+  const size_t lo = (size_t)g * chunk, hi = lo + chunk < total ? lo + chunk : total;
+  float s = 0.f;
+  // value i of the channel lies at (b Co + co) nv + v, i = b nv + v; b steps up as i passes it
+  size_t i = lo + threadIdx.x, b = i / nv, end = (b + 1) * nv;
+  const float* p = dy + (b * Co + co) * nv - b * nv;
+  auto at = [&](size_t k) {
+    while (k >= end) {
+      ++b;
+      end += nv;
+      p += (size_t)(Co - 1) * nv;
+    }
+    return __ldg(p + k);
+  };
+  while (i < hi) {
+    float v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = i + 256 * k < hi ? at(i + 256 * k) : 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (i + 256 * k < hi) s += v[k];
+    i += 2048;
+  }
+  __shared__ float red[32];
+  s = warp_sum_f(s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x < 68) {
-    float t = 0.f;
-    for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
-    if (threadIdx.x < 64) {
-      const int co = co0 + threadIdx.x / 16, ci = ci0 + threadIdx.x % 16;
-      if (co < Co && ci < Ci) part[((size_t)blockIdx.x * Co + co) * Ci + ci] = t;
-    } else if (partb && ci0 == 0 && co0 + (int)threadIdx.x - 64 < Co) {
-      partb[(size_t)blockIdx.x * Co + co0 + threadIdx.x - 64] = t;
-    }
+  if (threadIdx.x < 32) {
+    float t = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.f;
+    t = warp_sum_f(t);
+    if (threadIdx.x == 0) partb[(size_t)co * GB + g] = t;
   }
 }
 
-// dw[i] += sum_g part[g][i] (and db from partb): a block adds 32 values, its 8 warps the groups
-// g = w, w + 8, ..., then the warps' sums in order.
-__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ part,
-                                                      float* __restrict__ dw, int64_t count,
-                                                      const float* __restrict__ partb,
-                                                      float* __restrict__ db, int Co, int G) {
-  __shared__ float red[8][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t nb = (count + 31) / 32;
-  const bool isb = blockIdx.x >= nb;
-  const int64_t i = (isb ? blockIdx.x - nb : blockIdx.x) * 32 + lane, m = isb ? Co : count;
-  const float* p = isb ? partb : part;
+__global__ void k_bias_reduce(const float* __restrict__ partb, float* __restrict__ db, int Co, int GB) {
+  const int co = blockIdx.x * blockDim.x + threadIdx.x;
+  if (co >= Co) return;
   float s = 0.f;
-  if (i < m) {
-#pragma unroll 4
-    for (int g = warp; g < G; g += 8) s += __ldg(p + (size_t)g * m + i);
-  }
-  red[warp][lane] = s;
-  __syncthreads();
-  if (warp == 0 && i < m) {
-    float t = 0.f;
-    for (int w = 0; w < 8; ++w) t += red[w][lane];
-    (isb ? db : dw)[i] += t;
-  }
+  for (int g = 0; g < GB; ++g) s += partb[(size_t)co * GB + g];
+  db[co] += s;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -553,91 +538,66 @@ cudaError_t net_conv_dgrad(const float* dy, const void* w, void* wT_scratch, flo
   return net_conv_fwd(dy, wT_scratch, nullptr, dx, B, Co, Ci, n, ks, 0, 0, s);
 }
 
-// Partition of the weight gradient: input channels per block (16, or the next power of two of
-// fewer), the voxel tile of a unit (rows of up to 32 voxels, split evenly so that 40 or 56 leave
-// no ragged end; ty grows while the tile has room, so that short rows keep a small halo), and the
-// number of groups G: one block per SM on 152 SMs (three for the 1^3 kernel, which waits on
-// memory), evened out over the units.
-struct WgPlan {
-  int cit, G;
-  WgTile tl;
-};
-static WgPlan wgrad_plan(int B, int Ci, int Co, int n, int ks) {
-  WgPlan p{};
-  const int64_t slots = 152 * (ks == 1 ? 3 : 1);
-  if (ks == 1) {
-    const int64_t nblk = (int64_t)((Ci + 15) / 16) * ((Co + 3) / 4);
-    const int64_t units = ((int64_t)B * n * n * n + 2047) / 2048;
-    const int64_t g = slots / nblk;
-    p.G = (int)(g < 1 ? 1 : (g > units ? units : g));
-    return p;
-  }
-  p.cit = Ci > 8 ? 16 : Ci > 4 ? 8 : Ci > 2 ? 4 : 2;
-  const auto even = [](int len, int most) {
-    const int k = (len + most - 1) / most;
-    return (len + k - 1) / k;
-  };
-  WgTile& t = p.tl;
-  t.tx = even(n, 32);
-  t.ty = even(n, t.tx > 16 ? 4 : t.tx > 8 ? 4 : 8);
-  const int room = WG_TV / (t.tx * t.ty);
-  t.tz = even(n, room < 1 ? 1 : (room > 4 ? 4 : room));
-  t.ntx = (n + t.tx - 1) / t.tx;
-  t.nty = (n + t.ty - 1) / t.ty;
-  t.ntz = (n + t.tz - 1) / t.tz;
-  const int64_t nblk = (int64_t)((Ci + p.cit - 1) / p.cit) * ((Co + 15) / 16);
-  const int64_t units = (int64_t)t.ntx * t.nty * t.ntz * B;
-  int64_t g = slots / nblk;
-  g = g < 1 ? 1 : (g > units ? units : g);
-  const int64_t rounds = (units + g - 1) / g;
-  p.G = (int)((units + rounds - 1) / rounds);
-  return p;
+// Partition of the weight-gradient sums: G voxel groups (about 2048 chains of units per 16 output
+// channels and tap, at most one group per (batch, tile) unit), GB chunks per bias channel.
+static void wgrad_groups(int B, int Ci, int Co, int n, int* G, int* GB) {
+  const int units = tiles_of(n) * B;
+  const int cb = Ci * ((Co + CT - 1) / CT);
+  int g = (2048 + cb - 1) / cb;
+  *G = g < 1 ? 1 : (g > units ? units : g);
+  const int64_t total = (int64_t)B * n * n * n;
+  int64_t gb = (total + 8191) / 8192;
+  *GB = (int)(gb < 1 ? 1 : (gb > 64 ? 64 : gb));
 }
 
 int64_t net_conv_wgrad_scratch(int B, int Ci, int Co, int n, int ks) {
-  const WgPlan p = wgrad_plan(B, Ci, Co, n, ks);
-  return (int64_t)p.G * Co * Ci * ks * ks * ks + (int64_t)p.G * Co;
+  int G, GB;
+  wgrad_groups(B, Ci, Co, n, &G, &GB);
+  return (int64_t)G * Co * Ci * ks * ks * ks + (int64_t)Co * GB;
 }
 
 template <int CIT>
-static cudaError_t launch_wgrad3(const float* x, const float* dy, float* part, float* partb, int B,
-                                 int Ci, int Co, int n, const WgPlan& p, cudaStream_t s) {
-  // two staging buffers, or the row slices' sums at the end
-  const auto words = [](int halo) { return 2 * ((WG_TV * 16 + halo * (CIT + 1) + 3) & ~3); };
-  const int fl = words((p.tl.tx + 2) * (p.tl.ty + 2) * (p.tl.tz + 2)), fe = 72 * 6 * CIT;
-  const int smem = 4 * (fl > fe ? fl : fe);
-  const int kMost = 4 * words(34 * 6 * 4);   // the largest tile's
-  static const cudaError_t set = cudaFuncSetAttribute(
-      k_wgrad3<CIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+static cudaError_t launch_wgrad3(const float* x, const float* dy, float* part, int B, int Ci, int Co,
+                                 int n, int G, cudaStream_t s) {
+  constexpr int smem = 2 * 4 * wg_words(CIT);
+  static const cudaError_t set =
+      cudaFuncSetAttribute(k_wgrad3<CIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (set != cudaSuccess) return set;
-  if (smem > kMost) return cudaErrorInvalidValue;
-  const dim3 grid(p.G, ((Ci + CIT - 1) / CIT) * ((Co + 15) / 16));
-  k_wgrad3<CIT><<<grid, WG_NT, smem, s>>>(x, dy, part, partb, B, Ci, Co, n, p.tl, p.G);
+  const dim3 grid(G, ((Ci + CIT - 1) / CIT) * ((Co + CT - 1) / CT));
+  k_wgrad3<CIT><<<grid, wg_threads(CIT), smem, s>>>(x, dy, part, B, Ci, Co, n, G);
   return cudaGetLastError();
 }
 
 cudaError_t net_conv_wgrad(const float* x, const float* dy, float* dw, float* db, float* scratch,
                            int B, int Ci, int Co, int n, int ks, cudaStream_t s) {
-  const WgPlan p = wgrad_plan(B, Ci, Co, n, ks);
+  int G, GB;
+  wgrad_groups(B, Ci, Co, n, &G, &GB);
   const int64_t count = (int64_t)Co * Ci * ks * ks * ks;
-  float* partb = db ? scratch + (size_t)p.G * count : nullptr;
   cudaError_t e;
   if (ks == 1) {
-    const dim3 grid(p.G, ((Ci + 15) / 16) * ((Co + 3) / 4));
-    k_wgrad1<<<grid, 256, 0, s>>>(x, dy, scratch, partb, B, Ci, Co, n, p.G);
+    constexpr int smem = 2 * 4 * 2 * NTV * (CT + 1);
+    static const cudaError_t set =
+        cudaFuncSetAttribute(k_wgrad1, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (set != cudaSuccess) return set;
+    const dim3 grid(G, ((Ci + 15) / 16) * ((Co + CT - 1) / CT));
+    k_wgrad1<<<grid, 256, smem, s>>>(x, dy, scratch, B, Ci, Co, n, G);
     e = cudaGetLastError();
-  } else if (p.cit == 16) {
-    e = launch_wgrad3<16>(x, dy, scratch, partb, B, Ci, Co, n, p, s);
-  } else if (p.cit == 8) {
-    e = launch_wgrad3<8>(x, dy, scratch, partb, B, Ci, Co, n, p, s);
-  } else if (p.cit == 4) {
-    e = launch_wgrad3<4>(x, dy, scratch, partb, B, Ci, Co, n, p, s);
+  } else if (Ci > 8) {
+    e = launch_wgrad3<16>(x, dy, scratch, B, Ci, Co, n, G, s);
+  } else if (Ci > 4) {
+    e = launch_wgrad3<8>(x, dy, scratch, B, Ci, Co, n, G, s);
+  } else if (Ci > 2) {
+    e = launch_wgrad3<4>(x, dy, scratch, B, Ci, Co, n, G, s);
   } else {
-    e = launch_wgrad3<2>(x, dy, scratch, partb, B, Ci, Co, n, p, s);
+    e = launch_wgrad3<2>(x, dy, scratch, B, Ci, Co, n, G, s);
   }
   if (e != cudaSuccess) return e;
-  const unsigned nb = (unsigned)((count + 31) / 32 + (db ? (Co + 31) / 32 : 0));
-  k_wgrad_reduce<<<nb, 256, 0, s>>>(scratch, dw, count, partb, db, Co, p.G);
+  k_wgrad_reduce<<<(unsigned)((count + 63) / 64), 64, 0, s>>>(scratch, dw, count, G);
+  if (db) {
+    float* partb = scratch + (size_t)G * count;
+    k_bias_partial<<<dim3(Co, GB), 256, 0, s>>>(dy, partb, B, Co, n, GB);
+    k_bias_reduce<<<(Co + 127) / 128, 128, 0, s>>>(partb, db, Co, GB);
+  }
   return cudaGetLastError();
 }
 
