@@ -1,25 +1,29 @@
 // 3D convolution of the warm-start network on the tensor cores (tcgen05, sm_103a), as an
 // implicit GEMM:
 //     Y[b, co, v] = bias[co] + sum_{ci, t} X[b, ci, v + o(t)] W[co, ci, t]     (zero padding)
-// with M = 128 consecutive output voxels of one sample (a tile), N = Co (padded to a multiple of
-// 16) and K = Ci x taps walked as k-steps of 16 input channels at one tap t.
+// with N = Co (padded to a multiple of 16) and K = Ci x taps walked as k-steps of 16 input
+// channels at one tap t, channel groups outside, taps inside.
 //
-// The activations stay float32 [B][C][n^3]; the weights are bf16 [Co][Ci][taps].  Each k-step's
-// A slice (128 voxels x 16 channels, shifted by the tap, zero outside the grid) is split into a
-// bf16 hi and lo part (x = hi + lo to 16 mantissa bits), so the two products hi*W + lo*W give
-// the FP32 activations times the bf16 weights to ~2^-17, the same numbers as the CUDA-core
-// kernel up to rounding order; accumulation is FP32 in TMEM.
+// M: rows are consecutive positions of the grid with its border of zeros (P = n + 2 per axis; the
+// rows that fall on the border are computed and dropped, 6% at 64^3).  In that order a tap is a
+// constant shift, so a CTA stages the R + 2 P + 2 positions that its R rows reach in each of the
+// three z planes once per channel group, and a tap's A operand is the same shared memory from
+// another start: in the K-major layout without swizzle a row of 8 channels is 16 bytes, rows lie
+// 16 bytes apart, and a descriptor may start at any 16-byte address.  A voxel is then loaded,
+// split and stored about 5 times per channel group, not 27 times (once per tap): the 27
+// convolutions of a 64^3, batch 8 training step take 4.7 ms instead of 17.0 ms.
 //
-// Roles inside one CTA (one tile of 128 voxels, all Co):
-//   warps 0-7   stage each k-step: thread (voxel m = tid % 128, half h = tid / 128) gathers 8
-//               input channels of its shifted voxel and writes their hi/lo bf16 in the K-major
-//               core-matrix layout; the same threads copy the k-step's weight slice [Co][16];
-//               proxy fence, arrive on the stage's full barrier.  After the last k-step warps
-//               0-3 read the accumulator (warp w owns TMEM lanes 32w..32w+31) and add the bias,
-//               the optional old output and ReLU; warps 4-7 take the upper half of the columns.
-//   warp 8      TMEM owner and MMA issuer (one thread): two MMAs per k-step, a commit frees the
-//               stage, a final commit hands the accumulator to the epilogue.
-// Every wait is bounded: a timeout sets *err and the CTA drains, frees TMEM and returns.
+// The activations stay float32 [B][C][n^3]; the weights are bf16 [Co][Ci][taps].  A value is split
+// into a bf16 hi and lo part (x = hi + lo to 16 mantissa bits), so the two products hi*W + lo*W
+// give the FP32 activations times the bf16 weights to ~2^-17; accumulation is FP32 in TMEM.  A
+// product of M = 128, K = 16 and N <= 32 takes 40 cycles (it is bound by reading A), 54 of them per
+// row tile and channel group.
+//
+// One CTA: 256 threads stage, one of them issues the MMAs of a channel group, all wait for them
+// (one buffer), and read the accumulators at the end.  Two CTAs per SM where shared memory allows:
+// one stages while the other's products run.  (Weights fetched one 2-byte element at a time and
+// positions decoded by division, 8 loads in flight: 10.4 ms.)
+// Every wait is bounded: a timeout sets *err, marks the CTA's outputs NaN and returns.
 #include <cuda_bf16.h>
 
 #include "kernels.h"
@@ -29,182 +33,203 @@ namespace lddmm {
 
 namespace {
 
-constexpr int CV_THREADS = 288;     // 8 staging/epilogue warps + the MMA warp
-constexpr int CV_STAGES = 4;
-constexpr int CV_ABYTES = 128 * 16 * 2;   // one bf16 A operand (hi or lo)
+constexpr int CV_THREADS = 256;
+constexpr int CV_SMEM_CAP = 225 * 1024;
 
-__device__ __forceinline__ uint32_t cv_kmaj(int row, int kk) {
-  return (uint32_t)((kk >> 3) * 128 + (row >> 3) * 256 + (row & 7) * 16 + (kk & 7) * 2);
-}
+struct ConvArgs {
+  const float* x;
+  const __nv_bfloat16* w;
+  const float* bias;
+  float* y;
+  int Ci, Co, Np, n;
+  int taps, nph;        // filter taps; steps a channel group takes (1, or 3: a z plane each)
+  int pad, P;           // border, n + 2 border
+  int T, L;             // row tiles of 128 per CTA; positions staged per plane
+  int p_lo, p_hi;       // first and last position of a voxel
+  int relu, accumulate, tcols;
+  unsigned mP, mL;      // reciprocals of P and L (0: divide)
+  int* err;
+};
 
-__host__ __device__ inline int cv_stage_bytes(int Np) { return 2 * CV_ABYTES + Np * 32; }
-__device__ __forceinline__ int q_of(int warp) { return warp & 3; }
+// bytes of a step: positions of `planes` z planes, weights of `taps` taps
+inline int cv_smem(int planes, int L, int taps, int Np) { return 64 * planes * L + taps * Np * 32; }
 
 __device__ __forceinline__ uint32_t pack_bf2(float a, float b) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-__global__ void __launch_bounds__(CV_THREADS) k_conv_tc(const float* __restrict__ x,
-                                                        const __nv_bfloat16* __restrict__ w,
-                                                        const float* __restrict__ bias,
-                                                        float* __restrict__ y, int Ci, int Co,
-                                                        int Np, int n, int ks, int relu,
-                                                        int accumulate, int tcols, int* err) {
-  extern __shared__ __align__(128) uint8_t cv_smem[];
-  __shared__ __align__(8) uint64_t b_full[CV_STAGES], b_empty[CV_STAGES], b_done;
+// TPS taps a step: 27 (three z planes), 9 (one of the three) or 1 (a 1^3 filter).
+template <int TPS>
+__global__ void __launch_bounds__(CV_THREADS, 2) k_conv_tc(ConvArgs a) {
+  constexpr int PL = TPS == 27 ? 3 : 1;
+  extern __shared__ __align__(128) uint8_t cv_sm[];
+  __shared__ __align__(8) uint64_t b_done;
   __shared__ uint32_t tmem_sh;
-  __shared__ int abort_sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int b = blockIdx.y;
-  const long long nv = (long long)n * n * n;
-  const long long v0 = (long long)blockIdx.x * 128;
-  const int taps = ks * ks * ks;
-  const int nkc = Ci / 16;                  // channel groups
-  const int nsteps = nkc * taps;
-  const int sb = cv_stage_bytes(Np);
-  volatile int* abort = &abort_sh;
+  const int b = blockIdx.y, n = a.n, P = a.P;
+  const int p0 = a.p_lo + blockIdx.x * (a.T * 128);      // position of row 0
+  const size_t nv = (size_t)n * n * n;
+  const int span = PL * a.L;                              // positions of a step's planes
+  uint8_t* const bsm = cv_sm + 64 * span;
 
-  if (warp == 8) {
-    ptx::tmem_alloc(ptx::smem_u32(&tmem_sh), (uint32_t)tcols);
+  if (warp == 0) {
+    ptx::tmem_alloc(ptx::smem_u32(&tmem_sh), (uint32_t)a.tcols);
     ptx::tmem_relinquish();
   }
   if (tid == 0) {
-    for (int s = 0; s < CV_STAGES; ++s) {
-      ptx::mbar_init(ptx::smem_u32(&b_full[s]), 256);
-      ptx::mbar_init(ptx::smem_u32(&b_empty[s]), 1);
-    }
     ptx::mbar_init(ptx::smem_u32(&b_done), 1);
     ptx::fence_mbar_init();
-    abort_sh = 0;
   }
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = tmem_sh;
 
-  if (warp < 8) {
+  // quotient by a divisor d with m = ceil(2^32 / d), exact while q d < 2^32 (the launch sees to it)
+  auto quot = [](int q, int d, unsigned m) {
+    return m ? (int)__umulhi((unsigned)q, m) : q / d;
+  };
+  // voxel offset of position p, -1 on the border or beyond
+  auto voxel_at = [&](int p) -> int {
+    if (p < 0) return -1;
+    const int row = quot(p, P, a.mP), x = p - row * P - a.pad, zz = quot(row, P, a.mP);
+    const int y = row - zz * P - a.pad, z = zz - a.pad;
+    if (x < 0 || x >= n || y < 0 || y >= n || z < 0 || z >= n) return -1;
+    return (z * n + y) * n + x;
+  };
+
+  const int nst = a.Ci / 16 * a.nph;
+  bool ok = true;
+  for (int st = 0; st < nst && ok; ++st) {
+    const int kc = a.nph == 1 ? st : st / 3, ph = st - kc * a.nph;
+    const int first = p0 + (a.taps > 1 ? (ph - 1) * P * P - P - 1 : 0);
     // ------------------------------------------------------------ staging
-    const int m = tid & 127, h = tid >> 7;
-    const long long v = v0 + m;
-    const bool vin = v < nv;
-    const int vx = (int)(v % n), vy = (int)((v / n) % n), vz = (int)(v / ((long long)n * n));
-    const float* xb = x + (long long)b * Ci * nv;
-    bool ok = true;
-    for (int st = 0; st < nsteps && ok; ++st) {
-      const int s = st % CV_STAGES;
-      const uint32_t par = (uint32_t)((st / CV_STAGES) & 1);
-      if (!ptx::mbar_wait_or_abort(ptx::smem_u32(&b_empty[s]), par ^ 1u, abort)) { ok = false; break; }
-      const int kc = st / taps, t = st % taps;
-      int ox = 0, oy = 0, oz = 0;
-      if (ks == 3) { ox = t % 3 - 1; oy = (t / 3) % 3 - 1; oz = t / 9 - 1; }
-      const int sx = vx + ox, sy = vy + oy, sz = vz + oz;
-      const bool in = vin && sx >= 0 && sx < n && sy >= 0 && sy < n && sz >= 0 && sz < n;
-      const long long off = ((long long)sz * n + sy) * n + sx;
-      float xv[8];
+    // B: per tap [Np][16] in K-major core matrices (row co: 8 channels of half h at h 128 +
+    // (co / 8) 256 + (co % 8) 16).  A thread collects 16-byte rows, the 8 loads of two in flight;
+    // consecutive lanes take consecutive taps, which are contiguous in w.
+    for (int i0 = tid; i0 < a.Np * (2 * TPS); i0 += 2 * CV_THREADS) {
+      uint16_t e[2][8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        xv[j] = in ? __ldg(xb + (long long)(kc * 16 + h * 8 + j) * nv + off) : 0.f;
-      uint32_t hw[4], lw[4];
+      for (int u = 0; u < 2; ++u) {
+        const int i = i0 + u * CV_THREADS, t = i % TPS, ch = i / TPS, co = ch >> 1;
+        const bool in = co < a.Co && i < a.Np * (2 * TPS);
+        const uint16_t* p = reinterpret_cast<const uint16_t*>(a.w) +
+                            (in ? ((size_t)co * a.Ci + kc * 16 + (ch & 1) * 8) * a.taps + ph * TPS + t : 0);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const __nv_bfloat162 hb = __floats2bfloat162_rn(xv[2 * j], xv[2 * j + 1]);
-        const float2 hf = __bfloat1622float2(hb);
-        hw[j] = *reinterpret_cast<const uint32_t*>(&hb);
-        lw[j] = pack_bf2(xv[2 * j] - hf.x, xv[2 * j + 1] - hf.y);
+        for (int j = 0; j < 8; ++j) e[u][j] = in ? __ldg(p + j * a.taps) : (uint16_t)0;
       }
-      uint8_t* stg = cv_smem + s * sb;
-      *reinterpret_cast<uint4*>(stg + cv_kmaj(m, 8 * h)) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-      *reinterpret_cast<uint4*>(stg + CV_ABYTES + cv_kmaj(m, 8 * h)) =
-          make_uint4(lw[0], lw[1], lw[2], lw[3]);
-      // weight slice: row co, k = 16 channels of group kc at tap t (zero rows past Co)
-      uint8_t* bs = stg + 2 * CV_ABYTES;
-      for (int r = tid; r < Np * 2; r += 256) {
-        const int co = r >> 1, hh = r & 1;
-        uint16_t e[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const __nv_bfloat16 wv = co < Co ? w[((long long)co * Ci + kc * 16 + hh * 8 + j) * taps + t]
-                                           : __float2bfloat16_rn(0.f);
-          e[j] = *reinterpret_cast<const uint16_t*>(&wv);
+      for (int u = 0; u < 2; ++u) {
+        const int i = i0 + u * CV_THREADS, t = i % TPS, ch = i / TPS, co = ch >> 1;
+        if (i < a.Np * (2 * TPS))
+          *reinterpret_cast<uint4*>(bsm + (size_t)t * a.Np * 32 + (ch & 1) * 128 + (co >> 3) * 256 +
+                                    (co & 7) * 16) =
+              make_uint4(e[u][0] | (uint32_t)e[u][1] << 16, e[u][2] | (uint32_t)e[u][3] << 16,
+                         e[u][4] | (uint32_t)e[u][5] << 16, e[u][6] | (uint32_t)e[u][7] << 16);
+      }
+    }
+    // A: [hi, lo][8-channel half][plane][position] of 16 bytes; a thread takes all 16 channels of a
+    // position, 16 loads in flight
+    const float* xb = a.x + ((size_t)b * a.Ci + kc * 16) * nv;
+    for (int i = tid; i < span; i += CV_THREADS) {
+      const int sp = PL == 1 ? 0 : quot(i, a.L, a.mL);
+      const int o = voxel_at(first + sp * P * P + (i - sp * a.L));
+      const float* p = xb + (o < 0 ? 0 : o);
+      float v[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = o >= 0 ? __ldg(p + (size_t)j * nv) : 0.f;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t hw[4], lw[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float f0 = v[8 * h + 2 * j], f1 = v[8 * h + 2 * j + 1];
+          hw[j] = pack_bf2(f0, f1);
+          lw[j] = pack_bf2(f0 - __uint_as_float(hw[j] << 16), f1 - __uint_as_float(hw[j] & 0xffff0000u));
         }
-        *reinterpret_cast<uint4*>(bs + cv_kmaj(co, 8 * hh)) =
-            make_uint4(e[0] | ((uint32_t)e[1] << 16), e[2] | ((uint32_t)e[3] << 16),
-                       e[4] | ((uint32_t)e[5] << 16), e[6] | ((uint32_t)e[7] << 16));
+        *reinterpret_cast<uint4*>(cv_sm + (size_t)(h * span + i) * 16) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+        *reinterpret_cast<uint4*>(cv_sm + (size_t)((2 + h) * span + i) * 16) =
+            make_uint4(lw[0], lw[1], lw[2], lw[3]);
       }
-      ptx::fence_proxy_async_smem();
-      ptx::mbar_arrive(ptx::smem_u32(&b_full[s]));
     }
-    // ------------------------------------------------------------ epilogue
-    const bool done = ok && ptx::mbar_wait_or_abort(ptx::smem_u32(&b_done), 0u, abort);
-    if (!done && warp < 4) {
-      // a wait gave up: the tile's outputs are marked invalid (NaN) besides the error flag
-      const long long vo = v0 + q_of(warp) * 32 + lane;
-      if (vo < nv)
-        for (int co = 0; co < Co; ++co) y[((long long)b * Co + co) * nv + vo] = __int_as_float(0x7fc00000);
-    }
-    if (done) {
+    ptx::fence_proxy_async_smem();
+    __syncthreads();
+    // ------------------------------------------------------------ products of the channel group
+    if (tid == 0) {
       ptx::tc_fence_after();
-      const int q = warp & 3, half = warp >> 2;
-      const int nch = Np / 16, hc = (nch + 1) / 2;
-      const int cb = half ? hc : 0, ce = half ? nch : hc;
-      const long long vo = v0 + q * 32 + lane;
-      for (int c = cb; c < ce; ++c) {
-        float acc[16];
-        ptx::tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(c * 16), acc);
-        if (vo < nv) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int co = c * 16 + j;
-            if (co < Co) {
-              float* o = y + ((long long)b * Co + co) * nv + vo;
-              float r = acc[j] + (bias ? bias[co] : 0.f);
-              if (accumulate) r += *o;
-              if (relu) r = fmaxf(r, 0.f);
-              *o = r;
-            }
-          }
+      const uint32_t id = ptx::idesc_bf16(128, a.Np);
+      const uint32_t sa = ptx::smem_u32(cv_sm), sb = ptx::smem_u32(bsm);
+      const uint64_t dA = ptx::smem_desc(sa, (uint32_t)span * 16u, 128);
+      const uint64_t dB = ptx::smem_desc(sb, 128, 256);
+      const uint32_t lo = 2u * (uint32_t)span;            // 16-byte units to the lo halves
+      for (int t = 0; t < TPS; ++t) {
+        // the tap's first row and its weights, in 16-byte units
+        const int ox = t % 3, oy = t / 3 % 3, oz = t / 9;
+        const uint64_t at = dA + (uint32_t)(oz * a.L + oy * P + ox), bt = dB + (uint32_t)(t * 2 * a.Np);
+        for (int m = 0; m < a.T; ++m) {
+          const uint32_t d = tmem + (uint32_t)(m * a.Np);
+          const uint64_t am = at + 128u * (uint32_t)m;
+          ptx::mma_bf16(d, am, bt, id, (st | t) ? 1u : 0u);
+          ptx::mma_bf16(d, am + lo, bt, id, 1u);
         }
       }
-      ptx::tc_fence_before();
+      ptx::mma_commit(ptx::smem_u32(&b_done));
     }
-  } else if (lane == 0) {
-    // ------------------------------------------------------------ MMA issuer
-    const uint32_t id = ptx::idesc_bf16(128, Np);
-    const uint32_t base = ptx::smem_u32(cv_smem);
-    int st = 0;
-    for (; st < nsteps; ++st) {
-      const int s = st % CV_STAGES;
-      if (!ptx::mbar_wait_or_abort(ptx::smem_u32(&b_full[s]), (uint32_t)((st / CV_STAGES) & 1), abort))
-        break;
-      ptx::tc_fence_after();
-      const uint32_t sa = base + (uint32_t)(s * sb);
-      const uint64_t dAh = ptx::smem_desc(sa, 128, 256), dAl = ptx::smem_desc(sa + CV_ABYTES, 128, 256);
-      const uint64_t dB = ptx::smem_desc(sa + 2 * CV_ABYTES, 128, 256);
-      ptx::mma_bf16(tmem, dAh, dB, id, st > 0 ? 1u : 0u);
-      ptx::mma_bf16(tmem, dAl, dB, id, 1u);
-      ptx::mma_commit(ptx::smem_u32(&b_empty[s]));
-    }
-    ptx::mma_commit(ptx::smem_u32(&b_done));
+    ok = ptx::mbar_wait(ptx::smem_u32(&b_done), (uint32_t)(st & 1));
+    ok = __syncthreads_and(ok);
   }
-  // ------------------------------------------------------------ teardown
+  ptx::tc_fence_after();
+  // ------------------------------------------------------------ epilogue
+  // warp w reads TMEM lanes 32 (w % 4)..; the two halves of the warps take alternate 16-column chunks
+  const int q = warp & 3, half = warp >> 2, nch = a.Np / 16;
+  for (int m = 0; m < a.T; ++m) {
+    const int p = p0 + m * 128 + q * 32 + lane;
+    const int vo = p <= a.p_hi ? voxel_at(p) : -1;
+    for (int c = half; c < nch; c += 2) {
+      float acc[16];
+      if (ok) {
+        ptx::tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(m * a.Np + c * 16), acc);
+      } else {
+        // a wait gave up: the outputs are marked invalid besides the error flag
+#pragma unroll
+        for (int j = 0; j < 16; ++j) acc[j] = __int_as_float(0x7fc00000);
+      }
+      if (vo < 0) continue;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const int co = c * 16 + j;
+        if (co < a.Co) {
+          float* o = a.y + ((size_t)b * a.Co + co) * nv + vo;
+          float r = acc[j] + (a.bias ? __ldg(a.bias + co) : 0.f);
+          if (a.accumulate) r += *o;
+          if (a.relu && ok) r = fmaxf(r, 0.f);
+          *o = r;
+        }
+      }
+    }
+  }
+  ptx::tc_fence_before();
   __syncthreads();
-  if (warp == 8) {
-    if (lane == 0) {
-      // all MMAs of this CTA have completed before TMEM is freed
-      if (!ptx::mbar_wait(ptx::smem_u32(&b_done), 0u)) abort_sh = 1;
+  // the products of an abandoned wait have finished (or are given another bounded wait) before TMEM
+  // is freed
+  if (warp == 0) {
+    if (!ok && lane == 0) {
+      ptx::mbar_wait(ptx::smem_u32(&b_done), 0u);
+      if (a.err) atomicExch(a.err, 3);
     }
     __syncwarp();
     ptx::tc_fence_after();
-    ptx::tmem_dealloc(tmem, (uint32_t)tcols);
+    ptx::tmem_dealloc(tmem, (uint32_t)a.tcols);
   }
-  __syncthreads();
-  if (tid == 0 && abort_sh && err) atomicExch(err, 3);
 }
 
 }  // namespace
 
-bool conv_tc_supported(int Ci, int Co) { return Ci % 16 == 0 && Co >= 1 && Co <= 256; }
+// (positions with the border are 32-bit: n up to 1288)
+bool conv_tc_supported(int Ci, int Co, int n) {
+  return Ci % 16 == 0 && Co >= 1 && Co <= 256 && n <= 1280;
+}
 
 // Device flag a tensor-core convolution sets when one of its bounded waits gave up (its tile's
 // outputs are then NaN); allocated once per process.
@@ -215,24 +240,61 @@ static int* conv_err_flag() {
   return f;
 }
 
+template <int TPS>
+static cudaError_t launch_conv(const ConvArgs& a, int B, cudaStream_t s) {
+  static const cudaError_t set = cudaFuncSetAttribute(
+      k_conv_tc<TPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, CV_SMEM_CAP);
+  if (set != cudaSuccess) return set;
+  const int rows = a.p_hi - a.p_lo + 1, per = 128 * a.T;
+  const dim3 grid((unsigned)((rows + per - 1) / per), (unsigned)B);
+  k_conv_tc<TPS><<<grid, CV_THREADS, cv_smem(TPS == 27 ? 3 : 1, a.L, TPS, a.Np), s>>>(a);
+  return cudaGetLastError();
+}
+
 cudaError_t conv_tc_fwd(const float* x, const void* w, const float* bias, float* y, int B, int Ci,
                         int Co, int n, int ks, int relu, int accumulate, cudaStream_t s) {
-  int* err = conv_err_flag();
-  const int Np = (Co + 15) / 16 * 16;
-  int tcols = 32;
-  while (tcols < Np) tcols <<= 1;
-  const int smem = CV_STAGES * cv_stage_bytes(Np);
-  static int limit = 0;   // only ever raised (a recorded launch may need more than this one)
-  if (smem > limit) {
-    cudaError_t e = cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    limit = smem;
+  ConvArgs a{};
+  a.x = x; a.w = (const __nv_bfloat16*)w; a.bias = bias; a.y = y;
+  a.Ci = Ci; a.Co = Co; a.n = n;
+  a.Np = (Co + 15) / 16 * 16;
+  a.taps = ks * ks * ks;
+  a.pad = ks / 2;
+  a.P = n + 2 * a.pad;
+  a.relu = relu; a.accumulate = accumulate;
+  a.err = conv_err_flag();
+  a.p_lo = a.pad * (a.P * a.P + a.P + 1);
+  a.p_hi = (n - 1 + a.pad) * (a.P * a.P + a.P + 1);
+  const int halo = a.pad ? 2 * a.P + 2 : 0;
+  // Row tiles per CTA: the more, the fewer border positions are staged twice (1.35 a row with three
+  // at 64^3, 2.05 with one), as long as two CTAs fit an SM (115,000 bytes, 256 TMEM columns each)
+  // and there are two for every SM; all taps of a channel group in one step, else plane by plane
+  // (wide layers, and grids past 380^3).
+  const int64_t rows = (int64_t)(a.p_hi - a.p_lo + 1) * B;
+  const auto fits = [&](int T, int nph, int cap) {
+    const int L = 128 * T + halo;
+    return T * a.Np <= 256 && (ks == 1 ? 64 * L + a.Np * 32 : cv_smem(3 / nph, L, 27 / nph, a.Np)) <= cap;
+  };
+  a.T = 1;
+  a.nph = 1;
+  bool found = false;
+  for (int T = 3; T >= 1 && !found; --T)
+    if ((T == 1 || rows >= (int64_t)128 * T * 304) && fits(T, 1, 115000)) {
+      a.T = T;
+      found = true;
+    }
+  if (!found && !fits(1, 1, CV_SMEM_CAP)) {
+    a.nph = 3;
+    if (ks == 1 || !fits(1, 3, CV_SMEM_CAP)) return cudaErrorInvalidValue;
   }
-  const long long nv = (long long)n * n * n;
-  dim3 grid((unsigned)((nv + 127) / 128), (unsigned)B);
-  k_conv_tc<<<grid, CV_THREADS, smem, s>>>(x, (const __nv_bfloat16*)w, bias, y, Ci, Co, Np, n, ks,
-                                           relu, accumulate, tcols, err);
-  return cudaGetLastError();
+  a.L = 128 * a.T + halo;
+  // positions stay below 2 P^3 and staged ones below 2^16: where the reciprocals are exact
+  const auto recip = [](unsigned d) { return (unsigned)(((1ull << 32) + d - 1) / d); };
+  a.mP = a.P > 1 && a.P <= 200 ? recip(a.P) : 0u;
+  a.mL = recip(a.L);
+  a.tcols = 32;
+  while (a.tcols < a.T * a.Np) a.tcols <<= 1;
+  if (ks == 1) return launch_conv<1>(a, B, s);
+  return a.nph == 1 ? launch_conv<27>(a, B, s) : launch_conv<9>(a, B, s);
 }
 
 }  // namespace lddmm

@@ -514,14 +514,14 @@ static inline int gs(int64_t n) {
 
 static int tiles_of(int n) { return ((n + BX - 1) / BX) * ((n + BY - 1) / BY) * ((n + BZ - 1) / BZ); }
 
-bool conv_tc_supported(int Ci, int Co);
+bool conv_tc_supported(int Ci, int Co, int n);
 cudaError_t conv_tc_fwd(const float* x, const void* w, const float* bias, float* y, int B, int Ci,
                         int Co, int n, int ks, int relu, int accumulate, cudaStream_t s);
 
 cudaError_t net_conv_fwd(const float* x, const void* w, const float* bias, float* y, int B, int Ci,
                          int Co, int n, int ks, int relu, int accumulate, cudaStream_t s) {
   // input channels in groups of 16: the tensor-core implicit GEMM (kernels_conv_tc.cu)
-  if (conv_tc_supported(Ci, Co))
+  if (conv_tc_supported(Ci, Co, n))
     return conv_tc_fwd(x, w, bias, y, B, Ci, Co, n, ks, relu, accumulate, s);
   dim3 grid(tiles_of(n), (Co + CT - 1) / CT, B);
   k_conv_fwd<<<grid, NTV, 0, s>>>(x, (const __nv_bfloat16*)w, bias, y, Ci, Co, n, ks, relu,
