@@ -122,23 +122,26 @@ __global__ void k_transpose_flip(const __nv_bfloat16* __restrict__ w, __nv_bfloa
 // tile); part[g][co][ci][t] holds its end, and k_wgrad_reduce adds the groups in order.  No
 // floating-point atomics, the same bits on every run and for every shape of the block.
 // It is a product of Co x B n^3 by B n^3 x 27 Ci in FP32 (274 GFLOP in a training step at 64^3,
-// batch 8), so the FP32 pipes bound it and everything else has to stay off their issue slots.  A
-// block owns 16 output channels x CIT input channels of one group; it stages a unit's x (with halo,
-// [voxel][ci], rows of CIT + 1 words: conflict free both ways) and dy ([voxel][16 co], 16-byte quads
-// swizzled by voxel) by 4-byte asynchronous copies into two buffers, the next unit's under the
-// products of this one.  A thread owns one input channel, one dz and 2 output channels: it walks
-// the tile's 32 rows with a 3 x 3 window of x in registers, so a voxel costs 3 + 1 shared loads at
-// constant offsets for 18 FMAs.  The step's 14 such gradients take 8.2 ms; with one (co, tap) per
-// thread and two shared loads per FMA they took 57.
+// batch 8: 3.4 ms), so the FP32 pipes bound it and everything else has to stay off their issue
+// slots.  A block owns 16 output channels x CIT input channels of one group; it stages a unit's x
+// (with halo, [voxel][ci], rows of CIT + 1 words: conflict free both ways) and dy ([channel pair]
+// [voxel][2]) by 4-byte asynchronous copies into two buffers, the next unit's under the products of
+// this one.  A thread owns one input channel, one dz and 2 output channels: it walks the tile's rows
+// with three rows of x in registers, so a voxel costs 1.6 + 0.5 shared loads at constant offsets for
+// 18 FMAs.  The step's 14 such gradients take 6.3 ms: 6.8 with all positions decoded for every unit
+// and dy read a voxel at a time, 8.3 with 3 loads of x per voxel, 57 with one (co, tap) per thread
+// and two shared loads per FMA.  What is left: the partition leaves up to 24 SMs without a block,
+// and a sixth of the issue slots stage.
+constexpr int WG_DS = NTV * 2 + 4, WG_DY = CT / 2 * WG_DS;   // words of a channel pair of dy, of all
 constexpr int WG_CPT = 2, WG_HX = BX + 2, WG_HXY = (BX + 2) * (BY + 2), WG_HV = WG_HXY * (BZ + 2);
 __host__ __device__ constexpr int wg_threads(int cit) { return (cit * 3 * (CT / WG_CPT) + 31) / 32 * 32; }
-__host__ __device__ constexpr int wg_words(int cit) { return NTV * CT + WG_HV * (cit + 1); }
+__host__ __device__ constexpr int wg_words(int cit) { return WG_DY + WG_HV * (cit + 1); }
 
-// 4 bytes to shared memory, asynchronously; zeros when !in (the address is then not read)
-__device__ __forceinline__ void cp4(float* dst, const float* src, bool in) {
+// 4 bytes to shared memory, asynchronously; zeros when len = 0 (the address is then not read)
+__device__ __forceinline__ void cp4(float* dst, const float* src, int len) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
                    (uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src), "r"(in ? 4 : 0)
+               "l"(src), "r"(len)
                : "memory");
 }
 
@@ -161,82 +164,131 @@ __global__ void __launch_bounds__(wg_threads(CIT), 1) k_wgrad3(const float* __re
   for (int c = 0; c < WG_CPT; ++c)
 #pragma unroll
     for (int t = 0; t < 9; ++t) s[c][t] = 0.f;
-  auto stage = [&](int u, float* dys) {
-    float* xs = dys + NTV * CT;
-    const int b = u / tiles, tile = u - b * tiles;
-    const int tx0 = (tile % ntx) * BX, ty0 = ((tile / ntx) % nty) * BY, tz0 = (tile / (ntx * nty)) * BZ;
-    // A warp takes the channels w % CG, + CG, ..; a lane's position is decoded once for all of them.
-    // Addresses are clamped into the tensor, what lies outside the grid arrives as zero.
-    constexpr int CG = NW >= 4 && CIT >= 4 ? 4 : 1, PG = NW / CG;
-    const float* xb = x + ((size_t)b * Ci + ci0) * nv;
-    const int cw = warp % CG, cmax = Ci - 1 - ci0;
-    for (int e = (warp / CG) * 32 + lane; e < WG_HV; e += PG * 32) {
-      const int hz = e / WG_HXY, r = e - hz * WG_HXY, hy = r / WG_HX, hx = r - hy * WG_HX;
-      const int gx = tx0 + hx - 1, gy = ty0 + hy - 1, gz = tz0 + hz - 1;
-      const bool in = gx >= 0 && gx < n && gy >= 0 && gy < n && gz >= 0 && gz < n;
-      const float* p = xb + (in ? ((size_t)gz * n + gy) * n + gx : 0);
-      float* d = xs + e * XS + cw;
+  // Staging.  A warp takes the channels w % CG, + CG, .. of the positions of its lanes.  What only
+  // depends on the thread is kept: a position's offset from the tile's first voxel, and a bit for its
+  // place along each axis, which the unit's mask of places outside the grid is tested against.
+  // Addresses are clamped into the tensor, what lies outside the grid arrives as zero.
+  constexpr int CG = NW < 4 ? 1 : NW % 4 == 0 ? 4 : 2, PG = NW / CG, XP = (WG_HV + PG * 32 - 1) / (PG * 32);
+  constexpr int DP = (NTV + PG * 32 - 1) / (PG * 32);
+  static_assert(NW % CG == 0 && CIT % CG == 0, "every warp stages");
+  const int cw = warp % CG, cmax = Ci - 1 - ci0, omax = Co - 1 - co0;
+  const int e0 = (warp / CG) * 32 + lane;
+  int xrel[XP], drel[DP];
+  unsigned xbit[XP], dbit[DP];
+  auto place = [&](int hx, int hy, int hz, int& rel, unsigned& bit) {
+    rel = ((hz - 1) * n + hy - 1) * n + hx - 1;
+    bit = 1u << hx | 1u << (WG_HX + hy) | 1u << (WG_HX + BY + 2 + hz);
+  };
 #pragma unroll
-      for (int k = 0; k < CIT / CG; ++k) {
-        const int c = cw + k * CG;
-        cp4(d + k * CG, p + (size_t)min(c, cmax) * nv, in && c <= cmax);
-      }
+  for (int k = 0; k < XP; ++k) {
+    const int e = e0 + k * PG * 32, r = e % WG_HXY;
+    place(r % WG_HX, r / WG_HX, min(e / WG_HXY, BZ + 1), xrel[k], xbit[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < DP; ++k) {
+    const int v = e0 + k * PG * 32;
+    place(v % BX + 1, v / BX % BY + 1, min(v / (BX * BY), BZ - 1) + 1, drel[k], dbit[k]);
+  }
+  const int units = tiles * B;
+  // tile of the next unit to stage, and the step to the one after
+  int tx = blockIdx.x % ntx, ty = blockIdx.x / ntx % nty, tz = blockIdx.x / (ntx * nty) % ntz, b = blockIdx.x / tiles;
+  const int gx = G % ntx, gy = G / ntx % nty, gz = G / (ntx * nty) % ntz, gb = G / tiles;
+  auto stage = [&](float* dys) {
+    float* const xs = dys + WG_DY;
+    const int x0 = tx * BX, y0 = ty * BY, z0 = tz * BZ;
+    // places with no voxel: the first along an axis at its near face, those past n at the far one
+    auto outside = [&](int o, int len) {
+      const unsigned far = n - o + 1 < len ? ~0u << (n - o + 1) & ((1u << len) - 1) : 0u;
+      return far | (o == 0 ? 1u : 0u);
+    };
+    const unsigned mask = outside(x0, WG_HX) | outside(y0, BY + 2) << WG_HX |
+                          outside(z0, BZ + 2) << (WG_HX + BY + 2);
+    const size_t o = ((size_t)z0 * n + y0) * n + x0;
+    const float* const xb = x + ((size_t)b * Ci + ci0) * nv + o;
+    const float* const db = dy + ((size_t)b * Co + co0) * nv + o;
+    int off[XP], len[XP];
+#pragma unroll
+    for (int k = 0; k < XP; ++k) {
+      const bool in = !(xbit[k] & mask);
+      off[k] = in ? xrel[k] : 0;
+      len[k] = in ? 4 : 0;
     }
-    constexpr int DG = NW >= 4 ? 4 : 1;
-    const float* dyb = dy + ((size_t)b * Co + co0) * nv;
-    const int gw = warp % DG, omax = Co - 1 - co0;
-    for (int v = (warp / DG) * 32 + lane; v < NTV; v += NW / DG * 32) {
-      const int gx = tx0 + v % BX, gy = ty0 + v / BX % BY, gz = tz0 + v / (BX * BY);
-      const bool in = gx < n && gy < n && gz < n;
-      const float* p = dyb + (in ? ((size_t)gz * n + gy) * n + gx : 0);
-      const int sw = (v >> 1) & 3;
 #pragma unroll
-      for (int k = 0; k < CT / DG; ++k) {
-        const int c = gw + DG * k;
-        cp4(dys + v * CT + (((c >> 2) ^ sw) << 2) + (c & 3), p + (size_t)min(c, omax) * nv, in && c <= omax);
-      }
+    for (int j = 0; j < CIT / CG; ++j) {
+      const int c = cw + j * CG;
+      const float* const p = xb + (size_t)min(c, cmax) * nv;
+#pragma unroll
+      for (int k = 0; k < XP; ++k)
+        if (k < XP - 1 || e0 + k * PG * 32 < WG_HV)
+          cp4(xs + (e0 + k * PG * 32) * XS + c, p + off[k], c <= cmax ? len[k] : 0);
+    }
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+      const bool in = !(dbit[k] & mask);
+      off[k] = in ? drel[k] : 0;
+      len[k] = in ? 4 : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < CT / CG; ++j) {
+      const int c = cw + j * CG;
+      const float* const p = db + (size_t)min(c, omax) * nv;
+#pragma unroll
+      for (int k = 0; k < DP; ++k)
+        if (k < DP - 1 || e0 + k * PG * 32 < NTV)
+          cp4(dys + (c >> 1) * WG_DS + (e0 + k * PG * 32) * 2 + (c & 1), p + off[k], c <= omax ? len[k] : 0);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+    tx += gx;
+    ty += gy;
+    tz += gz;
+    b += gb;
+    if (tx >= ntx) { tx -= ntx; ++ty; }
+    if (ty >= nty) { ty -= nty; ++tz; }
+    if (tz >= ntz) { tz -= ntz; ++b; }
   };
-  const int units = tiles * B;
   int buf = 0;
-  if ((int)blockIdx.x < units) stage(blockIdx.x, wg_smem);
+  if ((int)blockIdx.x < units) stage(wg_smem);
   for (int u = blockIdx.x; u < units; u += G, buf ^= 1) {
     const float* dys = wg_smem + buf * wg_words(CIT);
-    const float* xs = dys + NTV * CT;
+    const float* xs = dys + WG_DY;
     if (u + G < units) {
-      stage(u + G, wg_smem + (buf ^ 1) * wg_words(CIT));
+      stage(wg_smem + (buf ^ 1) * wg_words(CIT));
       asm volatile("cp.async.wait_group 1;" ::: "memory");
     } else {
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
     __syncthreads();
     if (dz < 3) {
-      const int q = cog * WG_CPT >> 2, qo = cog * WG_CPT & 3;   // the thread's quad of dy, place in it
-      for (int r = 0; r < BY * BZ; ++r) {
-        const float* xr = xs + (((r / BY + dz) * (BY + 2) + r % BY) * WG_HX) * XS + ci;
-        const float* dr = dys + r * BX * CT + qo;
-        float w[3][3];
+      // rows of x stay in registers while they are in reach: row y + 1 is read in place of row y - 2
+      for (int lz = 0; lz < BZ; ++lz) {
+        const float* xr = xs + (lz + dz) * WG_HXY * XS + ci;
+        const float* dr = dys + cog * WG_DS + lz * BY * BX * 2;
+        float w[3][WG_HX];
 #pragma unroll
-        for (int d = 0; d < 3; ++d)
+        for (int d = 0; d < 2; ++d)
 #pragma unroll
-          for (int e = 0; e < 2; ++e) w[d][e] = xr[(d * WG_HX + e) * XS];
+          for (int e = 0; e < WG_HX; ++e) w[d][e] = xr[(d * WG_HX + e) * XS];
 #pragma unroll
-        for (int lx = 0; lx < BX; ++lx) {
+        for (int ly = 0; ly < BY; ++ly) {
 #pragma unroll
-          for (int d = 0; d < 3; ++d) w[d][2] = xr[(d * WG_HX + lx + 2) * XS];
-          const float2 g = *reinterpret_cast<const float2*>(dr + lx * CT + ((q ^ ((lx >> 1) & 3)) << 2));
+          for (int e = 0; e < WG_HX; ++e) w[(ly + 2) % 3][e] = xr[((ly + 2) * WG_HX + e) * XS];
 #pragma unroll
-          for (int d = 0; d < 3; ++d)
+          for (int lx = 0; lx < BX; lx += 2) {
+            const float4 g = *reinterpret_cast<const float4*>(dr + (ly * BX + lx) * 2);
 #pragma unroll
-            for (int e = 0; e < 3; ++e) {
-              s[0][d * 3 + e] = fmaf(g.x, w[d][e], s[0][d * 3 + e]);
-              s[1][d * 3 + e] = fmaf(g.y, w[d][e], s[1][d * 3 + e]);
-            }
+            for (int d = 0; d < 3; ++d)
 #pragma unroll
-          for (int d = 0; d < 3; ++d) {
-            w[d][0] = w[d][1];
-            w[d][1] = w[d][2];
+              for (int e = 0; e < 3; ++e) {
+                s[0][d * 3 + e] = fmaf(g.x, w[(ly + d) % 3][lx + e], s[0][d * 3 + e]);
+                s[1][d * 3 + e] = fmaf(g.y, w[(ly + d) % 3][lx + e], s[1][d * 3 + e]);
+              }
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+#pragma unroll
+              for (int e = 0; e < 3; ++e) {
+                s[0][d * 3 + e] = fmaf(g.z, w[(ly + d) % 3][lx + 1 + e], s[0][d * 3 + e]);
+                s[1][d * 3 + e] = fmaf(g.w, w[(ly + d) % 3][lx + 1 + e], s[1][d * 3 + e]);
+              }
           }
         }
       }
@@ -279,8 +331,8 @@ __global__ void __launch_bounds__(256, 1) k_wgrad1(const float* __restrict__ x,
     const size_t o = in ? ((size_t)gz * n + gy) * n + gx : 0;
     const float* xb = x + ((size_t)b * Ci + ci0) * nv + o;
     const float* db = dy + ((size_t)b * Co + co0) * nv + o;
-    for (int c = 0; c < ni; ++c) cp4(xs + tid * S1 + c, xb + (size_t)c * nv, in);
-    for (int c = 0; c < no; ++c) cp4(xs + HALF + tid * S1 + c, db + (size_t)c * nv, in);
+    for (int c = 0; c < ni; ++c) cp4(xs + tid * S1 + c, xb + (size_t)c * nv, in ? 4 : 0);
+    for (int c = 0; c < no; ++c) cp4(xs + HALF + tid * S1 + c, db + (size_t)c * nv, in ? 4 : 0);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   const int ci = tid & 15, co = tid >> 4;
