@@ -174,6 +174,24 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
       ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// 1 in one lane of a converged warp, 0 in the others.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.b32 %0, 1, 0, e;\n\t}" : "=r"(r));
+  return r;
+}
+// mma_bf16 by the elected lane, written for a whole converged warp: its operands stay in uniform
+// registers (40 cycles a product where a branch to one thread takes 50).
+__device__ __forceinline__ void mma_bf16_one(uint32_t elected, uint32_t d_tmem, uint64_t adesc,
+                                             uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\t"
+      "setp.ne.b32 e, %5, 0;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(elected)
+      : "memory");
+}
 // D[tmem] (+)= A[tmem] * B[smem]^T: A (M = 128 rows, 16 k) held in TMEM, row r in lane r, its
 // 16 bf16 packed two per 32-bit column in 8 consecutive columns from a_tmem (k even in the low
 // half).
