@@ -144,8 +144,8 @@ void launch_adj_init(const Grid& g, const float* uT, const float* I0, const floa
                      const float* M, float* gT, float scale, cudaStream_t s);
 void launch_adj_step(const Grid& g, const float* vj, const float* uj, const float* gnext,
                      float* gcur, float* gradj, float dtx, float dty, float dtz, cudaStream_t s);
-void launch_apply_L3(const Grid& g, const float* src, float* dst, float alpha, float gamma,
-                     float ihx2, float ihy2, float ihz2, float scale, bool accumulate,
+void launch_apply_L3(const Grid& g, const float* src, float* dst, float* clear, float alpha,
+                     float gamma, float ihx2, float ihy2, float ihz2, float scale, bool accumulate,
                      cudaStream_t s);
 
 // ---- smoothing operator K (kernels_dft.cu) ----

@@ -992,8 +992,8 @@ int lddmm_shoot(lddmm_ctx* ctx, const float* v0) {
   int rc;
   if ((rc = check_finite(ctx, v, F, "v0"))) return rc;
   // m_0 = L (L v_0) in stage
-  launch_apply_L3(g, v, ctx->work, ctx->p.alpha, ctx->p.gamma, ihx2, ihy2, ihz2, 1.0f, false, s);
-  launch_apply_L3(g, ctx->work, ctx->stage, ctx->p.alpha, ctx->p.gamma, ihx2, ihy2, ihz2, 1.0f,
+  launch_apply_L3(g, v, ctx->work, nullptr, ctx->p.alpha, ctx->p.gamma, ihx2, ihy2, ihz2, 1.0f, false, s);
+  launch_apply_L3(g, ctx->work, ctx->stage, nullptr, ctx->p.alpha, ctx->p.gamma, ihx2, ihy2, ihz2, 1.0f,
                   false, s);
   const float* uc = nullptr;
   int pf = 0;
@@ -1227,9 +1227,8 @@ int lddmm_energy_grad(lddmm_ctx* ctx, const float* v, float* grad, double* E) {
     if (j == T) return ctx->uall + (size_t)(nslots - 1) * F;
     return ctx->uall + (size_t)(j / c) * F;
   };
-  // forward sweep (energy, u_j kept or checkpointed)
+  // forward sweep (energy, u_j kept or checkpointed; u_0 = 0 is not stored)
   if ((rc = reset_acc(ctx))) return rc;
-  CK(cudaMemsetAsync(slot_of(0), 0, F * sizeof(float), s));
   launch_ereg(g, ctx->v, T, ctx->p.alpha, ctx->p.gamma, ihx2, ihy2, ihz2, ctx->acc, s, 0);
   const float* uc = nullptr;
   int pf = 0;
@@ -1250,6 +1249,7 @@ int lddmm_energy_grad(lddmm_ctx* ctx, const float* v, float* grad, double* E) {
   float* gnext = ctx->gA;
   float* gcur = ctx->gB;
   launch_adj_init(g, slot_of(T), L.I0, L.I1, L.M, gnext, (float)(2.0 * h3 / (sg * sg)), s);
+  CK(cudaMemsetAsync(gcur, 0, F * sizeof(float), s));
   int seg_base = -1;
   for (int j = T - 1; j >= 0; --j) {
     const float* uj;
@@ -1257,23 +1257,24 @@ int lddmm_energy_grad(lddmm_ctx* ctx, const float* v, float* grad, double* E) {
       uj = slot_of(j);
     } else {
       const int k = (j / c) * c;
-      if (seg_base != k) {   // recompute u_k .. u_{min(k+c,T)-1} from the checkpoint u_k
-        CK(cudaMemcpyAsync(ctx->seg, slot_of(k), F * sizeof(float), cudaMemcpyDeviceToDevice, s));
-        for (int i = 1; i < c && k + i < T; ++i)
-          launch_flow_only_fwd(g, ctx->v + (int64_t)(k + i - 1) * F, ctx->seg + (size_t)(i - 1) * F,
-                               ctx->seg + (size_t)i * F, dtx, dty, dtz, s, 0);
+      if (seg_base != k) {   // recompute u_{k+1} .. u_{min(k+c,T)-1} from the checkpoint u_k
+        const float* from = k ? slot_of(k) : nullptr;
+        for (int i = 1; i < c && k + i < T; ++i) {
+          float* to = ctx->seg + (size_t)(i - 1) * F;
+          launch_flow_only_fwd(g, ctx->v + (int64_t)(k + i - 1) * F, from, to, dtx, dty, dtz, s, 0);
+          from = to;
+        }
         seg_base = k;
       }
-      uj = ctx->seg + (size_t)(j - k) * F;
+      uj = j == k ? slot_of(k) : ctx->seg + (size_t)(j - k - 1) * F;
     }
     float* gradj = gout + (int64_t)j * F;
-    if (j > 0) CK(cudaMemsetAsync(gcur, 0, F * sizeof(float), s));
     launch_adj_step(g, ctx->v + (int64_t)j * F, j > 0 ? uj : nullptr, gnext, j > 0 ? gcur : nullptr,
                     gradj, dtx, dty, dtz, s);
-    // regulariser: + 2 dt h^3 L(L v_j)
-    launch_apply_L3(g, ctx->v + (int64_t)j * F, ctx->work, ctx->p.alpha, ctx->p.gamma, ihx2, ihy2,
-                    ihz2, 1.0f, false, s);
-    launch_apply_L3(g, ctx->work, gradj, ctx->p.alpha, ctx->p.gamma, ihx2, ihy2, ihz2,
+    // regulariser: + 2 dt h^3 L(L v_j); zeros for the sums of the next step
+    launch_apply_L3(g, ctx->v + (int64_t)j * F, ctx->work, j > 1 ? gnext : nullptr, ctx->p.alpha, ctx->p.gamma,
+                    ihx2, ihy2, ihz2, 1.0f, false, s);
+    launch_apply_L3(g, ctx->work, gradj, nullptr, ctx->p.alpha, ctx->p.gamma, ihx2, ihy2, ihz2,
                     (float)(2.0 * h3 / T), true, s);
     std::swap(gnext, gcur);
   }
