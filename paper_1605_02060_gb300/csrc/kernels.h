@@ -36,8 +36,9 @@ enum KernelId {
 // Velocity fields and images (vj, I0, I1, M) are stored as float (st = 0) or bf16 (st = 1);
 // displacements, J1, W, b and all arithmetic are float.  Maps (displacements) are planar,
 // [3][N], or, with quad = 1, [N] x (u_x, u_y, u_z, 0) (16 bytes a voxel): the iteration's
-// backward sweep (launch_flow_back) and the map phi_{0,1} it leaves use the quad layout, the
-// forward sweep (launch_fwd_fused) and phi_{1,0} the planar one.
+// backward sweep (launch_flow_back), the map phi_{0,1} it leaves and the steps of a forward sweep
+// without the residual use the quad layout, the iteration's forward sweep (launch_fwd_fused) and
+// phi_{1,0} the planar one.
 // Backward sweep step j (quad maps): u_cur = dt v_j / h + u_next(x + dt v_j / h)
 // (u_next == nullptr: id), then J1_j = I1 o phi, W_j = (M o phi) det(I + Du_cur), min det into
 // acc.  IM holds I1 and M interleaved as pairs (launch_interleave).
@@ -48,7 +49,8 @@ void launch_flow_back(const Grid& g, const void* vj, const float* u_next, float*
 void launch_interleave(const void* a, const void* b, void* out, int64_t n, cudaStream_t s,
                        int st);
 // Forward sweep step j: u_next = -dt v_j / h + u_cur(x - dt v_j / h) (u_cur == nullptr: id);
-// if last, J0_T = I0 o (id + u_next) and E_data.
+// if last, J0_T = I0 o (id + u_next) and E_data.  quad: u_cur and u_next in the quad layout, but
+// the last u_next planar.
 void launch_fwd_flow(const Grid& g, const void* vj, const float* u_cur, float* u_next,
                      float dtx, float dty, float dtz, bool last, const void* I0, const void* I1,
                      const void* M, float* J0T, Acc* acc, cudaStream_t s, int st, int rk = 0,
@@ -80,7 +82,9 @@ void launch_flow_only_back(const Grid& g, const void* vj, const float* u_next, f
 // A map in the quad layout ([N] x (u_x, u_y, u_z, 0), the iteration's sweeps) to the planar one
 // ([3][N]).
 void launch_quad_to_planar(const float* quad, float* planar, int64_t n, cudaStream_t s);
-void launch_warp(const Grid& g, const float* src, const float* u, float* dst, cudaStream_t s);
+// dst = src o (id + u), u planar or (quad = 1) in the quad layout; labels by nearest neighbour.
+void launch_warp(const Grid& g, const float* src, const float* u, float* dst, cudaStream_t s,
+                 int quad = 0);
 void launch_labels(const Grid& g, const uint16_t* L0, const float* u, uint16_t* dst,
                    cudaStream_t s);
 void launch_downsample(const Grid& fine, const Grid& coarse, int factor, const float* src,

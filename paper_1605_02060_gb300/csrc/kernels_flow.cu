@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(256) k_j0_edata_march(Grid g, const float* __r
 }
 
 // Forward sweep, last step: u_T = -dt v_{T-1}/h + u_cur(x - dt v_{T-1}/h), then J0_T = I0 o
-// (id + u_T) and E_data = sum M (J0_T - I1)^2.  Marches ZC planes per thread like k_disp_march
+// (id + u_T) and E_data = sum M (J0_T - I1)^2.  u_cur in layout Q, u_T planar.  Marches ZC planes per thread like k_disp_march
 // (the velocity of plane z+1 is loaded before plane z's lookups), so the three dependent
 // latencies of a voxel (v, the map at the displaced point, I0 at the mapped point) overlap with
 // the next plane's.
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(256) k_fwd_last_march(Grid g, const ST* __rest
         oy += r.y;
         oz += r.z;
       }
-      MapL<Q>::put(un, g.N, idx, ox, oy, oz);
+      MapL<false>::put(un, g.N, idx, ox, oy, oz);
       const float j0 = tri_apply_t(I0, tri_setup(g, (float)x + ox, (float)y + oy, (float)z + oz));
       J0T[idx] = j0;
       const float r = j0 - ldf(I1 + idx);
@@ -872,16 +872,35 @@ void launch_update(const Grid& g, void* vj, const float* Kb, float eps, cudaStre
 }
 
 // --------------------------------------------------------------------------------------------
-// Warp (trilinear pull-back) and label transfer (nearest neighbour, float32 rounding rule).
-__global__ void k_warp(Grid g, const float* __restrict__ src, const float* __restrict__ u,
-                       float* __restrict__ dst) {
-  int x, y, z, idx;
-  if (!voxel3d(g, x, y, z, idx)) return;
-  dst[idx] = tri_sample(src, g, (float)x + u[idx], (float)y + u[g.N + idx], (float)z + u[2 * g.N + idx]);
+// Warp (trilinear pull-back) and label transfer (nearest neighbour, float32 rounding rule).  A thread
+// marches ZC planes and asks for the map of the next before the lookup of this one; the march depth
+// is that of the flow steps.  264x160x228, a plane a thread before: warp 43 us (60), from a quad map
+// 45 (60 and 40 for a planar copy of it), labels 38 (57).
+template <bool Q, int ZC>
+__global__ void __launch_bounds__(256) k_warp(Grid g, const float* __restrict__ src,
+                                              const float* __restrict__ u, float* __restrict__ dst) {
+  const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
+  if (x >= g.nx || y >= g.ny) return;
+  const int z0 = blockIdx.z * ZC, z1 = min(z0 + ZC, g.nz), plane = g.nx * g.ny;
+  int idx = (z0 * g.ny + y) * g.nx + x;
+  float3 d = MapL<Q>::at(u, g.N, idx);
+  for (int z = z0; z < z1; ++z, idx += plane) {
+    const float3 dn = z + 1 < z1 ? MapL<Q>::at(u, g.N, idx + plane) : d;
+    dst[idx] = tri_sample(src, g, (float)x + d.x, (float)y + d.y, (float)z + d.z);
+    d = dn;
+  }
 }
 
-void launch_warp(const Grid& g, const float* src, const float* u, float* dst, cudaStream_t s) {
-  k_warp<<<grid3d(g), kBlock3d, 0, s>>>(g, src, u, dst);
+void launch_warp(const Grid& g, const float* src, const float* u, float* dst, cudaStream_t s, int quad) {
+  const bool one = flow_blocks(g) <= 256;
+  const dim3 grid = flow_grid(g, one ? 1 : kFlowZ);
+  if (quad) {
+    if (one) k_warp<true, 1><<<grid, kBlock3d, 0, s>>>(g, src, u, dst);
+    else k_warp<true, kFlowZ><<<grid, kBlock3d, 0, s>>>(g, src, u, dst);
+  } else {
+    if (one) k_warp<false, 1><<<grid, kBlock3d, 0, s>>>(g, src, u, dst);
+    else k_warp<false, kFlowZ><<<grid, kBlock3d, 0, s>>>(g, src, u, dst);
+  }
 }
 
 __device__ __forceinline__ int nn_index(float i, float u, int n) {
@@ -891,19 +910,30 @@ __device__ __forceinline__ int nn_index(float i, float u, int n) {
   return min(max(k, 0), n - 1);
 }
 
-__global__ void k_labels(Grid g, const uint16_t* __restrict__ L0, const float* __restrict__ u,
-                         uint16_t* __restrict__ dst) {
-  int x, y, z, idx;
-  if (!voxel3d(g, x, y, z, idx)) return;
-  const int ix = nn_index((float)x, u[idx], g.nx);
-  const int iy = nn_index((float)y, u[g.N + idx], g.ny);
-  const int iz = nn_index((float)z, u[2 * g.N + idx], g.nz);
-  dst[idx] = L0[(iz * g.ny + iy) * g.nx + ix];
+template <int ZC>
+__global__ void __launch_bounds__(256) k_labels(Grid g, const uint16_t* __restrict__ L0,
+                                                const float* __restrict__ u,
+                                                uint16_t* __restrict__ dst) {
+  const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
+  if (x >= g.nx || y >= g.ny) return;
+  const int z0 = blockIdx.z * ZC, z1 = min(z0 + ZC, g.nz), plane = g.nx * g.ny;
+  int idx = (z0 * g.ny + y) * g.nx + x;
+  float3 d = MapL<false>::at(u, g.N, idx);
+  for (int z = z0; z < z1; ++z, idx += plane) {
+    const float3 dn = z + 1 < z1 ? MapL<false>::at(u, g.N, idx + plane) : d;
+    const int ix = nn_index((float)x, d.x, g.nx), iy = nn_index((float)y, d.y, g.ny),
+              iz = nn_index((float)z, d.z, g.nz);
+    dst[idx] = __ldg(L0 + (iz * g.ny + iy) * g.nx + ix);
+    d = dn;
+  }
 }
 
 void launch_labels(const Grid& g, const uint16_t* L0, const float* u, uint16_t* dst,
                    cudaStream_t s) {
-  k_labels<<<grid3d(g), kBlock3d, 0, s>>>(g, L0, u, dst);
+  if (flow_blocks(g) <= 256)
+    k_labels<1><<<flow_grid(g, 1), kBlock3d, 0, s>>>(g, L0, u, dst);
+  else
+    k_labels<kFlowZ><<<flow_grid(g, kFlowZ), kBlock3d, 0, s>>>(g, L0, u, dst);
 }
 
 // --------------------------------------------------------------------------------------------

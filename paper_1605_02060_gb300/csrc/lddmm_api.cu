@@ -528,7 +528,7 @@ int refresh_maps(lddmm_ctx* ctx, bool energy) {
   for (int j = 0; j < T; ++j) {
     float* unx = ctx->uF[pf];
     launch_fwd_flow(g, vptr(ctx, j, N), uc, unx, dtx, dty, dtz, j == T - 1, L.I0, L.I1, L.M,
-                    ctx->J0T, ctx->acc, s, ctx->st, rk_of(ctx), 0);
+                    ctx->J0T, ctx->acc, s, ctx->st, rk_of(ctx), 1);
     uc = unx;
     pf ^= 1;
   }
@@ -540,7 +540,7 @@ int refresh_maps(lddmm_ctx* ctx, bool energy) {
 }
 
 // The iteration leaves phi_{0,1} in the quad layout (phi_{1,0} is planar); entry points that
-// read it (the inverse warp, landmarks, the map getter) take a planar copy in the K work buffer,
+// read it (landmarks, the map getter) take a planar copy in the K work buffer,
 // which is free between iterations.
 const float* planar_map(lddmm_ctx* ctx, const float* quad) {
   launch_quad_to_planar(quad, ctx->work, ctx->levels[ctx->cur].g.N, ctx->stream);
@@ -780,7 +780,7 @@ int lddmm_warp(lddmm_ctx* ctx, const float* src, float* dst, int direction) {
   if (rc) return rc;
   const bool dev = is_device_ptr(dst);
   float* d = dev ? dst : ctx->stage + g.N;
-  launch_warp(g, s, direction == 0 ? ctx->u10 : planar_map(ctx, ctx->u01), d, ctx->stream);
+  launch_warp(g, s, direction == 0 ? ctx->u10 : ctx->u01, d, ctx->stream, direction);
   CK(cudaGetLastError());
   if (!dev) return copy_out(ctx, dst, d, g.N * sizeof(float));
   return LDDMM_OK;
