@@ -168,10 +168,14 @@ void kplan_destroy(KPlan* kp) {
 // rows it copied into the other of two folded stages.  128 registers, four blocks of 4 warps (five
 // of 3) per SM: with prefetch through registers (167, 12 warps) a pass of 700 blocks left a second
 // wave of 100 and took 27 to 42 us.
-// At 132x80x114 (three components) the six passes take 36 + 19 + 28 + 21 + 17 + 37 us with the
-// update in the last (x lines are staged 4 bytes at a time, which sets their pace); as 64x64 tiles
-// of the unfolded product they took 6 x 53 us and the update 5.
+// At 132x80x114 (three components) the six passes take 31 + 18 + 28 + 19 + 16 + 33 us with the
+// update in the last; as 64x64 tiles of the unfolded product they took 6 x 53 us and the update 5.
+// What is left beside the FMAs is their issue: each stage's copies, folds and table tile are half of
+// the instructions of an x pass (two thirds with every place decoded anew: 36 and 37 us).  Where the
+// lines are whole 16-byte vectors x is copied as it lies, 5 vectors a line, and turned on the way to
+// the folded stage; else 4 bytes at a time.
 constexpr int FK = 8, FC = 128, FCS = FC + 4;   // rows per stage, columns per block, row stride
+constexpr int FX = 20;                          // floats of a line in a raw stage (x by vectors)
 
 struct FoldArgs {
   const float* in;
@@ -204,9 +208,11 @@ __global__ void __launch_bounds__(128, 4) k_fold(FoldArgs a) {
   const int tid = threadIdx.x, nt = blockDim.x;
   const int BP = 4 * a.tp, tabw = 2 * FK * BP;
   // forward: two raw stages, two folded ones; inverse: three stages used as they are; three tables
+  // (x lines by vectors: two raw stages of FX floats a line, two transposed ones)
+  const bool xv = XAX && a.vec;
   float* const raw = fs;
-  float* const eo = FWD ? fs + 2 * FE : fs;
-  float* const tab = fs + (FWD ? 4 : 3) * FE;
+  float* const eo = xv ? fs + 2 * FC * FX : FWD ? fs + 2 * FE : fs;
+  float* const tab = eo + (xv || FWD ? 2 : 3) * FE;
   const int tc = tid & 15, tp = tid >> 4;
   const int p0 = blockIdx.y * BP;
   const int c0 = blockIdx.x * FC;
@@ -240,6 +246,10 @@ __global__ void __launch_bounds__(128, 4) k_fold(FoldArgs a) {
       }
     }
   }
+  // x lines by vectors: the thread's vector xc of line xl, xl + xstep, .. (the last threads have none)
+  const int xstep = nt / (FX / 4), xc = tid % (FX / 4), xl = tid < xstep * (FX / 4) ? tid / (FX / 4) : FC;
+  // inverse tables: the thread's column ti and first row tk
+  const int tstep = nt / BP, ti = tid % BP, tk = tid / BP;
   auto cp = [&](float* dst, const float* src, bool in) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
                      (uint32_t)__cvta_generic_to_shared(dst)),
@@ -258,7 +268,18 @@ __global__ void __launch_bounds__(128, 4) k_fold(FoldArgs a) {
     if (k0 < H) {
       float* e = (FWD ? raw + (t & 1) * FE : eo + (t % 3) * FE);
       float* o = e + FK * FCS;
-      if constexpr (XAX) {
+      if (xv) {
+        // the aligned vectors of a line that hold the stage's elements: forward m = k0 .. k0 + 7 and
+        // n - k0 - 8 .. n - k0 + 3, inverse 2 k0 - 4 .. 2 k0 + 15
+        if (xl < FC) {
+          float* d = raw + (t & 1) * (FC * FX) + xl * FX + 4 * xc;
+          const int m = !FWD ? 2 * k0 - 4 + 4 * xc : xc < 2 ? k0 + 4 * xc : n - k0 - 16 + 4 * xc;
+          const bool in = m >= 0 && m < n;
+          int o = (c0 + xl) * n + m;
+          for (int l = xl; l < FC; l += xstep, d += xstep * FX, o += xstep * n)
+            cp16(d, a.in + o, in && c0 + l < a.ncols);
+        }
+      } else if constexpr (XAX) {
         int r0, r1;
         rows_of(k0 + (tid & 7), r0, r1);
         const int k = tid & 7;
@@ -291,13 +312,26 @@ __global__ void __launch_bounds__(128, 4) k_fold(FoldArgs a) {
       // table tile: entry (k, i) of C and S = the coefficient between contraction index k0 + k
       // and output index p0 + i; R is contiguous along m (forward k = m, inverse i = m)
       float* tb = tab + (t % 3) * tabw;
-      for (int q = tid; q < FK * BP; q += nt) {
-        const int k = FWD ? q % FK : q / BP, i = FWD ? q / FK : q - k * BP;
-        const int p = FWD ? p0 + i : k0 + k, m = FWD ? k0 + k : p0 + i;
-        const bool in = p < H && m < H, sn = in && p > 0 && 2 * p < n;
-        const float* rc = a.R + fold_row_c(p) * n + m;
-        cp(tb + k * BP + i, rc, in);
-        cp(tb + FK * BP + k * BP + i, rc + n, sn);       // the sin row follows the cos row
+      if (FWD) {
+        // a thread keeps k, its pairs are nt / FK apart
+        const int k = tid % FK, m = k0 + k;
+        for (int i = tid / FK; i < BP; i += nt / FK) {
+          const int p = p0 + i;
+          const float* rc = a.R + fold_row_c(p) * n + m;
+          const bool in = p < H && m < H;
+          cp(tb + k * BP + i, rc, in);
+          cp(tb + FK * BP + k * BP + i, rc + n, in && p > 0 && 2 * p < n);   // the sin row follows
+        }
+      } else {
+        // a thread keeps i, its rows of the contraction are nt / BP apart
+        const int m = p0 + ti;
+        for (int k = tk; k < FK; k += tstep) {
+          const int p = k0 + k;
+          const float* rc = a.R + fold_row_c(p) * n + m;
+          const bool in = p < H && m < H;
+          cp(tb + k * BP + ti, rc, in);
+          cp(tb + FK * BP + k * BP + ti, rc + n, in && p > 0 && 2 * p < n);
+        }
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -309,7 +343,35 @@ __global__ void __launch_bounds__(128, 4) k_fold(FoldArgs a) {
     const float* o = e + FK * FCS;
     float* ed = eo + (t & 1) * FE;
     float* od = ed + FK * FCS;
-    if constexpr (XAX) {
+    if (xv) {
+      for (int l = tid; l < FC; l += nt) {
+        const float4* q = reinterpret_cast<const float4*>(raw + (t & 1) * (FC * FX) + l * FX);
+        float v[FX];
+#pragma unroll
+        for (int c = 0; c < FX / 4; ++c) {
+          const float4 w = q[c];
+          v[4 * c] = w.x; v[4 * c + 1] = w.y; v[4 * c + 2] = w.z; v[4 * c + 3] = w.w;
+        }
+        if (k0 > 0 && 2 * (k0 + FK - 1) < n) {  // every element has its mirror
+#pragma unroll
+          for (int k = 0; k < FK; ++k) {
+            const float u = v[FWD ? k : 2 * k + 3], w = v[FWD ? 16 - k : 2 * k + 4];
+            ed[k * FCS + l] = FWD ? u + w : u;
+            od[k * FCS + l] = FWD ? u - w : w;
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < FK; ++k) {
+            const int kk = k0 + k;
+            const bool two = kk > 0 && 2 * kk < n;
+            const float u = kk < H ? (FWD ? v[k] : k == 0 && k0 == 0 ? v[4] : v[2 * k + 3]) : 0.f;
+            const float w = two ? (FWD ? v[16 - k] : v[2 * k + 4]) : 0.f;
+            ed[k * FCS + l] = FWD ? u + w : u;
+            od[k * FCS + l] = FWD ? (two ? u - w : 0.f) : w;
+          }
+        }
+      }
+    } else if constexpr (XAX) {
       const int k = tid & 7, kk = k0 + k;
       const bool mir = kk > 0 && 2 * kk < n;
       for (int l = tid >> 3; l < FC; l += nt >> 3) {
@@ -335,12 +397,13 @@ __global__ void __launch_bounds__(128, 4) k_fold(FoldArgs a) {
   issue(0);
   issue(1);
   asm volatile("cp.async.wait_group 1;" ::: "memory");
-  if (FWD) fold(0);
+  if (xv) __syncthreads();                    // a line's vectors come from several threads
+  if (FWD || xv) fold(0);
   __syncthreads();
   const int nst = (H + FK - 1) / FK;
   for (int t = 0; t < nst; ++t) {
     issue(t + 2);
-    const float* e = eo + (FWD ? (t & 1) : t % 3) * FE + 4 * tc;
+    const float* e = eo + (FWD || xv ? (t & 1) : t % 3) * FE + 4 * tc;
     const float* o = e + FK * FCS;
     const float* C = tab + (t % 3) * tabw + 4 * tp;
     const float* S = C + FK * BP;
@@ -364,7 +427,8 @@ __global__ void __launch_bounds__(128, 4) k_fold(FoldArgs a) {
         }
     }
     asm volatile("cp.async.wait_group 1;" ::: "memory");
-    if (FWD && t + 1 < nst) fold(t + 1);
+    if (xv) __syncthreads();
+    if ((FWD || xv) && t + 1 < nst) fold(t + 1);
     __syncthreads();
   }
 
@@ -504,9 +568,10 @@ static cudaError_t launch_fold(FoldArgs a, cudaStream_t s) {
   const int pad6 = (a.H + 23) / 24 * 6, pad8 = (a.H + 31) / 32 * 8;
   a.tp = pad6 <= pad8 ? 6 : 8;
   const int BP = 4 * a.tp;
-  const int stage = (FWD ? 4 : 3) * 2 * FK * FCS + 3 * 2 * FK * BP;
+  const int rows = XAX && a.vec ? 2 * FC * FX + 4 * FK * FCS : (FWD ? 4 : 3) * 2 * FK * FCS;
+  const int stage = rows + 3 * 2 * FK * BP;
   const int outw = XAX ? 64 * (2 * BP + 1) : 0;
-  const int smem = 4 * (stage > outw ? stage : outw);   // at most 39936 bytes
+  const int smem = 4 * (stage > outw ? stage : outw);   // at most 43520 bytes
   const dim3 grid((unsigned)((a.ncols + FC - 1) / FC), (unsigned)((a.H + BP - 1) / BP));
   k_fold<FWD, XAX><<<grid, 16 * a.tp, smem, s>>>(a);
   return cudaGetLastError();
@@ -697,7 +762,8 @@ static cudaError_t apply_K_fp32(const KPlan& kp, const float* in, float* out, fl
                                 int ncomp, cudaStream_t s, const Hook& hook, float* v_upd,
                                 float eps) {
   const int X = kp.nx, Y = kp.ny, Z = kp.nz, XY = X * Y, N = XY * Z;
-  const int vy = X % 4 == 0 && ((uintptr_t)work & 15) == 0 && ((uintptr_t)out & 15) == 0;
+  const auto v4 = [&](const float* p) { return X % 4 == 0 && ((uintptr_t)p & 15) == 0; };
+  const int vy = v4(work) && v4(out);
   const int vz = vy;                 // XY and N are multiples of X
   const bool sp = small_plane(kp, ncomp), sc = small_columns(kp, ncomp);
   auto axis = [&](int n, const float* R, int ncols, int W, int hi, int rs, int vec,
@@ -727,7 +793,7 @@ static cudaError_t apply_K_fp32(const KPlan& kp, const float* in, float* out, fl
   if (sp) {
     SMALL(KID_KX_FWD, small_xy(kp, true, in, a, ncomp, nullptr, 0.f, s));
   } else {
-    FOLD(KID_KX_FWD, true, true, axis(kp.nx, kp.Rx, ncomp * Y * Z, 1, X, 1, 0, in, work));
+    FOLD(KID_KX_FWD, true, true, axis(kp.nx, kp.Rx, ncomp * Y * Z, 1, X, 1, v4(in), in, work));
     FOLD(KID_KY_FWD, true, false, axis(kp.ny, kp.Ry, ncomp * Z * X, X, XY, X, vy, work, a));
   }
   if (sc) {
@@ -744,7 +810,7 @@ static cudaError_t apply_K_fp32(const KPlan& kp, const float* in, float* out, fl
     SMALL(KID_KX_INV, small_xy(kp, false, a, out, ncomp, v_upd, eps, s));
   } else {
     FOLD(KID_KY_INV, false, false, axis(kp.ny, kp.Ry, ncomp * Z * X, X, XY, X, vy, a, work));
-    FoldArgs xi = axis(kp.nx, kp.Rx, ncomp * Y * Z, 1, X, 1, 0, work, out);
+    FoldArgs xi = axis(kp.nx, kp.Rx, ncomp * Y * Z, 1, X, 1, v4(work), work, out);
     xi.v_upd = v_upd;
     xi.eps = eps;
     FOLD(KID_KX_INV, false, true, xi);
