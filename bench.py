@@ -60,6 +60,8 @@ def _csrc_hash():
 def algorithmic(kernel, N, dims, kmode, T=10, peaks=None):
     X, Y, Z = dims
     B = {"flow_back_disp": 36, "flow_back_terms": 28, "fwd_residual": 36,
+         # both in one pass over u_{j+1}: v_j, u_{j+1}, I1, M in; u_j, J1, W out
+         "flow_back": 52,
          "fwd_flow": 36, "update": 36,
          # residual b_j and map of step j + 1 over one read of u_j: u_j, I0, J1_j, W_j, v_j in;
          # b_j (split), u_{j+1} out

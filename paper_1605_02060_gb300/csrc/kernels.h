@@ -29,7 +29,7 @@ struct Hook {
 enum KernelId {
   KID_BACK_DISP = 0, KID_BACK_TERMS, KID_FWD_TERMS, KID_FWD_FLOW, KID_KX_FWD, KID_KY_FWD,
   KID_KZ_SYM, KID_KZ_INV, KID_KY_INV, KID_KX_INV, KID_UPDATE, KID_EREG, KID_KZ_FUSED,
-  KID_FWD_FUSED, KID_J0_EDATA, KID_COUNT
+  KID_FWD_FUSED, KID_J0_EDATA, KID_BACK_FUSED, KID_COUNT
 };
 
 // ---- flows (kernels_flow.cu) ----
@@ -39,12 +39,14 @@ enum KernelId {
 // backward sweep (launch_flow_back), the map phi_{0,1} it leaves and the steps of a forward sweep
 // without the residual use the quad layout, the iteration's forward sweep (launch_fwd_fused) and
 // phi_{1,0} the planar one.
-// Backward sweep step j (quad maps): u_cur = dt v_j / h + u_next(x + dt v_j / h)
-// (u_next == nullptr: id), then J1_j = I1 o phi, W_j = (M o phi) det(I + Du_cur), min det into
-// acc.  IM holds I1 and M interleaved as pairs (launch_interleave).
+// Backward sweep step j (quad maps): u_cur = dt v_j / h + u_next(x + dt v_j / h) (u_next == nullptr:
+// id) and, unless u_next is null, the terms of u_next = phi_{j+1,1} - id: J1 = I1 o phi, W = (M o phi)
+// det(I + Du_next), min det into acc.  launch_back_last: the terms of u = phi_{0,1} - id.  IM holds I1 and M interleaved as pairs (launch_interleave).
 void launch_flow_back(const Grid& g, const void* vj, const float* u_next, float* u_cur,
-                      const void* IM, float* J1j, float* Wj, float dtx, float dty, float dtz,
+                      const void* IM, float* J1, float* W, float dtx, float dty, float dtz,
                       Acc* acc, cudaStream_t s, const Hook& hook, int st, int rk = 0);
+void launch_back_last(const Grid& g, const float* u, const void* IM, float* J1, float* W, Acc* acc,
+                      cudaStream_t s, const Hook& hook, int st);
 // out[i] = (a[i], b[i]) as storage-type pairs.
 void launch_interleave(const void* a, const void* b, void* out, int64_t n, cudaStream_t s,
                        int st);

@@ -247,6 +247,57 @@ __device__ __forceinline__ float2 tri_apply_pair(const PT* __restrict__ f, const
   return r;
 }
 
+// Terms of a voxel column's plane z from the map at z - 1, z, z + 1 (uP, uC, uN); returns the
+// determinant.
+struct Sides {          // neighbours along x and y (one-sided at the faces), reciprocal distances
+  int xlo, xhi, ylo, yhi;
+  float ix, iy;
+};
+__device__ __forceinline__ Sides sides_of(const Grid& g, int x, int y) {
+  Sides s;
+  s.xlo = x > 0 ? x - 1 : x;
+  s.xhi = x < g.nx - 1 ? x + 1 : x;
+  s.ylo = y > 0 ? y - 1 : y;
+  s.yhi = y < g.ny - 1 ? y + 1 : y;
+  s.ix = (x > 0 && x < g.nx - 1) ? 0.5f : 1.0f;
+  s.iy = (y > 0 && y < g.ny - 1) ? 0.5f : 1.0f;
+  return s;
+}
+template <bool Q, typename PT>
+__device__ __forceinline__ float back_terms_at(const Grid& g, const float* __restrict__ uc,
+                                               const PT* __restrict__ IM, float* __restrict__ J1j,
+                                               float* __restrict__ Wj, int x, int y, int z,
+                                               const Sides& sd, const float (&uP)[3],
+                                               const float (&uC)[3], const float (&uN)[3]) {
+  const int zp = z * (g.nx * g.ny), i = zp + y * g.nx + x;
+  float D[3][3];
+  const float iz = (z > 0 && z < g.nz - 1) ? 0.5f : 1.0f;
+  {
+    const float3 xh = MapL<Q>::at(uc, g.N, zp + y * g.nx + sd.xhi);
+    const float3 xl = MapL<Q>::at(uc, g.N, zp + y * g.nx + sd.xlo);
+    const float3 yh = MapL<Q>::at(uc, g.N, zp + sd.yhi * g.nx + x);
+    const float3 yl = MapL<Q>::at(uc, g.N, zp + sd.ylo * g.nx + x);
+    const float xhv[3] = {xh.x, xh.y, xh.z}, xlv[3] = {xl.x, xl.y, xl.z};
+    const float yhv[3] = {yh.x, yh.y, yh.z}, ylv[3] = {yl.x, yl.y, yl.z};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      D[d][0] = (xhv[d] - xlv[d]) * sd.ix;
+      D[d][1] = (yhv[d] - ylv[d]) * sd.iy;
+      const float zh = z < g.nz - 1 ? uN[d] : uC[d], zl = z > 0 ? uP[d] : uC[d];
+      D[d][2] = (zh - zl) * iz;
+      D[d][d] += 1.0f;
+    }
+  }
+  const float det = D[0][0] * (D[1][1] * D[2][2] - D[1][2] * D[2][1]) -
+                    D[0][1] * (D[1][0] * D[2][2] - D[1][2] * D[2][0]) +
+                    D[0][2] * (D[1][0] * D[2][1] - D[1][1] * D[2][0]);
+  const Tri w = tri_setup(g, (float)x + uC[0], (float)y + uC[1], (float)z + uC[2]);
+  const float2 jm = tri_apply_pair(IM, w);
+  J1j[i] = jm.x;
+  Wj[i] = jm.y * det;
+  return det;
+}
+
 // At most 40 registers (6 blocks of 256 threads per SM): the march waits on its lookups, and the
 // extra warps in flight outweigh the few spilled values (48 registers, 5 blocks: 93 against
 // 87 us at 264x160x228; 32 registers spill inside the loop and take 130 us).
@@ -261,11 +312,7 @@ __global__ void __launch_bounds__(256, 6) k_back_terms_march(Grid g, const float
   if (in) {
     const int z0 = blockIdx.z * ZC, z1 = min(z0 + ZC, g.nz);
     const int plane = g.nx * g.ny, rowoff = y * g.nx;
-    // x and y stencils (central inside, one-sided at the faces)
-    const int xlo = x > 0 ? x - 1 : x, xhi = x < g.nx - 1 ? x + 1 : x;
-    const int ylo = y > 0 ? y - 1 : y, yhi = y < g.ny - 1 ? y + 1 : y;
-    const float ix = (x > 0 && x < g.nx - 1) ? 0.5f : 1.0f;
-    const float iy = (y > 0 && y < g.ny - 1) ? 0.5f : 1.0f;
+    const Sides sd = sides_of(g, x, y);
     auto ld3 = [&](int z, float* u) {
       const float3 r = MapL<Q>::at(uc, g.N, z * plane + rowoff + x);
       u[0] = r.x; u[1] = r.y; u[2] = r.z;
@@ -278,39 +325,63 @@ __global__ void __launch_bounds__(256, 6) k_back_terms_march(Grid g, const float
       // the plane after next, for the z-derivative of plane z + 1
       const int zn = z + 2 < g.nz ? z + 2 : g.nz - 1;
       if (z + 1 < z1) ld3(zn, uNN);
-      const int i = z * plane + rowoff + x;
-      float D[3][3];
-      const float iz = (z > 0 && z < g.nz - 1) ? 0.5f : 1.0f;
-      {
-        const int zp = z * plane;
-        const float3 xh = MapL<Q>::at(uc, g.N, zp + rowoff + xhi);
-        const float3 xl = MapL<Q>::at(uc, g.N, zp + rowoff + xlo);
-        const float3 yh = MapL<Q>::at(uc, g.N, zp + yhi * g.nx + x);
-        const float3 yl = MapL<Q>::at(uc, g.N, zp + ylo * g.nx + x);
-        const float xhv[3] = {xh.x, xh.y, xh.z}, xlv[3] = {xl.x, xl.y, xl.z};
-        const float yhv[3] = {yh.x, yh.y, yh.z}, ylv[3] = {yl.x, yl.y, yl.z};
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-          D[d][0] = (xhv[d] - xlv[d]) * ix;
-          D[d][1] = (yhv[d] - ylv[d]) * iy;
-          const float zh = z < g.nz - 1 ? uN[d] : uC[d], zl = z > 0 ? uP[d] : uC[d];
-          D[d][2] = (zh - zl) * iz;
-          D[d][d] += 1.0f;
-        }
-      }
-      const float det = D[0][0] * (D[1][1] * D[2][2] - D[1][2] * D[2][1]) -
-                        D[0][1] * (D[1][0] * D[2][2] - D[1][2] * D[2][0]) +
-                        D[0][2] * (D[1][0] * D[2][1] - D[1][1] * D[2][0]);
-      const Tri w = tri_setup(g, (float)x + uC[0], (float)y + uC[1], (float)z + uC[2]);
-      const float2 jm = tri_apply_pair(IM, w);
-      J1j[i] = jm.x;
-      Wj[i] = jm.y * det;
-      dmin = fminf(dmin, det);
+      dmin = fminf(dmin, back_terms_at<Q>(g, uc, IM, J1j, Wj, x, y, z, sd, uP, uC, uN));
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         uP[d] = uC[d];
         uC[d] = uN[d];
         uN[d] = uNN[d];
+      }
+    }
+  }
+  block_min_atomic(dmin, &acc->min_det_ord);
+}
+
+// Backward sweep, one step of a small or middling grid: the terms of u_{j+1} (J1, W, min det) and u_j =
+// dt v_j / h + u_{j+1}(x + dt v_j / h) in one pass over u_{j+1} (quad maps), as k_back_terms_march and
+// k_disp_march give them: one launch, and the lookups of either in flight together.  The rule and its
+// figures are at launch_flow_back.
+template <typename ST, int ZC>
+__global__ void __launch_bounds__(256, ZC == 1 ? 4 : 5) k_back_fused_march(
+    Grid g, const ST* __restrict__ vj, const float* __restrict__ uc, float* __restrict__ un,
+    float dtx, float dty, float dtz, const typename Pair<ST>::T* __restrict__ IM,
+    float* __restrict__ J1, float* __restrict__ W, Acc* acc) {
+  const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y;
+  const bool in = x < g.nx && y < g.ny;
+  float dmin = 3.0e38f;
+  if (in) {
+    const int z0 = blockIdx.z * ZC, z1 = min(z0 + ZC, g.nz);
+    const int plane = g.nx * g.ny;
+    int idx = (z0 * g.ny + y) * g.nx + x;
+    const Sides sd = sides_of(g, x, y);
+    float a0 = ldf(vj + idx), a1 = ldf(vj + g.N + idx), a2 = ldf(vj + 2 * g.N + idx);
+    auto ld3 = [&](int z, float* u) {
+      const float3 r = MapL<true>::at(uc, g.N, z * plane + y * g.nx + x);
+      u[0] = r.x; u[1] = r.y; u[2] = r.z;
+    };
+    float uP[3], uC[3], uN[3];
+    ld3(z0 > 0 ? z0 - 1 : z0, uP);
+    ld3(z0, uC);
+    for (int z = z0; z < z1; ++z, idx += plane) {
+      float n0 = 0.f, n1 = 0.f, n2 = 0.f;
+      if (z + 1 < z1) {
+        n0 = ldf_now(vj + idx + plane);
+        n1 = ldf_now(vj + g.N + idx + plane);
+        n2 = ldf_now(vj + 2 * g.N + idx + plane);
+      }
+      ld3(z + 1 < g.nz ? z + 1 : z, uN);
+      const float dx = dtx * a0, dy = dty * a1, dz = dtz * a2;
+      const float3 r =
+          MapL<true>::lerp(uc, g.N, tri_setup(g, (float)x + dx, (float)y + dy, (float)z + dz));
+      MapL<true>::put(un, g.N, idx, dx + r.x, dy + r.y, dz + r.z);
+      dmin = fminf(dmin, back_terms_at<true>(g, uc, IM, J1, W, x, y, z, sd, uP, uC, uN));
+      a0 = n0;
+      a1 = n1;
+      a2 = n2;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        uP[d] = uC[d];
+        uC[d] = uN[d];
       }
     }
   }
@@ -353,15 +424,55 @@ static void launch_back_terms(const Grid& g, const float* uc, const void* IM, fl
     k_back_terms_march<ST, 8, true><<<flow_grid(g, 8), kBlock3d, 0, s>>>(g, uc, im, J1j, Wj, acc);
 }
 
-void launch_flow_back(const Grid& g, const void* vj, const float* u_next, float* u_cur,
-                      const void* IM, float* J1j, float* Wj, float dtx, float dty, float dtz,
-                      Acc* acc, cudaStream_t s, const Hook& hook, int st, int rk) {
+// One kernel or two, by the number of four-plane blocks (us a step; two kernels cost a launch besides):
+//                    33x20x29 (48)   64^3 (256)   132x80x114 (1450)   128^3 (2048)   264x160x228 (10260)
+//   two              1.9 + 2.2       3.6 + 4.2    11.7 + 12.8         14.9 + 20.4    71 + 80
+//   one, 1 plane     3.1             6.6          26.5                41.5           196
+//   one, 8 planes    10              12           21.6                43             155
+// Blocks of 8 planes pay while the SMs hold them all at once, five each (141x97x109, 910 of them: 32.7
+// us against 15.1 + 14.2); on the large grids the 48 registers leave too few warps in flight.
+template <typename ST>
+static void flow_back(const Grid& g, const ST* vj, const float* u_next, float* u_cur, const void* IM,
+                      float* J1, float* W, float dtx, float dty, float dtz, Acc* acc, cudaStream_t s,
+                      const Hook& hook, int rk) {
+  const int nb = flow_blocks(g);
+  const dim3 by8 = flow_grid(g, 8);
+  if (u_next && !rk && (nb <= 256 || by8.x * by8.y * by8.z <= 152 * 5)) {
+    const typename Pair<ST>::T* im = reinterpret_cast<const typename Pair<ST>::T*>(IM);
+    hook(KID_BACK_FUSED, 0);
+    if (nb <= 256)
+      k_back_fused_march<ST, 1><<<flow_grid(g, 1), kBlock3d, 0, s>>>(g, vj, u_next, u_cur, dtx, dty,
+                                                                     dtz, im, J1, W, acc);
+    else
+      k_back_fused_march<ST, 8><<<by8, kBlock3d, 0, s>>>(g, vj, u_next, u_cur, dtx, dty, dtz, im, J1,
+                                                         W, acc);
+    hook(KID_BACK_FUSED, 1);
+    return;
+  }
+  if (u_next) {
+    hook(KID_BACK_TERMS, 0);
+    launch_back_terms<ST>(g, u_next, IM, J1, W, acc, s);
+    hook(KID_BACK_TERMS, 1);
+  }
   hook(KID_BACK_DISP, 0);
-  disp_step(+1, g, vj, u_next, u_cur, dtx, dty, dtz, s, st, rk, 1);
+  launch_disp_march<ST, 1, true>(g, vj, u_next, u_cur, dtx, dty, dtz, s, rk);
   hook(KID_BACK_DISP, 1);
+}
+
+void launch_flow_back(const Grid& g, const void* vj, const float* u_next, float* u_cur,
+                      const void* IM, float* J1, float* W, float dtx, float dty, float dtz,
+                      Acc* acc, cudaStream_t s, const Hook& hook, int st, int rk) {
+  if (st)
+    flow_back(g, (const __nv_bfloat16*)vj, u_next, u_cur, IM, J1, W, dtx, dty, dtz, acc, s, hook, rk);
+  else
+    flow_back(g, (const float*)vj, u_next, u_cur, IM, J1, W, dtx, dty, dtz, acc, s, hook, rk);
+}
+
+void launch_back_last(const Grid& g, const float* u, const void* IM, float* J1, float* W, Acc* acc,
+                      cudaStream_t s, const Hook& hook, int st) {
   hook(KID_BACK_TERMS, 0);
-  if (st) launch_back_terms<__nv_bfloat16>(g, u_cur, IM, J1j, Wj, acc, s);
-  else launch_back_terms<float>(g, u_cur, IM, J1j, Wj, acc, s);
+  if (st) launch_back_terms<__nv_bfloat16>(g, u, IM, J1, W, acc, s);
+  else launch_back_terms<float>(g, u, IM, J1, W, acc, s);
   hook(KID_BACK_TERMS, 1);
 }
 

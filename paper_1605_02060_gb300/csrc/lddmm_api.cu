@@ -178,7 +178,7 @@ const char* kernel_name(int kid) {
   static const char* names[KID_COUNT] = {"flow_back_disp", "flow_back_terms", "fwd_residual",
                                          "fwd_flow", "K_x_fwd", "K_y_fwd", "K_z_symbol",
                                          "K_z_inv", "K_y_inv", "K_x_inv_update", "update", "ereg",
-                                         "K_z_fused", "fwd_fused", "fwd_J0T_Edata"};
+                                         "K_z_fused", "fwd_fused", "fwd_J0T_Edata", "flow_back"};
   return (kid >= 0 && kid < KID_COUNT) ? names[kid] : "?";
 }
 
@@ -392,11 +392,12 @@ int record_step(lddmm_ctx* ctx) {
   int pb = 0;
   for (int j = T - 1; j >= 0; --j) {
     float* uc = ctx->uB[pb];
-    launch_flow_back(g, vptr(ctx, j, N), un, uc, L.IM, ctx->J1 + j * N, ctx->W + j * N, dtx,
-                     dty, dtz, ctx->acc, s, hk, ctx->st, rk_of(ctx));
+    launch_flow_back(g, vptr(ctx, j, N), un, uc, L.IM, ctx->J1 + (j + 1) * N, ctx->W + (j + 1) * N,
+                     dtx, dty, dtz, ctx->acc, s, hk, ctx->st, rk_of(ctx));
     un = uc;
     pb ^= 1;
   }
+  launch_back_last(g, un, L.IM, ctx->J1, ctx->W, ctx->acc, s, hk, ctx->st);
   ctx->u01 = un;
   // E_reg of the velocity at the start of the iteration (before the forward sweep updates it)
   hk(KID_EREG, 0);
