@@ -28,6 +28,7 @@
 
 #include "kernels.h"
 #include "tc_ptx.cuh"
+#include "tmem_ahead.cuh"
 
 namespace lddmm {
 
@@ -581,15 +582,14 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
         conv_ok = ptx::mbar_wait_or_abort(ptx::smem_u32(&b_tfull[0]), (uint32_t)i & 1u, abort, a.poll);
         ptx::tc_fence_after();
         const uint32_t t1 = tmem + ((uint32_t)(q * 32) << 16);
-        // the first chunk's load, then always the next one's while this one is converted
-        uint32_t uc[16], un[16];
-        if (conv_ok && part < nch) ptx::tmem_issue16(t1 + (uint32_t)(part * 16), uc);
+        // the first chunk, then always the next one's load while this one is converted
+        TmemAhead<ptx::TmemLd16> tm;
+        if (conv_ok && part < nch) tm.first(t1 + (uint32_t)(part * 16));
         for (int kb = 0; conv_ok && kb < nkb; ++kb) {
           const int c1 = min(4 * kb + 4, nch);
           // this part's chunks of the block: c = part (mod nparts)
           for (int c = 4 * kb + (part + nparts * nkb * 4 - 4 * kb) % nparts; c < c1; c += nparts) {
-            ptx::tmem_wait16(uc);
-            if (c + nparts < nch) ptx::tmem_issue16(t1 + (uint32_t)((c + nparts) * 16), un);
+            if (c + nparts < nch) tm.ahead(t1 + (uint32_t)((c + nparts) * 16));
             const float4* lz4 = reinterpret_cast<const float4*>(a.lz + c * 16);
             uint32_t hw[8], lw[8];
 #pragma unroll
@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
 #pragma unroll
               for (int jj = 0; jj < 2; ++jj) {
                 const int j = 2 * j4 + jj;
-                const float v0 = __uint_as_float(uc[2 * j]), v1 = __uint_as_float(uc[2 * j + 1]);
+                const float v0 = __uint_as_float(tm.u[2 * j]), v1 = __uint_as_float(tm.u[2 * j + 1]);
                 if constexpr (EPI == EPI_ZZ_RN) {
                   const float d0 = fmaf(a.alpha, sxy + zl[2 * jj], a.gamma);
                   const float d1 = fmaf(a.alpha, sxy + zl[2 * jj + 1], a.gamma);
@@ -613,8 +613,7 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
             }
             ptx::tmem_st8(t1 + (uint32_t)(c * 16), hw);
             if (a.split) ptx::tmem_st8(t1 + (uint32_t)(c * 16 + 8), lw);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) uc[j] = un[j];
+            if (c + nparts < nch) tm.advance();
           }
           ptx::tmem_wait_st();
           ptx::tc_fence_before();
@@ -668,12 +667,11 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
         const bool gvalid = line0 < a.nlines;
         const int E = (int)o.E, D = (int)o.D;
         const int t = (int)line0 / E, e0 = (int)line0 - t * E, r3 = t / D, r1 = t - r3 * D;
-        uint32_t uc[16], un[16];
-        if (cnt > 0) ptx::tmem_issue16(tcol(chunk_at(0)), uc);
+        TmemAhead<ptx::TmemLd16> tm;
+        if (cnt > 0) tm.first(tcol(chunk_at(0)));
         for (int k = 0; k < cnt; ++k) {
           const int c = chunk_at(k);
-          ptx::tmem_wait16(uc);
-          if (k + 1 < cnt) ptx::tmem_issue16(tcol(chunk_at(k + 1)), un);
+          if (k + 1 < cnt) tm.ahead(tcol(chunk_at(k + 1)));
           if (k + 1 == ntl) {             // the second product's columns are read
             ptx::tc_fence_before();
             ptx::mbar_arrive(ptx::smem_u32(&b_ttail));
@@ -683,7 +681,7 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
 #pragma unroll
           for (int j = 0; j < 16; j += 2) {
             uint32_t h, lo;
-            split2(__uint_as_float(uc[j]), __uint_as_float(uc[j + 1]), h, lo);
+            split2(__uint_as_float(tm.u[j]), __uint_as_float(tm.u[j + 1]), h, lo);
             wt[j * 32 + lane] = (uint16_t)h;
             wt[(j + 1) * 32 + lane] = (uint16_t)(h >> 16);
             wt[512 + j * 32 + lane] = (uint16_t)lo;
@@ -696,8 +694,7 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
             if (a.split) ptx::tma_store_5d(&tmO, wts + 1024u, e0, r1, c * 16, r3, 1);
             ptx::bulk_commit();
           }
-#pragma unroll
-          for (int j = 0; j < 16; ++j) uc[j] = un[j];
+          if (k + 1 < cnt) tm.advance();
         }
       } else if constexpr (staged) {
         // Transposed split output.  Per 16-column chunk the four quadrant warps of this column
