@@ -5,8 +5,36 @@
 #include <stdint.h>
 
 #include "common.cuh"
+#include "per_device.h"
 
 namespace lddmm {
+
+// Raises a kernel's dynamic shared memory limit to `bytes`, once on each device; `set` is the kernel's
+// own record.  The limit is the most the kernel is ever launched with, not one launch's need: a lower
+// value would undo what an earlier launch (a recorded graph node) counts on.
+template <typename Kernel>
+cudaError_t raise_smem_limit(PerDevice<bool>& set, Kernel* kernel, int bytes) {
+  int dev = -1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  set.get(dev, [&] {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return e == cudaSuccess;
+  });
+  return e;
+}
+
+// SMs of the current device.
+inline int sm_count() {
+  static PerDevice<int> kept;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
+  const int n = kept.get(dev, [&] {
+    int m = 0;
+    return cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? m : 0;
+  });
+  return n > 0 ? n : 148;
+}
 
 // Accumulators written by the reduction kernels (device memory, reset per iteration).
 struct Acc {

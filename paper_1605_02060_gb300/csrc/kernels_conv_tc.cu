@@ -286,19 +286,24 @@ bool conv_tc_supported(int Ci, int Co, int n) {
 }
 
 // Device flag a tensor-core convolution sets when one of its bounded waits gave up (its tile's
-// outputs are then NaN); allocated once per process.
+// outputs are then NaN); allocated once on each device.
 static int* conv_err_flag() {
-  static int* f = nullptr;
-  if (!f && cudaMalloc((void**)&f, sizeof(int)) == cudaSuccess) cudaMemset(f, 0, sizeof(int));
-  else cudaGetLastError();
-  return f;
+  static PerDevice<int*> kept;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev >= kKeptDevices) return nullptr;
+  return kept.get(dev, [] {
+    int* f = nullptr;
+    if (cudaMalloc((void**)&f, sizeof(int)) == cudaSuccess) cudaMemset(f, 0, sizeof(int));
+    else cudaGetLastError();
+    return f;
+  });
 }
 
 template <int TPS>
 static cudaError_t launch_conv(const ConvArgs& a, int B, cudaStream_t s) {
-  static const cudaError_t set = cudaFuncSetAttribute(
-      k_conv_tc<TPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, CV_SMEM_CAP);
-  if (set != cudaSuccess) return set;
+  static PerDevice<bool> set;
+  const cudaError_t e = raise_smem_limit(set, k_conv_tc<TPS>, CV_SMEM_CAP);
+  if (e != cudaSuccess) return e;
   // persistent: two CTAs per SM share the blocks (the weights are staged once per CTA)
   const int smem = (int)cv_smem(a.slots, a.L, TPS * (a.wres ? a.Ci / 16 * a.nph : 1), a.Np);
   const int cap = (smem <= CV_SMEM_PAIR ? 304 : 152) / a.NS, grid = a.NS * (a.nblk < cap ? a.nblk : cap);

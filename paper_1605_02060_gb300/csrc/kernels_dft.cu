@@ -741,12 +741,11 @@ static bool small_columns(const KPlan& kp, int ncomp) {
 // x and y forward (in -> out) or inverse (in -> out, or the update of v) of every plane.
 static cudaError_t small_xy(const KPlan& kp, bool fwd, const float* in, float* out, int ncomp,
                             float* v_upd, float eps, cudaStream_t s) {
-  static const cudaError_t set[2] = {
-      cudaFuncSetAttribute(k_small_xy<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SN_SMEM),
-      cudaFuncSetAttribute(k_small_xy<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SN_SMEM)};
-  if (set[0] != cudaSuccess || set[1] != cudaSuccess) return set[0] != cudaSuccess ? set[0] : set[1];
+  static PerDevice<bool> set[2];
   const int smem = 4 * small_xy_floats(kp.nx, kp.ny);
   auto* k = fwd ? k_small_xy<true> : k_small_xy<false>;
+  const cudaError_t e = raise_smem_limit(set[fwd], k, SN_SMEM);
+  if (e != cudaSuccess) return e;
   k<<<ncomp * kp.nz, SN_NT, smem, s>>>(in, out, kp.nx, kp.ny, kp.Rx, kp.Ry, v_upd, eps);
   return cudaGetLastError();
 }

@@ -782,8 +782,6 @@ __global__ void __launch_bounds__(KS_NT, 1) k_dft_ks(const __grid_constant__ CUt
   if (threadIdx.x == 0 && abort_sh) atomicExch(a.err, 3);
 }
 
-int g_ks_sms = 0;
-
 EncodeTiledFn encode_fn() {
   static EncodeTiledFn fn = nullptr;
   static bool tried = false;
@@ -966,23 +964,12 @@ cudaError_t ks_axis_pass(const KPlan& kp, int axis, bool inverse, int split, con
             : epi == EPI_UPD_1    ? k_dft_ks<EPI_UPD_1>
             : epi == EPI_ZZ_RN    ? k_dft_ks<EPI_ZZ_RN>
                                   : k_dft_ks<EPI_ZZ>;
-  // The limit is set once per kernel, to the cap every pass stays under: a per-pass value would
-  // lower it below what an earlier launch of the same kernel (a recorded graph node) needs.
-  static bool limit_set[EPI_COUNT] = {};
   if (smem > KS_SMEM_CAP) return cudaErrorNotSupported;
-  if (!limit_set[epi]) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         KS_SMEM_CAP);
-    if (e != cudaSuccess) return e;
-    limit_set[epi] = true;
-  }
-  if (!g_ks_sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&g_ks_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (g_ks_sms <= 0) g_ks_sms = 148;
-  }
-  const int grid = a.ntiles < g_ks_sms ? a.ntiles : g_ks_sms;
+  static PerDevice<bool> limit_set[EPI_COUNT];
+  const cudaError_t e = raise_smem_limit(limit_set[epi], kern, KS_SMEM_CAP);
+  if (e != cudaSuccess) return e;
+  const int sms = sm_count();
+  const int grid = a.ntiles < sms ? a.ntiles : sms;
   if (grid > 0) kern<<<grid, KS_NT, smem, s>>>(tmA, tmB, tmB2, tmO, a);
   return cudaGetLastError();
 }

@@ -654,9 +654,9 @@ template <int CIT>
 static cudaError_t launch_wgrad3(const float* x, const float* dy, float* part, int B, int Ci, int Co,
                                  int n, int G, cudaStream_t s) {
   constexpr int smem = 2 * 4 * wg_words(CIT);
-  static const cudaError_t set =
-      cudaFuncSetAttribute(k_wgrad3<CIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (set != cudaSuccess) return set;
+  static PerDevice<bool> set;
+  const cudaError_t e = raise_smem_limit(set, k_wgrad3<CIT>, smem);
+  if (e != cudaSuccess) return e;
   const dim3 grid(G, ((Ci + CIT - 1) / CIT) * ((Co + CT - 1) / CT));
   k_wgrad3<CIT><<<grid, wg_threads(CIT), smem, s>>>(x, dy, part, B, Ci, Co, n, G);
   return cudaGetLastError();
@@ -670,9 +670,8 @@ cudaError_t net_conv_wgrad(const float* x, const float* dy, float* dw, float* db
   cudaError_t e;
   if (ks == 1) {
     constexpr int smem = 2 * 4 * 2 * NTV * (CT + 1);
-    static const cudaError_t set =
-        cudaFuncSetAttribute(k_wgrad1, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (set != cudaSuccess) return set;
+    static PerDevice<bool> set;
+    if ((e = raise_smem_limit(set, k_wgrad1, smem)) != cudaSuccess) return e;
     const dim3 grid(G, ((Ci + 15) / 16) * ((Co + CT - 1) / CT));
     k_wgrad1<<<grid, 256, smem, s>>>(x, dy, scratch, B, Ci, Co, n, G);
     e = cudaGetLastError();

@@ -50,6 +50,7 @@ constexpr int RAW_BYTES = TC_BM * 16 * 4;   // fp32 slice
 constexpr int AOP_BYTES = TC_BM * 16 * 2;   // one bf16 operand slice (hi or lo)
 
 __host__ __device__ inline int stage_bytes(int Npad) { return RAW_BYTES + 2 * AOP_BYTES + Npad * 64; }
+constexpr int TC_SMEM_CAP = 4 * (RAW_BYTES + 2 * AOP_BYTES + 512 * 64);   // four stages of the longest axis
 
 // byte offset of (row, kk) inside one K-major no-swizzle slice of 16 columns
 __device__ __forceinline__ uint32_t kmajor_off(int row, int kk) {
@@ -302,15 +303,9 @@ static int pow2_cols(int n) {
 template <int LOADT, int S>
 static cudaError_t launch_tc(const TcArgs& a, cudaStream_t s) {
   const int smem = S * stage_bytes(a.Npad);
-  // the kernel's shared-memory limit only ever rises: an earlier launch (a recorded graph node)
-  // may need more than this one
-  static int limit = 0;
-  if (smem > limit) {
-    cudaError_t e = cudaFuncSetAttribute(k_dft_tc<LOADT, S>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    limit = smem;
-  }
+  static PerDevice<bool> set;
+  const cudaError_t e = raise_smem_limit(set, k_dft_tc<LOADT, S>, TC_SMEM_CAP);
+  if (e != cudaSuccess) return e;
   const int grid = (a.M + TC_BM - 1) / TC_BM;
   if (grid > 0) k_dft_tc<LOADT, S><<<grid, TC_THREADS, smem, s>>>(a);
   return cudaGetLastError();
