@@ -144,7 +144,9 @@ int lddmm_warp(lddmm_ctx* ctx, const float* src, float* dst, int direction);
  * clamped to the grid (§2.5).  uint16 labels, nx*ny*nz each, current level grid. */
 int lddmm_transfer_labels(lddmm_ctx* ctx, const uint16_t* L0, uint16_t* dst);
 
-/* Velocity field of the current level, [T][3][nz][ny][nx] float32. */
+/* Velocity field of the current level, [T][3][nz][ny][nx] float32.  lddmm_set_velocity refuses a
+ * field with NaN or Inf (LDDMM_ERR_NONFINITE); v is then 0, whatever memory src lies in and in
+ * either storage.  After any other error set v again. */
 int lddmm_get_velocity(lddmm_ctx* ctx, float* dst);
 int lddmm_set_velocity(lddmm_ctx* ctx, const float* src);
 
@@ -193,8 +195,9 @@ int lddmm_landmark_error(lddmm_ctx* ctx, const float* xk, const float* yk, int n
  * v0.  The momentum m_0 = L^T L v0 is transported by the flow, m_j = |D phi| (D phi)^T (m_0 o phi)
  * with phi = phi_{j,0} from the same semi-Lagrangian steps as the forward sweep, and
  * v_j = K m_j with the context's K.  v0: float [3][nz][ny][nx] of the current level, device or
- * host memory, in physical units.  Needs float storage (params.storage = 0) and the one-lookup
- * flow (flags bit 2 clear). */
+ * host memory, in physical units; with NaN or Inf in it the call fails and v is 0, as for
+ * lddmm_set_velocity.  Needs float storage (params.storage = 0) and the one-lookup flow (flags
+ * bit 2 clear). */
 int lddmm_shoot(lddmm_ctx* ctx, const float* v0);
 
 /* Image-LDDMM preprocessing (§2.2): the masks are applied to the images and the masked I0 is

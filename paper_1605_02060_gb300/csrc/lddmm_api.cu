@@ -824,8 +824,23 @@ int lddmm_get_velocity(lddmm_ctx* ctx, float* dst) {
   return wait_stream(ctx);
 }
 
-int lddmm_set_velocity(lddmm_ctx* ctx, const float* src) {
-  if (!ctx || !src) return fail(ctx, LDDMM_ERR_INVALID_ARG, "NULL argument");
+namespace {
+// Before v is written: what describes the old field no longer holds, however the call ends.
+void forget_velocity(lddmm_ctx* ctx) {
+  ctx->maps_valid = false;
+  ctx->j0_valid = false;
+  ctx->last_E = -1.0;
+}
+
+// After a new v was refused: rc is returned, v is 0 (the check follows the store, in one pass over
+// the field, so the old one is gone).
+int refused_velocity(lddmm_ctx* ctx, int rc) {
+  if (rc == LDDMM_ERR_NONFINITE)
+    CK(cudaMemsetAsync(ctx->v, 0, (size_t)ctx->p.T * 3 * ctx->levels[ctx->cur].g.N * ctx->es, ctx->stream));
+  return rc;
+}
+
+int store_velocity(lddmm_ctx* ctx, const float* src) {
   const Grid& g = ctx->levels[ctx->cur].g;
   const int64_t n = (int64_t)ctx->p.T * 3 * g.N;
   int rc;
@@ -846,10 +861,15 @@ int lddmm_set_velocity(lddmm_ctx* ctx, const float* src) {
       launch_to_storage(ctx->stage, vptr(ctx, j, g.N), 3 * (int64_t)g.N, ctx->stream, ctx->st);
     }
   }
-  ctx->maps_valid = false;
-  ctx->j0_valid = false;
-  ctx->last_E = -1.0;
   return LDDMM_OK;
+}
+}  // namespace
+
+int lddmm_set_velocity(lddmm_ctx* ctx, const float* src) {
+  if (!ctx || !src) return fail(ctx, LDDMM_ERR_INVALID_ARG, "NULL argument");
+  forget_velocity(ctx);
+  const int rc = store_velocity(ctx, src);
+  return rc ? refused_velocity(ctx, rc) : LDDMM_OK;
 }
 
 int lddmm_get_field(lddmm_ctx* ctx, int which, float* dst) {
@@ -989,9 +1009,10 @@ int lddmm_shoot(lddmm_ctx* ctx, const float* v0) {
   const float dtx = dtv(ctx, L.hx), dty = dtv(ctx, L.hy), dtz = dtv(ctx, L.hz);
   const float ihx2 = 1.0f / (L.hx * L.hx), ihy2 = 1.0f / (L.hy * L.hy), ihz2 = 1.0f / (L.hz * L.hz);
   float* v = reinterpret_cast<float*>(ctx->v);
+  forget_velocity(ctx);
   CK(cudaMemcpyAsync(v, v0, F * sizeof(float), cudaMemcpyDefault, s));
   int rc;
-  if ((rc = check_finite(ctx, v, F, "v0"))) return rc;
+  if ((rc = check_finite(ctx, v, F, "v0"))) return refused_velocity(ctx, rc);
   // m_0 = L (L v_0) in stage
   launch_apply_L3(g, v, ctx->work, nullptr, ctx->p.alpha, ctx->p.gamma, ihx2, ihy2, ihz2, 1.0f, false, s);
   launch_apply_L3(g, ctx->work, ctx->stage, nullptr, ctx->p.alpha, ctx->p.gamma, ihx2, ihy2, ihz2, 1.0f,
@@ -1010,9 +1031,6 @@ int lddmm_shoot(lddmm_ctx* ctx, const float* v0) {
     pf ^= 1;
   }
   CK(cudaGetLastError());
-  ctx->maps_valid = false;
-  ctx->j0_valid = false;
-  ctx->last_E = -1.0;
   return LDDMM_OK;
 }
 
