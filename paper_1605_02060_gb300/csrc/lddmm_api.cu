@@ -830,6 +830,7 @@ void forget_velocity(lddmm_ctx* ctx) {
   ctx->maps_valid = false;
   ctx->j0_valid = false;
   ctx->last_E = -1.0;
+  ctx->have_prev = false;    // backtracking does not go back past it
 }
 
 // After a new v was refused: rc is returned, v is 0 (the check follows the store, in one pass over
