@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "../../include/lddmm.h"
+#include "dft_rows.cuh"
 #include "kernels.h"
 
 namespace lddmm {
@@ -198,8 +199,6 @@ struct FoldArgs {
   float eps;
 };
 
-__device__ __forceinline__ int fold_row_c(int p) { return p ? 2 * p - 1 : 0; }
-
 // FWD: rows m -> pairs p; else pairs p -> rows m.  XAX: lines contiguous along the axis.
 template <bool FWD, bool XAX>
 __global__ void __launch_bounds__(128, 4) k_fold(FoldArgs a) {
@@ -217,6 +216,7 @@ __global__ void __launch_bounds__(128, 4) k_fold(FoldArgs a) {
   const int p0 = blockIdx.y * BP;
   const int c0 = blockIdx.x * FC;
   const int n = a.n, H = a.H;
+  const unsigned n4 = 4u * (unsigned)n;
   float ac[4][8], as[4][8];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -315,9 +315,10 @@ __global__ void __launch_bounds__(128, 4) k_fold(FoldArgs a) {
       if (FWD) {
         // a thread keeps k, its pairs are nt / FK apart
         const int k = tid % FK, m = k0 + k;
+        const char* col = reinterpret_cast<const char*>(a.R + m);
         for (int i = tid / FK; i < BP; i += nt / FK) {
           const int p = p0 + i;
-          const float* rc = a.R + fold_row_c(p) * n + m;
+          const float* rc = reinterpret_cast<const float*>(col + fold_row_bytes(p, n4));
           const bool in = p < H && m < H;
           cp(tb + k * BP + i, rc, in);
           cp(tb + FK * BP + k * BP + i, rc + n, in && p > 0 && 2 * p < n);   // the sin row follows
@@ -325,9 +326,10 @@ __global__ void __launch_bounds__(128, 4) k_fold(FoldArgs a) {
       } else {
         // a thread keeps i, its rows of the contraction are nt / BP apart
         const int m = p0 + ti;
+        const char* col = reinterpret_cast<const char*>(a.R + m);
         for (int k = tk; k < FK; k += tstep) {
           const int p = k0 + k;
-          const float* rc = a.R + fold_row_c(p) * n + m;
+          const float* rc = reinterpret_cast<const float*>(col + fold_row_bytes(p, n4));
           const bool in = p < H && m < H;
           cp(tb + k * BP + ti, rc, in);
           cp(tb + FK * BP + k * BP + ti, rc + n, in && p > 0 && 2 * p < n);
