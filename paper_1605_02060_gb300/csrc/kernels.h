@@ -200,7 +200,15 @@ struct KPlan {
   int* err;  // device flag set by a tensor-core kernel whose bounded wait timed out
   // probes per pipeline wait in the pre-split tensor-core pass (0: the default, 2^22)
   uint32_t poll_limit;
+  bool sym_normal;   // symbol_is_normal of the grid (false: nothing is known)
 };
+// Whether every value of the symbol's square (gamma + alpha lambda)^2 on a grid of this spacing is a
+// normal number with a normal reciprocal, so that a product with the reciprocal may take the
+// division's place.  lambda lies in [0, 4 (hx^-2 + hy^-2 + hz^-2)]; the bounds leave a factor of 4.
+inline bool symbol_is_normal(double hx, double hy, double hz, double alpha, double gamma) {
+  const double top = gamma + alpha * 4.0 * (1.0 / (hx * hx) + 1.0 / (hy * hy) + 1.0 / (hz * hz));
+  return gamma >= 0x1p-62 && top <= 0x1p62;
+}
 // Build device tables for one grid (allocates; free with kplan_destroy).
 cudaError_t kplan_create(KPlan* kp, int nx, int ny, int nz, float hx, float hy, float hz,
                          float alpha, float gamma);

@@ -138,6 +138,7 @@ extern "C" int lddmm_apply_K_noalloc(const float* src, float* dst, int nx, int n
   KPlan kp{};
   kp.nx = nx; kp.ny = ny; kp.nz = nz;
   kp.alpha = alpha; kp.gamma = gamma;
+  kp.sym_normal = symbol_is_normal(hx, hy, hz, alpha, gamma);
   kp.Rx = R[0]; kp.Ry = R[1]; kp.Rz = R[2];
   kp.lx = lam[0]; kp.ly = lam[1]; kp.lz = lam[2];
   cudaError_t e = apply_K(kp, LDDMM_K_FP32, src, dst, work, 1, s);
