@@ -65,6 +65,7 @@ struct KsArgs {
   const float* ly;
   const float* lz;
   float alpha, gamma;
+  int sym_normal;      // KPlan's
   int X, Y;            // zz: line l = (c X + x) Y + y, Y rounded up to 8
   int* err;
   uint32_t poll;       // probes per pipeline wait before the CTA aborts
@@ -123,7 +124,7 @@ __device__ __forceinline__ void split2(float x0, float x1, uint32_t& h, uint32_t
                                                   x1 - __uint_as_float(h & 0xffff0000u));
   l = *reinterpret_cast<const uint32_t*>(&lb);
 }
-// x / y through the hardware reciprocal (y a normal number: the symbol's square)
+// x / y through the hardware reciprocal; y, the square of the symbol, and 1 / y are normal numbers.
 __device__ __forceinline__ float div_fast(float x, float y) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(y));
@@ -255,11 +256,13 @@ __device__ __forceinline__ void store_rows(const KsOut& o, float eps, float* sg,
 // divides by the symbol with the roundings of k_dft_tc, for plain bf16 products on the grids (X no
 // multiple of 4) that come from it: there one FP32 rounding decides bf16 digits, which a
 // registration's iterations carry on.  (Split products keep 16 digits more; their error against
-// FP64 is the same with the faster division, 45 -> 23 us at 141x97x109.)
+// FP64 is the same with the faster division, 45 -> 23 us at 141x97x109.)  It also takes every grid
+// on which the hardware reciprocal does not do: it flushes a subnormal square of the symbol, or one
+// past 2^126, to infinity or 0.
 enum { EPI_T = 0, EPI_ROWS, EPI_ROWS_1, EPI_UPD, EPI_UPD_1, EPI_ZZ, EPI_ZZ_RN, EPI_COUNT };
 
 __host__ __device__ inline int ks_epi(const KsArgs& a) {
-  if (a.zz) return a.split || a.X % 4 == 0 ? EPI_ZZ : EPI_ZZ_RN;
+  if (a.zz) return a.sym_normal && (a.split || a.X % 4 == 0) ? EPI_ZZ : EPI_ZZ_RN;
   if (is_upd_host(a.o.kind)) return a.o.P % 4 == 0 ? EPI_UPD : EPI_UPD_1;
   if (a.o.G == 1) return a.o.P % 4 == 0 ? EPI_ROWS : EPI_ROWS_1;
   return EPI_T;
@@ -868,6 +871,7 @@ cudaError_t ks_axis_pass(const KPlan& kp, int axis, bool inverse, int split, con
   if (o.G == 1 && (o.D != 1 || o.E != 1 || o.F != 1)) return cudaErrorInvalidValue;
   a.lx = kp.lx; a.ly = kp.ly; a.lz = kp.lz;
   a.alpha = kp.alpha; a.gamma = kp.gamma;
+  a.sym_normal = kp.sym_normal;
   a.X = kp.nx; a.Y = ks_pitch(kp.ny);
   a.err = kp.err;
   a.poll = kp.poll_limit ? kp.poll_limit : (1u << 22);
