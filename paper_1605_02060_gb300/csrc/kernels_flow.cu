@@ -430,14 +430,19 @@ static void launch_back_terms(const Grid& g, const float* uc, const void* IM, fl
 //   one, 1 plane     3.1             6.6          26.5                41.5           196
 //   one, 8 planes    10              12           21.6                43             155
 // Blocks of 8 planes pay while the SMs hold them all at once, five each (141x97x109, 910 of them: 32.7
-// us against 15.1 + 14.2); on the large grids the 48 registers leave too few warps in flight.
+// us against 15.1 + 14.2; on the large grids the 48 registers leave too few warps in flight), and from
+// 3.3 of them per SM on: with fewer, the eight planes in a row take longer than two short kernels.  A
+// time step against two kernels' (us, float / bf16 storage; blocks of 8 planes in brackets):
+//   50x77x60 (140) +2.7 / +2.6, 80^3 (300) +2.8 / +1.4, 101x70x125 (468) +1.2 / +0.5,
+//   66x90x110 (504) -0.6 / -0.9, 112x96x96 (576) -2.2 / -3.1, 132x80x114 (750) -3.5 / -5.2.
 template <typename ST>
 static void flow_back(const Grid& g, const ST* vj, const float* u_next, float* u_cur, const void* IM,
                       float* J1, float* W, float dtx, float dty, float dtz, Acc* acc, cudaStream_t s,
                       const Hook& hook, int rk) {
   const int nb = flow_blocks(g);
   const dim3 by8 = flow_grid(g, 8);
-  if (u_next && !rk && (nb <= 256 || by8.x * by8.y * by8.z <= 152 * 5)) {
+  const int nb8 = (int)(by8.x * by8.y * by8.z), sms = sm_count();
+  if (u_next && !rk && (nb <= 256 || (10 * (int64_t)nb8 >= 33 * sms && nb8 <= 5 * sms))) {
     const typename Pair<ST>::T* im = reinterpret_cast<const typename Pair<ST>::T*>(IM);
     hook(KID_BACK_FUSED, 0);
     if (nb <= 256)
