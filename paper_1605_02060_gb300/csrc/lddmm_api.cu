@@ -15,6 +15,7 @@
 
 #include "../../include/lddmm.h"
 #include "kernels.h"
+#include "memory_span.h"
 
 using namespace lddmm;
 
@@ -121,15 +122,39 @@ bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Memory a kernel of the current device reads and writes directly (not another GPU's).
-bool is_local_ptr(const void* p) {
+using AddressRangeFn = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+
+// cuMemGetAddressRange from the driver (nullptr when unavailable).
+AddressRangeFn address_range_fn() {
+  static const AddressRangeFn fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &p, 12000, cudaEnableDefault, &q) ==
+            cudaSuccess &&
+        q == cudaDriverEntryPointSuccess)
+      return reinterpret_cast<AddressRangeFn>(p);
+    cudaGetLastError();
+    return AddressRangeFn(nullptr);
+  }();
+  return fn;
+}
+
+// Whether a kernel of the current device may read and write [p, p + bytes) directly: memory of this
+// GPU (not another's) in one allocation that holds the whole range.  Anything else goes by
+// cudaMemcpyAsync, which checks ranges itself: a buffer that is too short is its error to report.
+bool is_local_span(const void* p, size_t bytes) {
   cudaPointerAttributes a;
   int dev = -1;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == dev);
+  if (a.type != cudaMemoryTypeManaged && (a.type != cudaMemoryTypeDevice || a.device != dev)) return false;
+  const AddressRangeFn range = address_range_fn();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+  return range && range(&base, &size, at) == CUDA_SUCCESS && span_holds(base, size, at, bytes);
 }
 
 // Bounded host wait.  The first two milliseconds poll without sleeping (a sleep of 5 us takes the
@@ -810,8 +835,9 @@ int lddmm_get_velocity(lddmm_ctx* ctx, float* dst) {
   if (!ctx || !dst) return fail(ctx, LDDMM_ERR_INVALID_ARG, "NULL argument");
   const Grid& g = ctx->levels[ctx->cur].g;
   if (ctx->st == 0) return copy_out(ctx, dst, ctx->v, (size_t)ctx->p.T * 3 * g.N * sizeof(float));
-  if (is_local_ptr(dst)) {
-    launch_from_storage(ctx->v, dst, (int64_t)ctx->p.T * 3 * g.N, ctx->stream, ctx->st);
+  const int64_t n = (int64_t)ctx->p.T * 3 * g.N;
+  if (is_local_span(dst, n * sizeof(float))) {
+    launch_from_storage(ctx->v, dst, n, ctx->stream, ctx->st);
     CK(cudaGetLastError());
     return wait_stream(ctx);
   }
@@ -845,7 +871,7 @@ int store_velocity(lddmm_ctx* ctx, const float* src) {
   const Grid& g = ctx->levels[ctx->cur].g;
   const int64_t n = (int64_t)ctx->p.T * 3 * g.N;
   int rc;
-  if (is_local_ptr(src)) {
+  if (is_local_span(src, n * sizeof(float))) {
     // stored and checked in one pass
     CK(cudaMemsetAsync(ctx->flag, 0, sizeof(int), ctx->stream));
     launch_store_checked(src, ctx->v, n, ctx->flag, ctx->stream, ctx->st);
