@@ -9,8 +9,8 @@
 // The surface voxels are listed by 8x8x8 cells (a block per cell counts its voxels, a scan places
 // the cells, a second pass writes each voxel's position within its cell as 9 bits), and a query
 // visits the other surface's cells in shells around its own until the next shell cannot hold
-// anything nearer.  Registered surfaces lie a few voxels apart, so a query meets a few hundred
-// candidates.  Distances are compared in FP32 (every rounding in them is monotone in |dx|, |dy|,
+// anything nearer, or, further away, the cells that its cell cannot rule out.  Registered surfaces
+// lie a few voxels apart, so a query meets a few hundred candidates.  Distances are compared in FP32 (every rounding in them is monotone in |dx|, |dy|,
 // |dz|, so a cell whose nearest corner is no nearer than the best holds nothing nearer) and the
 // winner's distance is recomputed in FP64.  The order statistics are found by radix selection on
 // the bit patterns of the (non-negative) FP64 distances.
@@ -115,14 +115,30 @@ __global__ void __launch_bounds__(1024) k_cell_scan(unsigned* __restrict__ start
 
 // d[mask][i] = distance (physical units, FP64) from surface voxel i of the mask (blockIdx.y, in
 // list order) to the nearest surface voxel of the other.  One block per cell; a thread takes a
-// voxel of the cell.  What it costs is the candidates' FP32 arithmetic: at 264x160x228 (6e4
-// voxels each) both directions take 34 us, against 5.1 ms for comparing every pair.
+// voxel of the cell.  It looks in the cells around its own, shell by shell; what that costs is the
+// candidates' FP32 arithmetic: at 264x160x228 (6e4 voxels each, a few voxels apart) both directions
+// take 34 us, against 5.1 ms for comparing every pair.  Past kNearShells the empty cells of the shells
+// would be most of the work: there the block passes over all cells once, for the least distance at
+// which some cell is sure to hold a voxel, and again for the cells that may hold a nearer one, and its
+// voxels look in those only.  Surfaces far apart at 264x160x228 (us a call; every pair / all shells /
+// this way): ellipsoids at opposite ends 1329 / 6147 / 419, the first face against the last 3701 /
+// 7987 / 1929, a voxel in either corner 264 / 3610 / 213, an ellipsoid and a corner 4733 / 7333 / 379.
+constexpr int kNearShells = 2, kCand = 512, kFewOpen = 4;
+
+__device__ __forceinline__ float dist2(int ix, int iy, int iz, float hx, float hy, float hz) {
+  const float x = (float)ix * hx, y = (float)iy * hy, z = (float)iz * hz;
+  return fmaf(x, x, fmaf(y, y, z * z));
+}
+
 __global__ void __launch_bounds__(64) k_nearest(Grid g, CellGrid cg,
                                                 const unsigned* __restrict__ start,
                                                 const uint16_t* __restrict__ list, unsigned nA,
                                                 float hx, float hy, float hz,
                                                 double* __restrict__ dA, double* __restrict__ dB) {
-  const int c = blockIdx.x, side = blockIdx.y;
+  __shared__ int cand[3][kCand];       // cells that may hold the nearest voxel of some query
+  __shared__ unsigned wcnt[2];
+  __shared__ float wmin[2];
+  const int c = blockIdx.x, side = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
   const unsigned* sq = start + side * (size_t)(cg.ncell + 1);
   const unsigned* so = start + (side ^ 1) * (size_t)(cg.ncell + 1);
   const uint16_t* lq = list + (side ? nA : 0u);
@@ -133,64 +149,178 @@ __global__ void __launch_bounds__(64) k_nearest(Grid g, CellGrid cg,
   const int cx = c % cg.ncx, cy = (c / cg.ncx) % cg.ncy, cz = c / (cg.ncx * cg.ncy);
   const int rmax = max(max(max(cx, cg.ncx - 1 - cx), max(cy, cg.ncy - 1 - cy)),
                        max(cz, cg.ncz - 1 - cz));
-  for (unsigned i = q0 + threadIdx.x; i < q1; i += blockDim.x) {
-    const unsigned code = lq[i];
+  float ub = -1.f;                     // far cells: the bound (once it is known),
+  int ncand = -1;                      // and the cells within it, when cand holds all of them
+  for (unsigned base = q0; base < q1; base += 64) {
+    const unsigned i = base + tid;
+    const bool on = i < q1;
+    const unsigned code = on ? lq[i] : 0u;
     const int px = cx * kCell + (code & 7), py = cy * kCell + ((code >> 3) & 7),
               pz = cz * kCell + (code >> 6);
-    float best = 3.0e38f;
-    int wx = 0, wy = 0, wz = 0;
-    for (int r = 0; r <= rmax; ++r) {
+    // the nearest voxel so far of the query at (x, y, z)
+    struct Near {
+      float best;
+      int x, y, z;
+    };
+    // the voxels of cell (x, y, z), which has some, unless none can be nearer
+    auto look = [&](Near& w, int qx, int qy, int qz, int x, int y, int z) {
+      const int oc = (z * cg.ncy + y) * cg.ncx + x;
+      const int bx = max(max(x * kCell - qx, qx - (x * kCell + kCell - 1)), 0),
+                by = max(max(y * kCell - qy, qy - (y * kCell + kCell - 1)), 0),
+                bz = max(max(z * kCell - qz, qz - (z * kCell + kCell - 1)), 0);
+      if (dist2(bx, by, bz, hx, hy, hz) >= w.best) return;
+      for (unsigned k = so[oc], p1 = so[oc + 1]; k < p1; ++k) {
+        const unsigned oq = __ldg(lo + k);
+        const int ox = x * kCell + (oq & 7), oy = y * kCell + ((oq >> 3) & 7),
+                  oz = z * kCell + (oq >> 6);
+        const float d2 = dist2(qx - ox, qy - oy, qz - oz, hx, hy, hz);
+        if (d2 < w.best) w = Near{d2, ox, oy, oz};
+      }
+    };
+    Near w{3.0e38f, 0, 0, 0};
+    bool open = on;                    // a nearer voxel may lie beyond the shells
+    for (int r = 0; open; ++r) {
+      if (r > rmax) {
+        open = false;
+        break;
+      }
       if (r > 0) {
         // the nearest a voxel of shell r or beyond can lie: past one of the faces of shell r - 1
         const int e = (r - 1) * kCell;
-        float b = 3.0e38f;
         const float fx = (float)min(px - (cx * kCell - e) + 1, cx * kCell + kCell + e - px) * hx;
         const float fy = (float)min(py - (cy * kCell - e) + 1, cy * kCell + kCell + e - py) * hy;
         const float fz = (float)min(pz - (cz * kCell - e) + 1, cz * kCell + kCell + e - pz) * hz;
-        b = fminf(fx, fminf(fy, fz));
-        if (b * b >= best) break;
+        const float b = fminf(fx, fminf(fy, fz));
+        if (b * b >= w.best) {
+          open = false;
+          break;
+        }
       }
+      if (r > kNearShells) break;
       const int z0 = max(cz - r, 0), z1 = min(cz + r, cg.ncz - 1);
       const int y0 = max(cy - r, 0), y1 = min(cy + r, cg.ncy - 1);
       for (int z = z0; z <= z1; ++z) {
         const int bz = max(max(z * kCell - pz, pz - (z * kCell + kCell - 1)), 0);
-        const float gz = (float)bz * hz;
         for (int y = y0; y <= y1; ++y) {
           const int by = max(max(y * kCell - py, py - (y * kCell + kCell - 1)), 0);
-          const float gy = (float)by * hy;
-          const float gyz = fmaf(gy, gy, gz * gz);
-          if (gyz >= best) continue;
+          if (dist2(0, by, bz, hx, hy, hz) >= w.best) continue;
           const bool face = z - cz == r || cz - z == r || y - cy == r || cy - y == r;
           const int step = face || r == 0 ? 1 : 2 * r;
           for (int x = cx - r; x <= cx + r; x += step) {
             if (x < 0 || x >= cg.ncx) continue;
             const int oc = (z * cg.ncy + y) * cg.ncx + x;
-            const unsigned p0 = so[oc], p1 = so[oc + 1];
-            if (p0 == p1) continue;
-            const int bx = max(max(x * kCell - px, px - (x * kCell + kCell - 1)), 0);
-            const float gx = (float)bx * hx;
-            if (fmaf(gx, gx, gyz) >= best) continue;
-            for (unsigned k = p0; k < p1; ++k) {
-              const unsigned oq = __ldg(lo + k);
-              const int qx = x * kCell + (oq & 7), qy = y * kCell + ((oq >> 3) & 7),
-                        qz = z * kCell + (oq >> 6);
-              const float dx = (float)(px - qx) * hx, dy = (float)(py - qy) * hy,
-                          dz = (float)(pz - qz) * hz;
-              const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-              if (d2 < best) {
-                best = d2;
-                wx = qx;
-                wy = qy;
-                wz = qz;
-              }
-            }
+            if (so[oc] != so[oc + 1]) look(w, px, py, pz, x, y, z);
           }
         }
       }
     }
-    const double dx = (double)(px - wx) * hx, dy = (double)(py - wy) * hy,
-                 dz = (double)(pz - wz) * hz;
-    d[i] = sqrt(dx * dx + dy * dy + dz * dz);
+    if (__syncthreads_or(open)) {
+      // of cell o (o >= ncell: none): has it voxels?
+      auto some = [&](int o) { return o < cg.ncell && so[o] != so[o + 1]; };
+      auto decode = [&](int o, int& x, int& y, int& z) {
+        const int t = o / cg.ncx;
+        x = o - t * cg.ncx;
+        z = t / cg.ncy;
+        y = t - z * cg.ncy;
+      };
+      if (ub < 0.f) {
+        float u = 3.0e38f;
+        for (int o0 = tid; o0 < cg.ncell; o0 += 4 * 64) {
+          bool has[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) has[k] = some(o0 + k * 64);
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (has[k]) {
+              int x, y, z;
+              decode(o0 + k * 64, x, y, z);
+              // no voxel of the one cell is further from one of the other than their far corners
+              u = fminf(u, dist2(kCell * abs(x - cx) + kCell - 1, kCell * abs(y - cy) + kCell - 1,
+                                 kCell * abs(z - cz) + kCell - 1, hx, hy, hz));
+            }
+        }
+        for (int o = 16; o; o >>= 1) u = fminf(u, __shfl_xor_sync(0xffffffffu, u, o));
+        if (lane == 0) wmin[tid >> 5] = u;
+        __syncthreads();
+        ub = fminf(wmin[0], wmin[1]);
+      }
+      // some voxel lies within the bound: a query that knows none looks for any up to it
+      if (open && w.best > ub) w.best = __uint_as_float(__float_as_uint(ub) + 1u);
+      auto look_in = [&](int n) {      // the first n candidates, by the open queries
+        unsigned mine = __ballot_sync(0xffffffffu, open);
+        if (__popc(mine) > kFewOpen) {
+          if (open)
+            for (int k = 0; k < n; ++k) look(w, px, py, pz, cand[0][k], cand[1][k], cand[2][k]);
+          return;
+        }
+        // a warp with few open queries takes them one by one, a lane every 32nd cell
+        for (; mine; mine &= mine - 1) {
+          const int src = __ffs(mine) - 1;
+          const int qx = __shfl_sync(0xffffffffu, px, src), qy = __shfl_sync(0xffffffffu, py, src),
+                    qz = __shfl_sync(0xffffffffu, pz, src);
+          Near t{__shfl_sync(0xffffffffu, w.best, src), 0, 0, 0};
+          const float had = t.best;
+          for (int k = lane; k < n; k += 32) look(t, qx, qy, qz, cand[0][k], cand[1][k], cand[2][k]);
+          const unsigned m = __reduce_min_sync(0xffffffffu, __float_as_uint(t.best));
+          const int from = __ffs(__ballot_sync(0xffffffffu, __float_as_uint(t.best) == m)) - 1;
+          const Near f{__uint_as_float(m), __shfl_sync(0xffffffffu, t.x, from),
+                       __shfl_sync(0xffffffffu, t.y, from), __shfl_sync(0xffffffffu, t.z, from)};
+          if (lane == src && f.best < had) w = f;
+        }
+      };
+      if (ncand >= 0) {
+        look_in(ncand);
+      } else {
+        int n = 0;
+        bool all = true;
+        for (int o0 = 0; o0 < cg.ncell; o0 += 4 * 64) {
+          bool in[4];
+          int x[4], y[4], z[4];
+          unsigned b[4], m = 0;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) in[k] = some(o0 + k * 64 + tid);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (in[k]) {
+              decode(o0 + k * 64 + tid, x[k], y[k], z[k]);
+              in[k] = dist2(max(kCell * abs(x[k] - cx) - (kCell - 1), 0),
+                            max(kCell * abs(y[k] - cy) - (kCell - 1), 0),
+                            max(kCell * abs(z[k] - cz) - (kCell - 1), 0), hx, hy, hz) <= ub;
+            }
+            b[k] = __ballot_sync(0xffffffffu, in[k]);
+            m += __popc(b[k]);
+          }
+          if (lane == 0) wcnt[tid >> 5] = m;
+          __syncthreads();
+          int at = n + (tid >= 32 ? (int)wcnt[0] : 0);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            if (in[k]) {
+              const int e = at + __popc(b[k] & ((1u << lane) - 1u));
+              cand[0][e] = x[k];
+              cand[1][e] = y[k];
+              cand[2][e] = z[k];
+            }
+            at += __popc(b[k]);
+          }
+          n += (int)(wcnt[0] + wcnt[1]);
+          __syncthreads();
+          if (n > kCand - 4 * 64) {
+            look_in(n);
+            __syncthreads();
+            n = 0;
+            all = false;
+          }
+        }
+        look_in(n);
+        if (all) ncand = n;
+      }
+    }
+    if (on) {
+      const double dx = (double)(px - w.x) * hx, dy = (double)(py - w.y) * hy,
+                   dz = (double)(pz - w.z) * hz;
+      d[i] = sqrt(dx * dx + dy * dy + dz * dz);
+    }
   }
 }
 
