@@ -121,8 +121,9 @@ __global__ void __launch_bounds__(1024) k_cell_scan(unsigned* __restrict__ start
 // would be most of the work: there the block passes over all cells once, for the least distance at
 // which some cell is sure to hold a voxel, and again for the cells that may hold a nearer one, and its
 // voxels look in those only.  Surfaces far apart at 264x160x228 (us a call; every pair / all shells /
-// this way): ellipsoids at opposite ends 1329 / 6147 / 419, the first face against the last 3701 /
-// 7987 / 1929, a voxel in either corner 264 / 3610 / 213, an ellipsoid and a corner 4733 / 7333 / 379.
+// this way): ellipsoids at opposite ends 1329 / 6147 / 453, the first face against the last 3701 /
+// 7987 / 2156, a voxel in either corner 264 / 3610 / 211, an ellipsoid and a corner 4733 / 7333 / 343.
+// (20 blocks on an SM: registers and candidates as three coordinates, 6 KB, cost the near search 1 us.)
 constexpr int kNearShells = 2, kCand = 512, kFewOpen = 4;
 
 __device__ __forceinline__ float dist2(int ix, int iy, int iz, float hx, float hy, float hz) {
@@ -130,12 +131,12 @@ __device__ __forceinline__ float dist2(int ix, int iy, int iz, float hx, float h
   return fmaf(x, x, fmaf(y, y, z * z));
 }
 
-__global__ void __launch_bounds__(64) k_nearest(Grid g, CellGrid cg,
+__global__ void __launch_bounds__(64, 20) k_nearest(Grid g, CellGrid cg,
                                                 const unsigned* __restrict__ start,
                                                 const uint16_t* __restrict__ list, unsigned nA,
                                                 float hx, float hy, float hz,
                                                 double* __restrict__ dA, double* __restrict__ dB) {
-  __shared__ int cand[3][kCand];       // cells that may hold the nearest voxel of some query
+  __shared__ int cand[kCand];          // cells that may hold the nearest voxel of some query
   __shared__ unsigned wcnt[2];
   __shared__ float wmin[2];
   const int c = blockIdx.x, side = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
@@ -162,20 +163,22 @@ __global__ void __launch_bounds__(64) k_nearest(Grid g, CellGrid cg,
       float best;
       int x, y, z;
     };
-    // the voxels of cell (x, y, z), which has some, unless none can be nearer
-    auto look = [&](Near& w, int qx, int qy, int qz, int x, int y, int z) {
-      const int oc = (z * cg.ncy + y) * cg.ncx + x;
-      const int bx = max(max(x * kCell - qx, qx - (x * kCell + kCell - 1)), 0),
-                by = max(max(y * kCell - qy, qy - (y * kCell + kCell - 1)), 0),
-                bz = max(max(z * kCell - qz, qz - (z * kCell + kCell - 1)), 0);
-      if (dist2(bx, by, bz, hx, hy, hz) >= w.best) return;
-      for (unsigned k = so[oc], p1 = so[oc + 1]; k < p1; ++k) {
+    // the voxels p0 .. p1 - 1 of the list, of cell (x, y, z)
+    auto scan = [&](Near& w, int qx, int qy, int qz, unsigned p0, unsigned p1, int x, int y, int z) {
+      for (unsigned k = p0; k < p1; ++k) {
         const unsigned oq = __ldg(lo + k);
         const int ox = x * kCell + (oq & 7), oy = y * kCell + ((oq >> 3) & 7),
                   oz = z * kCell + (oq >> 6);
         const float d2 = dist2(qx - ox, qy - oy, qz - oz, hx, hy, hz);
         if (d2 < w.best) w = Near{d2, ox, oy, oz};
       }
+    };
+    // cell oc at (x, y, z), unless nothing in it can be nearer
+    auto look = [&](Near& w, int qx, int qy, int qz, int oc, int x, int y, int z) {
+      const int bx = max(max(x * kCell - qx, qx - (x * kCell + kCell - 1)), 0),
+                by = max(max(y * kCell - qy, qy - (y * kCell + kCell - 1)), 0),
+                bz = max(max(z * kCell - qz, qz - (z * kCell + kCell - 1)), 0);
+      if (dist2(bx, by, bz, hx, hy, hz) < w.best) scan(w, qx, qy, qz, so[oc], so[oc + 1], x, y, z);
     };
     Near w{3.0e38f, 0, 0, 0};
     bool open = on;                    // a nearer voxel may lie beyond the shells
@@ -201,15 +204,21 @@ __global__ void __launch_bounds__(64) k_nearest(Grid g, CellGrid cg,
       const int y0 = max(cy - r, 0), y1 = min(cy + r, cg.ncy - 1);
       for (int z = z0; z <= z1; ++z) {
         const int bz = max(max(z * kCell - pz, pz - (z * kCell + kCell - 1)), 0);
+        const float gz = (float)bz * hz;
         for (int y = y0; y <= y1; ++y) {
           const int by = max(max(y * kCell - py, py - (y * kCell + kCell - 1)), 0);
-          if (dist2(0, by, bz, hx, hy, hz) >= w.best) continue;
+          const float gy = (float)by * hy, gyz = fmaf(gy, gy, gz * gz);
+          if (gyz >= w.best) continue;
           const bool face = z - cz == r || cz - z == r || y - cy == r || cy - y == r;
           const int step = face || r == 0 ? 1 : 2 * r;
           for (int x = cx - r; x <= cx + r; x += step) {
             if (x < 0 || x >= cg.ncx) continue;
             const int oc = (z * cg.ncy + y) * cg.ncx + x;
-            if (so[oc] != so[oc + 1]) look(w, px, py, pz, x, y, z);
+            const unsigned p0 = so[oc], p1 = so[oc + 1];
+            if (p0 == p1) continue;
+            const int bx = max(max(x * kCell - px, px - (x * kCell + kCell - 1)), 0);
+            const float gx = (float)bx * hx;
+            if (fmaf(gx, gx, gyz) < w.best) scan(w, px, py, pz, p0, p1, x, y, z);
           }
         }
       }
@@ -249,8 +258,11 @@ __global__ void __launch_bounds__(64) k_nearest(Grid g, CellGrid cg,
       auto look_in = [&](int n) {      // the first n candidates, by the open queries
         unsigned mine = __ballot_sync(0xffffffffu, open);
         if (__popc(mine) > kFewOpen) {
-          if (open)
-            for (int k = 0; k < n; ++k) look(w, px, py, pz, cand[0][k], cand[1][k], cand[2][k]);
+          for (int k = 0; k < n; ++k) {
+            int x, y, z;
+            decode(cand[k], x, y, z);
+            if (open) look(w, px, py, pz, cand[k], x, y, z);
+          }
           return;
         }
         // a warp with few open queries takes them one by one, a lane every 32nd cell
@@ -260,7 +272,11 @@ __global__ void __launch_bounds__(64) k_nearest(Grid g, CellGrid cg,
                     qz = __shfl_sync(0xffffffffu, pz, src);
           Near t{__shfl_sync(0xffffffffu, w.best, src), 0, 0, 0};
           const float had = t.best;
-          for (int k = lane; k < n; k += 32) look(t, qx, qy, qz, cand[0][k], cand[1][k], cand[2][k]);
+          for (int k = lane; k < n; k += 32) {
+            int x, y, z;
+            decode(cand[k], x, y, z);
+            look(t, qx, qy, qz, cand[k], x, y, z);
+          }
           const unsigned m = __reduce_min_sync(0xffffffffu, __float_as_uint(t.best));
           const int from = __ffs(__ballot_sync(0xffffffffu, __float_as_uint(t.best) == m)) - 1;
           const Near f{__uint_as_float(m), __shfl_sync(0xffffffffu, t.x, from),
@@ -275,17 +291,16 @@ __global__ void __launch_bounds__(64) k_nearest(Grid g, CellGrid cg,
         bool all = true;
         for (int o0 = 0; o0 < cg.ncell; o0 += 4 * 64) {
           bool in[4];
-          int x[4], y[4], z[4];
           unsigned b[4], m = 0;
 #pragma unroll
           for (int k = 0; k < 4; ++k) in[k] = some(o0 + k * 64 + tid);
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             if (in[k]) {
-              decode(o0 + k * 64 + tid, x[k], y[k], z[k]);
-              in[k] = dist2(max(kCell * abs(x[k] - cx) - (kCell - 1), 0),
-                            max(kCell * abs(y[k] - cy) - (kCell - 1), 0),
-                            max(kCell * abs(z[k] - cz) - (kCell - 1), 0), hx, hy, hz) <= ub;
+              int x, y, z;
+              decode(o0 + k * 64 + tid, x, y, z);
+              in[k] = dist2(max(kCell * abs(x - cx) - (kCell - 1), 0), max(kCell * abs(y - cy) - (kCell - 1), 0),
+                            max(kCell * abs(z - cz) - (kCell - 1), 0), hx, hy, hz) <= ub;
             }
             b[k] = __ballot_sync(0xffffffffu, in[k]);
             m += __popc(b[k]);
@@ -295,12 +310,7 @@ __global__ void __launch_bounds__(64) k_nearest(Grid g, CellGrid cg,
           int at = n + (tid >= 32 ? (int)wcnt[0] : 0);
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            if (in[k]) {
-              const int e = at + __popc(b[k] & ((1u << lane) - 1u));
-              cand[0][e] = x[k];
-              cand[1][e] = y[k];
-              cand[2][e] = z[k];
-            }
+            if (in[k]) cand[at + __popc(b[k] & ((1u << lane) - 1u))] = o0 + k * 64 + tid;
             at += __popc(b[k]);
           }
           n += (int)(wcnt[0] + wcnt[1]);
