@@ -128,10 +128,11 @@ void launch_from_storage(const void* src, float* dst, int64_t n, cudaStream_t s,
 // *flag |= bit when a[0..n) holds a NaN or an infinity.
 void launch_check_finite(const float* a, int64_t n, int* flag, cudaStream_t s, int bit = 1);
 void launch_fill(float* a, int64_t n, float value, cudaStream_t s);
-// hist (3 x 65536, zeroed): voxels per label of A, of B and of both at once; out = mean Dice over
-// the labels > 0 present in either (1 when there are none).
-void launch_dice(const uint16_t* A, const uint16_t* B, int64_t n,
-                 unsigned long long* hist /* 3 x 65536 */, double* out, cudaStream_t s);
+// hist (kDiceWords, the first kDiceZero of them zeroed): voxels per label of A, of B and of both at
+// once, 65536 each, and the mean's scratch; out = mean Dice over the labels > 0 present in either (1 when there are none).
+constexpr int kDiceBlocks = 64, kDiceZero = 3 * 65536 + 2, kDiceWords = kDiceZero + 2 * kDiceBlocks;
+void launch_dice(const uint16_t* A, const uint16_t* B, int64_t n, unsigned long long* hist,
+                 double* out, cudaStream_t s);
 
 // ---- registration-quality measures of §2.7 (kernels_metrics.cu) ----
 // 8x8x8-voxel cells of a grid.

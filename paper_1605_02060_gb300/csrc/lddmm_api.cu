@@ -59,7 +59,7 @@ struct lddmm_ctx {
   Acc* acc_init = nullptr;  // the accumulators' start value (device copy, written at creation)
   Acc* acc_host = nullptr;  // pinned
   int* flag = nullptr;      // device int
-  unsigned long long* hist = nullptr;  // 3 x 65536, the largest label, the mean Dice
+  unsigned long long* hist = nullptr;  // kDiceWords, the mean Dice
   // map state
   const float* u10 = nullptr;
   const float* u01 = nullptr;
@@ -728,7 +728,7 @@ int lddmm_create(const lddmm_params* p, const float* I0, const float* I1, const 
        A(dalloc(&ctx->J1, T * N)) && A(dalloc(&ctx->W, T * N)) && A(dalloc(&ctx->b, ctx->kcap)) &&
        A(dalloc(&ctx->work, ctx->kcap)) && A(dalloc(&ctx->J0T, N)) && A(dalloc(&ctx->stage, 3 * N + 64 + surface_select_bytes() / 4)) &&
        A(dalloc(&ctx->acc, 1)) && A(dalloc(&ctx->acc_init, 1)) && A(dalloc(&ctx->flag, 1)) &&
-       A(dalloc(&ctx->hist, 3 * 65536 + 2)) &&
+       A(dalloc(&ctx->hist, kDiceWords + 1)) &&
        A(cudaMallocHost((void**)&ctx->acc_host, sizeof(Acc)));
   if (ok && (p->flags & 1)) ok = A(dalloc(&ctx->v_prev, ve));
   g_fail_alloc_countdown = 0;
@@ -959,9 +959,9 @@ int lddmm_dice(lddmm_ctx* ctx, const uint16_t* A, const uint16_t* B, int64_t n, 
     if (!da) { CK(cudaMemcpyAsync(tmp, A, n * 2, cudaMemcpyDefault, ctx->stream)); a = tmp; }
     if (!db) { CK(cudaMemcpyAsync(tmp + n, B, n * 2, cudaMemcpyDefault, ctx->stream)); b = tmp + n; }
   }
-  CK(cudaMemsetAsync(ctx->hist, 0, (3 * 65536 + 1) * sizeof(unsigned long long), ctx->stream));
+  CK(cudaMemsetAsync(ctx->hist, 0, kDiceZero * sizeof(unsigned long long), ctx->stream));
   // the mean goes through the pinned accumulator block (free outside an energy read)
-  double* mean = reinterpret_cast<double*>(ctx->hist + 3 * 65536 + 1);
+  double* mean = reinterpret_cast<double*>(ctx->hist + kDiceWords);
   launch_dice(a, b, n, ctx->hist, mean, ctx->stream);
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(ctx->acc_host, mean, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
