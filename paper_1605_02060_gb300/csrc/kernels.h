@@ -67,9 +67,10 @@ enum KernelId {
 // backward sweep (launch_flow_back), the map phi_{0,1} it leaves and the steps of a forward sweep
 // without the residual use the quad layout, the iteration's forward sweep (launch_fwd_fused) and
 // phi_{1,0} the planar one.
-// Backward sweep step j (quad maps): u_cur = dt v_j / h + u_next(x + dt v_j / h) (u_next == nullptr:
-// id) and, unless u_next is null, the terms of u_next = phi_{j+1,1} - id: J1 = I1 o phi, W = (M o phi)
-// det(I + Du_next), min det into acc.  launch_back_last: the terms of u = phi_{0,1} - id.  IM holds I1 and M interleaved as pairs (launch_interleave).
+// Backward sweep step j (quad maps): u_cur = dt v_j / h + u_next(x + dt v_j / h) (u_next ==
+// nullptr: id) and, unless u_next is null, the terms of u_next = phi_{j+1,1} - id: J1 = I1 o phi,
+// W = (M o phi) det(I + Du_next), min det into acc.  launch_back_last: the terms of
+// u = phi_{0,1} - id.  IM holds I1 and M interleaved as pairs (launch_interleave).
 void launch_flow_back(const Grid& g, const void* vj, const float* u_next, float* u_cur,
                       const void* IM, float* J1, float* W, float dtx, float dty, float dtz,
                       Acc* acc, cudaStream_t s, const Hook& hook, int st, int rk = 0);
@@ -80,13 +81,13 @@ void launch_interleave(const void* a, const void* b, void* out, int64_t n, cudaS
                        int st);
 // Forward sweep step j: u_next = -dt v_j / h + u_cur(x - dt v_j / h) (u_cur == nullptr: id);
 // if last, J0_T = I0 o (id + u_next) and E_data.  quad: u_cur and u_next in the quad layout, but
-// the last u_next planar.
+// the last u_next planar; else all planar, for float fields and one lookup a step only.
 void launch_fwd_flow(const Grid& g, const void* vj, const float* u_cur, float* u_next,
                      float dtx, float dty, float dtz, bool last, const void* I0, const void* I1,
                      const void* M, float* J0T, Acc* acc, cudaStream_t s, int st, int rk = 0,
                      int quad = 0);
-// Forward sweep step j (planar maps) in one pass over u_cur = phi_{j,0} - id (nullptr: id): the residual
-// b = c W_j (J0_j - J1_j) grad J0_j / h with J0_j = I0 o (id + u_cur) (bsplit 0: b as 3 fp32
+// Forward sweep step j (planar maps) in one pass over u_cur = phi_{j,0} - id (nullptr: id): the
+// residual b = c W_j (J0_j - J1_j) grad J0_j / h with J0_j = I0 o (id + u_cur) (bsplit 0: b as 3 fp32
 // fields; 1 / 2: b split for the pre-split K, bf16 hi plane / hi and lo planes, rows of pitch
 // px), and u_next as launch_fwd_flow (without J0_T and E_data: launch_j0_edata gives them).
 void launch_fwd_fused(const Grid& g, const void* vj, const float* u_cur, float* u_next,
@@ -101,14 +102,13 @@ void launch_ereg(const Grid& g, const void* v, int T, float alpha, float gamma, 
                  float ihy2, float ihz2, Acc* acc, cudaStream_t s, int st);
 // v_j <- v_j - eps (2 v_j - Kb), 3 components.
 void launch_update(const Grid& g, void* vj, const float* Kb, float eps, cudaStream_t s, int st);
-// Displacement of phi_{1,0} / phi_{0,1} only (flows without the residual), to refresh maps.
-// rk = 1: RK4 along each step (v_j held over the step) instead of one lookup.
-void launch_flow_only_fwd(const Grid& g, const void* vj, const float* u_cur, float* u_next,
-                          float dtx, float dty, float dtz, cudaStream_t s, int st, int rk = 0,
-                          int quad = 0);
+// Displacement of phi_{1,0} (planar) / phi_{0,1} (quad) only: flows without the residual, to
+// recompute or refresh maps.  rk = 1: RK4 along each step (v_j held over the step) instead of one
+// lookup.
+void launch_flow_only_fwd(const Grid& g, const float* vj, const float* u_cur, float* u_next,
+                          float dtx, float dty, float dtz, cudaStream_t s);
 void launch_flow_only_back(const Grid& g, const void* vj, const float* u_next, float* u_cur,
-                           float dtx, float dty, float dtz, cudaStream_t s, int st, int rk = 0,
-                           int quad = 0);
+                           float dtx, float dty, float dtz, cudaStream_t s, int st, int rk = 0);
 // A map in the quad layout ([N] x (u_x, u_y, u_z, 0), the iteration's sweeps) to the planar one
 // ([3][N]).
 void launch_quad_to_planar(const float* quad, float* planar, int64_t n, cudaStream_t s);

@@ -9,8 +9,9 @@
 //   update          v_j <- v_j - eps (2 v_j - K b_j).
 // Maps are displacements u = phi - id in voxels; dt v / h converts a velocity to voxels.
 // The velocity field and the images are stored as ST = float or bf16 (the precision form);
-// every computation is FP32 and reductions are FP64.  Kernels run on (32, 8) blocks over a
-// (ceil(nx/32), ceil(ny/8), nz) grid: rows of x are coalesced and no voxel index is divided.
+// every computation is FP32 and reductions are FP64.  Kernels run on (32, 8) blocks over the x-y
+// plane, a thread for a voxel or marching up a few planes: rows of x are coalesced and no voxel
+// index is divided.
 #include "kernels.h"
 
 namespace lddmm {
@@ -174,12 +175,15 @@ template <typename ST, int SGN, bool Q, int ZC>
 static void launch_disp_march_z(const Grid& g, const void* vj, const float* uin, float* uout,
                                 float dtx, float dty, float dtz, cudaStream_t s, int rk) {
   const dim3 grid = flow_grid(g, ZC);
-  if (rk)
-    k_disp_march<ST, SGN, ZC, true, Q><<<grid, kBlock3d, 0, s>>>(g, (const ST*)vj, uin, uout, dtx,
-                                                                 dty, dtz);
-  else
-    k_disp_march<ST, SGN, ZC, false, Q><<<grid, kBlock3d, 0, s>>>(g, (const ST*)vj, uin, uout, dtx,
-                                                                  dty, dtz);
+  if constexpr (Q) {       // (planar maps take one lookup a step)
+    if (rk) {
+      k_disp_march<ST, SGN, ZC, true, Q><<<grid, kBlock3d, 0, s>>>(g, (const ST*)vj, uin, uout, dtx,
+                                                                   dty, dtz);
+      return;
+    }
+  }
+  k_disp_march<ST, SGN, ZC, false, Q><<<grid, kBlock3d, 0, s>>>(g, (const ST*)vj, uin, uout, dtx,
+                                                                dty, dtz);
 }
 
 template <typename ST, int SGN, bool Q>
@@ -191,22 +195,16 @@ static void launch_disp_march(const Grid& g, const void* vj, const float* uin, f
     launch_disp_march_z<ST, SGN, Q, kFlowZ>(g, vj, uin, uout, dtx, dty, dtz, s, rk);
 }
 
-template <bool Q>
-static void disp_step_l(int sgn, const Grid& g, const void* vj, const float* uin, float* uout,
-                        float dtx, float dty, float dtz, cudaStream_t s, int st, int rk) {
-  if (sgn > 0) {
-    if (st) launch_disp_march<__nv_bfloat16, 1, Q>(g, vj, uin, uout, dtx, dty, dtz, s, rk);
-    else launch_disp_march<float, 1, Q>(g, vj, uin, uout, dtx, dty, dtz, s, rk);
-  } else {
-    if (st) launch_disp_march<__nv_bfloat16, -1, Q>(g, vj, uin, uout, dtx, dty, dtz, s, rk);
-    else launch_disp_march<float, -1, Q>(g, vj, uin, uout, dtx, dty, dtz, s, rk);
-  }
-}
-
+// One step of a map in the quad layout.
 static void disp_step(int sgn, const Grid& g, const void* vj, const float* uin, float* uout,
-                      float dtx, float dty, float dtz, cudaStream_t s, int st, int rk, int quad) {
-  if (quad) disp_step_l<true>(sgn, g, vj, uin, uout, dtx, dty, dtz, s, st, rk);
-  else disp_step_l<false>(sgn, g, vj, uin, uout, dtx, dty, dtz, s, st, rk);
+                      float dtx, float dty, float dtz, cudaStream_t s, int st, int rk) {
+  if (sgn > 0) {
+    if (st) launch_disp_march<__nv_bfloat16, 1, true>(g, vj, uin, uout, dtx, dty, dtz, s, rk);
+    else launch_disp_march<float, 1, true>(g, vj, uin, uout, dtx, dty, dtz, s, rk);
+  } else {
+    if (st) launch_disp_march<__nv_bfloat16, -1, true>(g, vj, uin, uout, dtx, dty, dtz, s, rk);
+    else launch_disp_march<float, -1, true>(g, vj, uin, uout, dtx, dty, dtz, s, rk);
+  }
 }
 
 // Backward sweep, part 2: J1_j = I1 o phi_{j,1}, W_j = (M o phi_{j,1}) det D phi_{j,1}.
@@ -263,7 +261,7 @@ __device__ __forceinline__ Sides sides_of(const Grid& g, int x, int y) {
   s.iy = (y > 0 && y < g.ny - 1) ? 0.5f : 1.0f;
   return s;
 }
-template <bool Q, typename PT>
+template <typename PT>
 __device__ __forceinline__ float back_terms_at(const Grid& g, const float* __restrict__ uc,
                                                const PT* __restrict__ IM, float* __restrict__ J1j,
                                                float* __restrict__ Wj, int x, int y, int z,
@@ -273,10 +271,10 @@ __device__ __forceinline__ float back_terms_at(const Grid& g, const float* __res
   float D[3][3];
   const float iz = (z > 0 && z < g.nz - 1) ? 0.5f : 1.0f;
   {
-    const float3 xh = MapL<Q>::at(uc, g.N, zp + y * g.nx + sd.xhi);
-    const float3 xl = MapL<Q>::at(uc, g.N, zp + y * g.nx + sd.xlo);
-    const float3 yh = MapL<Q>::at(uc, g.N, zp + sd.yhi * g.nx + x);
-    const float3 yl = MapL<Q>::at(uc, g.N, zp + sd.ylo * g.nx + x);
+    const float3 xh = MapL<true>::at(uc, g.N, zp + y * g.nx + sd.xhi);
+    const float3 xl = MapL<true>::at(uc, g.N, zp + y * g.nx + sd.xlo);
+    const float3 yh = MapL<true>::at(uc, g.N, zp + sd.yhi * g.nx + x);
+    const float3 yl = MapL<true>::at(uc, g.N, zp + sd.ylo * g.nx + x);
     const float xhv[3] = {xh.x, xh.y, xh.z}, xlv[3] = {xl.x, xl.y, xl.z};
     const float yhv[3] = {yh.x, yh.y, yh.z}, ylv[3] = {yl.x, yl.y, yl.z};
 #pragma unroll
@@ -301,7 +299,7 @@ __device__ __forceinline__ float back_terms_at(const Grid& g, const float* __res
 // At most 40 registers (6 blocks of 256 threads per SM): the march waits on its lookups, and the
 // extra warps in flight outweigh the few spilled values (48 registers, 5 blocks: 93 against
 // 87 us at 264x160x228; 32 registers spill inside the loop and take 130 us).
-template <typename ST, int ZC, bool Q>
+template <typename ST, int ZC>
 __global__ void __launch_bounds__(256, 6) k_back_terms_march(Grid g, const float* __restrict__ uc,
                                                           const typename Pair<ST>::T* __restrict__ IM,
                                                           float* __restrict__ J1j,
@@ -314,7 +312,7 @@ __global__ void __launch_bounds__(256, 6) k_back_terms_march(Grid g, const float
     const int plane = g.nx * g.ny, rowoff = y * g.nx;
     const Sides sd = sides_of(g, x, y);
     auto ld3 = [&](int z, float* u) {
-      const float3 r = MapL<Q>::at(uc, g.N, z * plane + rowoff + x);
+      const float3 r = MapL<true>::at(uc, g.N, z * plane + rowoff + x);
       u[0] = r.x; u[1] = r.y; u[2] = r.z;
     };
     float uP[3], uC[3], uN[3], uNN[3];
@@ -325,7 +323,7 @@ __global__ void __launch_bounds__(256, 6) k_back_terms_march(Grid g, const float
       // the plane after next, for the z-derivative of plane z + 1
       const int zn = z + 2 < g.nz ? z + 2 : g.nz - 1;
       if (z + 1 < z1) ld3(zn, uNN);
-      dmin = fminf(dmin, back_terms_at<Q>(g, uc, IM, J1j, Wj, x, y, z, sd, uP, uC, uN));
+      dmin = fminf(dmin, back_terms_at(g, uc, IM, J1j, Wj, x, y, z, sd, uP, uC, uN));
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         uP[d] = uC[d];
@@ -374,7 +372,7 @@ __global__ void __launch_bounds__(256, ZC == 1 ? 4 : 5) k_back_fused_march(
       const float3 r =
           MapL<true>::lerp(uc, g.N, tri_setup(g, (float)x + dx, (float)y + dy, (float)z + dz));
       MapL<true>::put(un, g.N, idx, dx + r.x, dy + r.y, dz + r.z);
-      dmin = fminf(dmin, back_terms_at<true>(g, uc, IM, J1, W, x, y, z, sd, uP, uC, uN));
+      dmin = fminf(dmin, back_terms_at(g, uc, IM, J1, W, x, y, z, sd, uP, uC, uN));
       a0 = n0;
       a1 = n1;
       a2 = n2;
@@ -417,11 +415,11 @@ static void launch_back_terms(const Grid& g, const float* uc, const void* IM, fl
   const typename Pair<ST>::T* im = reinterpret_cast<const typename Pair<ST>::T*>(IM);
   const int nb = flow_blocks(g);
   if (nb <= 256)
-    k_back_terms_march<ST, 1, true><<<flow_grid(g, 1), kBlock3d, 0, s>>>(g, uc, im, J1j, Wj, acc);
+    k_back_terms_march<ST, 1><<<flow_grid(g, 1), kBlock3d, 0, s>>>(g, uc, im, J1j, Wj, acc);
   else if (nb <= 8192)
-    k_back_terms_march<ST, 4, true><<<flow_grid(g, 4), kBlock3d, 0, s>>>(g, uc, im, J1j, Wj, acc);
+    k_back_terms_march<ST, 4><<<flow_grid(g, 4), kBlock3d, 0, s>>>(g, uc, im, J1j, Wj, acc);
   else
-    k_back_terms_march<ST, 8, true><<<flow_grid(g, 8), kBlock3d, 0, s>>>(g, uc, im, J1j, Wj, acc);
+    k_back_terms_march<ST, 8><<<flow_grid(g, 8), kBlock3d, 0, s>>>(g, uc, im, J1j, Wj, acc);
 }
 
 // One kernel or two, by the number of four-plane blocks (us a step; two kernels cost a launch besides):
@@ -482,9 +480,8 @@ void launch_back_last(const Grid& g, const float* u, const void* IM, float* J1, 
 }
 
 void launch_flow_only_back(const Grid& g, const void* vj, const float* u_next, float* u_cur,
-                           float dtx, float dty, float dtz, cudaStream_t s, int st, int rk,
-                           int quad) {
-  disp_step(+1, g, vj, u_next, u_cur, dtx, dty, dtz, s, st, rk, quad);
+                           float dtx, float dty, float dtz, cudaStream_t s, int st, int rk) {
+  disp_step(+1, g, vj, u_next, u_cur, dtx, dty, dtz, s, st, rk);
 }
 
 // --------------------------------------------------------------------------------------------
@@ -739,7 +736,8 @@ void launch_fwd_flow(const Grid& g, const void* vj, const float* u_cur, float* u
                      const void* M, float* J0T, Acc* acc, cudaStream_t s, int st, int rk,
                      int quad) {
   if (!last) {
-    disp_step(-1, g, vj, u_cur, u_next, dtx, dty, dtz, s, st, rk, quad);
+    if (quad) disp_step(-1, g, vj, u_cur, u_next, dtx, dty, dtz, s, st, rk);
+    else launch_flow_only_fwd(g, (const float*)vj, u_cur, u_next, dtx, dty, dtz, s);
     return;
   }
   const dim3 grid((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + kFlowZ - 1) / kFlowZ);
@@ -751,8 +749,7 @@ void launch_fwd_flow(const Grid& g, const void* vj, const float* u_cur, float* u
     if (st) { if (rk) FWD_LAST(__nv_bfloat16, true, true); else FWD_LAST(__nv_bfloat16, false, true); }
     else { if (rk) FWD_LAST(float, true, true); else FWD_LAST(float, false, true); }
   } else {
-    if (st) { if (rk) FWD_LAST(__nv_bfloat16, true, false); else FWD_LAST(__nv_bfloat16, false, false); }
-    else { if (rk) FWD_LAST(float, true, false); else FWD_LAST(float, false, false); }
+    FWD_LAST(float, false, false);
   }
 #undef FWD_LAST
 }
@@ -914,10 +911,9 @@ void launch_ereg(const Grid& g, const void* v, int T, float alpha, float gamma, 
   }
 }
 
-void launch_flow_only_fwd(const Grid& g, const void* vj, const float* u_cur, float* u_next,
-                          float dtx, float dty, float dtz, cudaStream_t s, int st, int rk,
-                          int quad) {
-  disp_step(-1, g, vj, u_cur, u_next, dtx, dty, dtz, s, st, rk, quad);
+void launch_flow_only_fwd(const Grid& g, const float* vj, const float* u_cur, float* u_next,
+                          float dtx, float dty, float dtz, cudaStream_t s) {
+  launch_disp_march<float, -1, false>(g, vj, u_cur, u_next, dtx, dty, dtz, s, 0);
 }
 
 // quad map [N] x (x, y, z, 0) -> planar [3][N]

@@ -541,7 +541,7 @@ int refresh_maps(lddmm_ctx* ctx, bool energy) {
   int pb = 0;
   for (int j = T - 1; j >= 0; --j) {
     float* uc = ctx->uB[pb];
-    launch_flow_only_back(g, vptr(ctx, j, N), un, uc, dtx, dty, dtz, s, ctx->st, rk_of(ctx), 1);
+    launch_flow_only_back(g, vptr(ctx, j, N), un, uc, dtx, dty, dtz, s, ctx->st, rk_of(ctx));
     un = uc;
     pb ^= 1;
   }
@@ -1048,7 +1048,7 @@ int lddmm_shoot(lddmm_ctx* ctx, const float* v0) {
   int pf = 0;
   for (int j = 0; j + 1 < T; ++j) {
     float* un = ctx->uF[pf];
-    launch_flow_only_fwd(g, v + (int64_t)j * F, uc, un, dtx, dty, dtz, s, 0, 0);
+    launch_flow_only_fwd(g, v + (int64_t)j * F, uc, un, dtx, dty, dtz, s);
     CK(transport_momentum(g, ctx->stage, un, L.hx, L.hy, L.hz, ctx->b, s));
     CK(apply_K(L.kp, ctx->p.k_mode, ctx->b, ctx->b, ctx->work, 3, s, Hook(), nullptr, 0.f,
                ctx->kcap));
@@ -1307,7 +1307,7 @@ int lddmm_energy_grad(lddmm_ctx* ctx, const float* v, float* grad, double* E) {
         const float* from = k ? slot_of(k) : nullptr;
         for (int i = 1; i < c && k + i < T; ++i) {
           float* to = ctx->seg + (size_t)(i - 1) * F;
-          launch_flow_only_fwd(g, ctx->v + (int64_t)(k + i - 1) * F, from, to, dtx, dty, dtz, s, 0);
+          launch_flow_only_fwd(g, ctx->v + (int64_t)(k + i - 1) * F, from, to, dtx, dty, dtz, s);
           from = to;
         }
         seg_base = k;
