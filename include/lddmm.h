@@ -108,7 +108,8 @@ typedef struct {
 } lddmm_energy;
 
 /* Fill p with the defaults used by the tests: h = 1, T = 10, alpha = 0.02, gamma = 1,
- * sigma = 0.1, eps = 1e-3, 20 iterations, one level, K by FP32 DFT products (LDDMM_K_FP32), fp32 storage, timeout 600 s. */
+ * sigma = 0.1, eps = 1e-3, 20 iterations, one level, K by FP32 DFT products (LDDMM_K_FP32), fp32
+ * storage, timeout 600 s. */
 int lddmm_default_params(lddmm_params* p, int nx, int ny, int nz);
 
 /* Create a context: validates p, allocates device buffers for all levels, copies I0
@@ -180,7 +181,8 @@ int lddmm_dice(lddmm_ctx* ctx, const uint16_t* A, const uint16_t* B, int64_t n, 
  * out[0] = d_H = max of both directed maxima; out[1] = d_M = median of the union of the directed
  * distances of S_A to S_B and of S_B to S_A (mean of the two middle values for an even count);
  * out[2], out[3] = the number of surface voxels of A and of B.  Host memory.
- * Uses the context's work buffers (no allocation) and waits for the result (bounded).  LDDMM_ERR_INVALID_ARG when a mask has no surface voxel. */
+ * Uses the context's work buffers (no allocation) and waits for the result (bounded).
+ * LDDMM_ERR_INVALID_ARG when a mask has no surface voxel. */
 int lddmm_surface_distance(lddmm_ctx* ctx, const uint8_t* A, const uint8_t* B, double out[4]);
 
 /* Landmark errors e_k = |phi(x_k) - y_k| (§2.7) for the current v: phi(x) = x + u01(x) carries
@@ -257,8 +259,8 @@ int lddmm_apply_K_noalloc(const float* src, float* dst, int nx, int ny, int nz, 
                           float hy, float hz, float alpha, float gamma, void* stream);
 
 /* ---- Learned warm start: kernels of a 3D convolutional encoder-decoder that predicts an initial
- * velocity from a mask pair (no counterpart in the paper: §2.4 optimises from v = 0).  All pointers are device
- * pointers; work is enqueued on `stream` (NULL = legacy default stream); LDDMM_ERR_INVALID_ARG
+ * velocity from a mask pair (no counterpart in the paper: §2.4 optimises from v = 0).  All pointers
+ * are device pointers; work is enqueued on `stream` (NULL = legacy default stream); LDDMM_ERR_INVALID_ARG
  * on a bad shape, LDDMM_ERR_CUDA on a launch failure.  Layout: activations [B][C][n][n][n]
  * float32; weights [Co][Ci][k^3] bf16 (k = 3, zero padding 1, or k = 1); FP32 accumulation. */
 /* y (+)= conv(x, w) + bias (bias may be NULL), then ReLU if relu. */

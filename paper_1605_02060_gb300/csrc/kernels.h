@@ -9,9 +9,9 @@
 
 namespace lddmm {
 
-// Raises a kernel's dynamic shared memory limit to `bytes`, once on each device; `set` is the kernel's
-// own record.  The limit is the most the kernel is ever launched with, not one launch's need: a lower
-// value would undo what an earlier launch (a recorded graph node) counts on.
+// Raises a kernel's dynamic shared memory limit to `bytes`, once on each device; `set` is the
+// kernel's own record.  The limit is the most the kernel is ever launched with, not one launch's
+// need: a lower value would undo what an earlier launch (a recorded graph node) counts on.
 template <typename Kernel>
 cudaError_t raise_smem_limit(PerDevice<bool>& set, Kernel* kernel, int bytes) {
   int dev = -1;
@@ -87,8 +87,8 @@ void launch_fwd_flow(const Grid& g, const void* vj, const float* u_cur, float* u
                      const void* M, float* J0T, Acc* acc, cudaStream_t s, int st, int rk = 0,
                      int quad = 0);
 // Forward sweep step j (planar maps) in one pass over u_cur = phi_{j,0} - id (nullptr: id): the
-// residual b = c W_j (J0_j - J1_j) grad J0_j / h with J0_j = I0 o (id + u_cur) (bsplit 0: b as 3 fp32
-// fields; 1 / 2: b split for the pre-split K, bf16 hi plane / hi and lo planes, rows of pitch
+// residual b = c W_j (J0_j - J1_j) grad J0_j / h with J0_j = I0 o (id + u_cur) (bsplit 0: b as 3
+// fp32 fields; 1 / 2: b split for the pre-split K, bf16 hi plane / hi and lo planes, rows of pitch
 // px), and u_next as launch_fwd_flow (without J0_T and E_data: launch_j0_edata gives them).
 void launch_fwd_fused(const Grid& g, const void* vj, const float* u_cur, float* u_next,
                       float dtx, float dty, float dtz, const void* I0, const float* J1j,
@@ -123,13 +123,15 @@ void launch_upsample(const Grid& coarse, const Grid& fine, float ratio, const vo
                      void* dst, int nfields, cudaStream_t s, int st);
 void launch_to_storage(const float* src, void* dst, int64_t n, cudaStream_t s, int st);
 // launch_to_storage that also sets *flag when src holds NaN or Inf (both float: a checked copy).
-void launch_store_checked(const float* src, void* dst, int64_t n, int* flag, cudaStream_t s, int st);
+void launch_store_checked(const float* src, void* dst, int64_t n, int* flag, cudaStream_t s,
+                          int st);
 void launch_from_storage(const void* src, float* dst, int64_t n, cudaStream_t s, int st);
 // *flag |= bit when a[0..n) holds a NaN or an infinity.
 void launch_check_finite(const float* a, int64_t n, int* flag, cudaStream_t s, int bit = 1);
 void launch_fill(float* a, int64_t n, float value, cudaStream_t s);
 // hist (kDiceWords, the first kDiceZero of them zeroed): voxels per label of A, of B and of both at
-// once, 65536 each, and the mean's scratch; out = mean Dice over the labels > 0 present in either (1 when there are none).
+// once, 65536 each, and the mean's scratch; out = mean Dice over the labels > 0 present in either
+// (1 when there are none).
 constexpr int kDiceBlocks = 64, kDiceZero = 3 * 65536 + 2, kDiceWords = kDiceZero + 2 * kDiceBlocks;
 void launch_dice(const uint16_t* A, const uint16_t* B, int64_t n, unsigned long long* hist,
                  double* out, cudaStream_t s);
@@ -143,7 +145,8 @@ int64_t surface_select_bytes();
 cudaError_t surface_count(const Grid& g, const uint8_t* A, const uint8_t* B, unsigned* start,
                           cudaStream_t s);
 // After surface_count: list (na + nb entries), the directed distances dA (na) and dB (nb), sel
-// (surface_select_bytes() of scratch) and out[0] = their maximum, out[1], out[2] = the two middle values (equal for an odd number).
+// (surface_select_bytes() of scratch) and out[0] = their maximum, out[1], out[2] = the two middle
+// values (equal for an odd number).
 cudaError_t surface_distances(const Grid& g, const uint8_t* A, const uint8_t* B, unsigned* start,
                               uint16_t* list, unsigned na, unsigned nb, float hx, float hy,
                               float hz, double* dA, double* dB, void* sel, double* out,
@@ -203,8 +206,8 @@ struct KPlan {
   uint32_t poll_limit;
   bool sym_normal;   // symbol_is_normal of the grid (false: nothing is known)
 };
-// Whether every value of the symbol's square (gamma + alpha lambda)^2 on a grid of this spacing is a
-// normal number with a normal reciprocal, so that a product with the reciprocal may take the
+// Whether every value of the symbol's square (gamma + alpha lambda)^2 on a grid of this spacing is
+// a normal number with a normal reciprocal, so that a product with the reciprocal may take the
 // division's place.  lambda lies in [0, 4 (hx^-2 + hy^-2 + hz^-2)]; the bounds leave a factor of 4.
 inline bool symbol_is_normal(double hx, double hy, double hz, double alpha, double gamma) {
   const double top = gamma + alpha * 4.0 * (1.0 / (hx * hx) + 1.0 / (hy * hy) + 1.0 / (hz * hz));
@@ -238,7 +241,8 @@ struct KsOut {
 // cuTensorMapEncodeTiled from the driver, as void* (nullptr when unavailable).
 void* tma_encode_fn();
 // The pre-split path (all six products on k_dft_ks).  Row pitch of a split line (elements),
-// the sizes it takes, whether it applies, and the floats a buffer needs for any intermediate field of ncomp components.
+// the sizes it takes, whether it applies, and the floats a buffer needs for any intermediate field
+// of ncomp components.
 int ks_pitch(int L);
 bool ks_shape(int nx, int ny, int nz);
 bool ks_supported(const KPlan& kp);

@@ -163,12 +163,12 @@ __device__ __forceinline__ uint2 f4_to_bf4(float4 w) {
   return make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
 }
 
-// Row-wise outputs (o.G == 1, line l at l * o.P): the 16 columns n0.. of the warp's 32 lines
-// line0.. (lane = line on entry) leave through the warp's shared-memory tile.  VEC (rows start on a
-// 4-element boundary: X a multiple of 4): a lane reads and writes 4 consecutive columns of one
-// line, 8 lines per instruction.  Else one column, 2 lines (two runs of 64 bytes) per instruction.
-// The old v that the update combines with the 16 columns n0.. of the warp's 32 lines, in the
-// lane order store_rows uses: old[4 it + k] (VEC) or old[it].
+// Row-wise outputs (o.G == 1, line l at l * o.P).  VEC (rows start on a 4-element boundary: X a
+// multiple of 4): a lane reads and writes 4 consecutive columns of one line, 8 lines per
+// instruction.  Else one column, 2 lines (two runs of 64 bytes) per instruction.
+
+// The old v that the update combines with the 16 columns n0.. of the warp's 32 lines line0.., in
+// the lane order store_rows uses: old[4 it + k] (VEC) or old[it].
 template <bool VEC>
 __device__ __forceinline__ void load_old_rows(const KsOut& o, int lane, long long line0,
                                               long long nlines, int n0, int ncols, float* old) {
@@ -203,6 +203,8 @@ __device__ __forceinline__ void load_old_rows(const KsOut& o, int lane, long lon
   }
 }
 
+// The 16 columns n0.. of the warp's 32 lines line0.. (lane = line on entry) leave through the
+// warp's shared-memory tile.
 template <bool VEC>
 __device__ __forceinline__ void store_rows(const KsOut& o, float eps, float* sg, int lane,
                                            long long line0, long long nlines, int n0, int ncols,
@@ -250,7 +252,6 @@ __device__ __forceinline__ void store_rows(const KsOut& o, float eps, float* sg,
 
 // Epilogue kinds: each pass is compiled with only its own output path, so that the registers of
 // the other paths do not count against it (the kernel runs at the 128-register limit of 448
-// threads).
 // threads).  EPI_T transposed split outputs, EPI_ZZ the fused z pass's, EPI_ROWS and EPI_UPD rows
 // that start on a 4-element boundary, EPI_ROWS_1 and EPI_UPD_1 other rows.  EPI_ZZ_RN forms and
 // divides by the symbol with the roundings of k_dft_tc, for plain bf16 products on the grids (X no

@@ -1,6 +1,6 @@
-// What the library keeps once for each GPU of the process: limits of kernels, the SM count, flags in
-// device memory.  (A function's attributes belong to the device that is current when they are set:
-// kept for the whole process, they are missing on the second GPU.)
+// What the library keeps once for each GPU of the process: limits of kernels, the SM count, flags
+// in device memory.  (A function's attributes belong to the device that is current when they are
+// set: kept for the whole process, they are missing on the second GPU.)
 #pragma once
 #include <mutex>
 
